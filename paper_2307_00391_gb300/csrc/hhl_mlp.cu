@@ -11,6 +11,7 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "hhl_common.cuh"
@@ -22,151 +23,198 @@ constexpr int kIn = HHL_MLP_IN, kH = HHL_MLP_HIDDEN, kOut = HHL_MLP_OUT;
 constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kH * kIn, kOffW2 = kOffB1 + kH, kOffB2 = kOffW2 + kH * kH,
               kOffW3 = kOffB2 + kH, kOffB3 = kOffW3 + kOut * kH, kParams = kOffB3 + kOut;
 static_assert(kParams == HHL_MLP_PARAMS, "parameter layout");
-constexpr int kRows = 32;  // rows per CTA
-constexpr int kThr = 128;  // one thread per hidden unit
-constexpr size_t kFwdSmem = ((size_t)(kH + 2 * kRows) * (kH + 1) + kRows * kIn) * sizeof(float);
-constexpr size_t kBwdSmem = ((size_t)(kH + 4 * kRows) * (kH + 1) + kRows * kIn + kRows * kOut) * sizeof(float);
+constexpr int kRows = 4;         // rows per CTA of the row pass
+constexpr int kThr = 128;        // one thread per hidden unit
+constexpr int kGradThr = 1024;   // gradient pass: 2 units x 128 inputs x 4 row groups
+constexpr int kGradUnits = 2;
+constexpr int kGradRows = 1024;  // rows of one gradient chunk
+static_assert(kRows == 4 && kThr == kH && kGradThr == kGradUnits * kH * 4, "thread maps below");
 
-// forward for kRows rows; if act1/act2 given, the activations are stored (training)
-__global__ void __launch_bounds__(kThr) k_mlp_forward(const __nv_bfloat16* __restrict__ wb, const float* __restrict__ p,
-                                                      const float* __restrict__ x, int rows, float* __restrict__ y,
-                                                      float* __restrict__ act1, float* __restrict__ act2) {
-  extern __shared__ float smem_f[];
-  float(*sW2)[kH + 1] = reinterpret_cast<float(*)[kH + 1]>(smem_f);
-  float(*h1)[kH + 1] = reinterpret_cast<float(*)[kH + 1]>(smem_f + kH * (kH + 1));
-  float(*h2)[kH + 1] = reinterpret_cast<float(*)[kH + 1]>(smem_f + (kH + kRows) * (kH + 1));
-  float(*sx)[kIn] = reinterpret_cast<float(*)[kIn]>(smem_f + (kH + 2 * kRows) * (kH + 1));
-  const int j = threadIdx.x;
+__device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
+
+// The rows of a batch, four per CTA, thread j = hidden unit j of both layers: forward, and with
+// TRAIN the loss and the gradients with respect to the pre-activations (ga1, ga2), stored with the
+// activations for the gradient pass. A thread keeps its row of W2 (128 BF16 values) in
+// registers and reads the four rows' activations as one 16-byte broadcast per input. Bound by
+// latency: a 256-row batch is 64 CTAs. (32 rows per CTA and W2 converted into shared memory filled
+// 8 SMs: forward 41 us, loss and backward 96 us; this pass takes 6 and 9 us.)
+template <bool TRAIN>
+__global__ void __launch_bounds__(kThr) k_mlp_rows(const __nv_bfloat16* __restrict__ wb, const float* __restrict__ p,
+                                                   const float* __restrict__ x, const float* __restrict__ target,
+                                                   int rows, float* __restrict__ y, float* __restrict__ act,
+                                                   float* __restrict__ gy, float* __restrict__ loss_part) {
+  __shared__ float4 h1s[kH], h2s[kH], g2s[kH];  // unit j of the four rows
+  __shared__ float sx[kRows][kIn];
+  __shared__ float sgy[kRows][kOut], sloss[kRows];
+  const int j = threadIdx.x, lane = j & 31, warp = j >> 5;
   const int r0 = blockIdx.x * kRows;
-  for (int e = j; e < kH * kH; e += kThr) sW2[e / kH][e % kH] = __bfloat162float(wb[kOffW2 + e]);
-  for (int e = j; e < kRows * kIn; e += kThr) {
-    const int r = e / kIn, i = e % kIn;
-    sx[r][i] = (r0 + r < rows) ? x[(size_t)(r0 + r) * kIn + i] : 0.f;
+  const int nr = min(kRows, rows - r0);
+  uint32_t w2[kH / 2];
+  {
+    const uint4* src = reinterpret_cast<const uint4*>(wb + kOffW2 + j * kH);
+#pragma unroll
+    for (int q = 0; q < kH / 8; ++q) {
+      const uint4 v = src[q];
+      w2[4 * q] = v.x;
+      w2[4 * q + 1] = v.y;
+      w2[4 * q + 2] = v.z;
+      w2[4 * q + 3] = v.w;
+    }
   }
-  __syncthreads();
+  if (j < kRows * kIn) sx[j / kIn][j % kIn] = j / kIn < nr ? x[(size_t)r0 * kIn + j] : 0.f;
   float w1[kIn];
 #pragma unroll
   for (int i = 0; i < kIn; ++i) w1[i] = __bfloat162float(wb[kOffW1 + j * kIn + i]);
   const float bb1 = p[kOffB1 + j], bb2 = p[kOffB2 + j];
+  __syncthreads();
+  float h1[kRows], h2[kRows];
+#pragma unroll
   for (int r = 0; r < kRows; ++r) {
     float a = bb1;
 #pragma unroll
     for (int i = 0; i < kIn; ++i) a = fmaf(w1[i], sx[r][i], a);
-    h1[r][j] = tanhf(a);
+    h1[r] = tanhf(a);
   }
+  h1s[j] = make_float4(h1[0], h1[1], h1[2], h1[3]);
   __syncthreads();
-  for (int r = 0; r < kRows; ++r) {
-    float a = bb2;
-#pragma unroll 8
-    for (int k = 0; k < kH; ++k) a = fmaf(sW2[j][k], h1[r][k], a);
-    h2[r][j] = tanhf(a);
+  float a[kRows] = {bb2, bb2, bb2, bb2};
+#pragma unroll
+  for (int k = 0; k < kH; k += 2) {
+    const float wl = bf_lo(w2[k / 2]), wh = bf_hi(w2[k / 2]);
+    const float4 u = h1s[k], v = h1s[k + 1];
+    a[0] = fmaf(wh, v.x, fmaf(wl, u.x, a[0]));
+    a[1] = fmaf(wh, v.y, fmaf(wl, u.y, a[1]));
+    a[2] = fmaf(wh, v.z, fmaf(wl, u.z, a[2]));
+    a[3] = fmaf(wh, v.w, fmaf(wl, u.w, a[3]));
   }
+#pragma unroll
+  for (int r = 0; r < kRows; ++r) h2[r] = tanhf(a[r]);
+  h2s[j] = make_float4(h2[0], h2[1], h2[2], h2[3]);
   __syncthreads();
-  if (j < kRows * kOut) {
-    const int r = j / kOut, o = j % kOut;
-    float a = p[kOffB3 + o];
-    for (int k = 0; k < kH; ++k) a = fmaf(__bfloat162float(wb[kOffW3 + o * kH + k]), h2[r][k], a);
-    if (r0 + r < rows) y[(size_t)(r0 + r) * kOut + o] = a;
-  }
-  if (act1 != nullptr) {
-    for (int r = 0; r < kRows; ++r)
-      if (r0 + r < rows) {
-        act1[(size_t)(r0 + r) * kH + j] = h1[r][j];
-        act2[(size_t)(r0 + r) * kH + j] = h2[r][j];
+  {  // output layer: warp r sums row r
+    float o0 = 0.f, o1 = 0.f;
+#pragma unroll
+    for (int q = 0; q < kH / 32; ++q) {
+      const int k = lane + 32 * q;
+      const float h = reinterpret_cast<const float*>(&h2s[k])[warp];
+      o0 = fmaf(__bfloat162float(wb[kOffW3 + k]), h, o0);
+      o1 = fmaf(__bfloat162float(wb[kOffW3 + kH + k]), h, o1);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      o0 += __shfl_xor_sync(0xffffffffu, o0, o);
+      o1 += __shfl_xor_sync(0xffffffffu, o1, o);
+    }
+    if (lane < kOut) {
+      const float v = (lane == 0 ? o0 : o1) + p[kOffB3 + lane];
+      const bool ok = warp < nr;
+      if (!TRAIN) {
+        if (ok) y[(size_t)(r0 + warp) * kOut + lane] = v;
+      } else {
+        // loss = sum_{r,o} (y - t)^2 / (rows * kOut); gy = d loss / d y
+        const float scale = 1.f / (float)(rows * kOut);
+        const float d = ok ? v - target[(size_t)(r0 + warp) * kOut + lane] : 0.f;
+        sgy[warp][lane] = 2.f * d * scale;
+        if (ok) gy[(size_t)(r0 + warp) * kOut + lane] = 2.f * d * scale;
+        const float l = d * d * scale;
+        const float l1 = __shfl_xor_sync(0x3u, l, 1);
+        if (lane == 0) sloss[warp] = l + l1;
       }
+    }
   }
-}
-
-// loss = sum_{r,o} (y - t)^2 / (rows * kOut); gy = d loss / d y
-__global__ void k_mlp_loss(const float* __restrict__ y, const float* __restrict__ t, int rows, float* __restrict__ gy,
-                           float* __restrict__ loss) {
-  const float scale = 1.f / (float)(rows * kOut);
-  float acc = 0.f;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < rows * kOut; e += gridDim.x * blockDim.x) {
-    const float d = y[e] - t[e];
-    gy[e] = 2.f * d * scale;
-    acc += d * d * scale;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc);
-}
-
-// backward for kRows rows; gradients accumulated (atomically) into g (kParams floats)
-__global__ void __launch_bounds__(kThr) k_mlp_backward(const __nv_bfloat16* __restrict__ wb, const float* __restrict__ x,
-                                                       const float* __restrict__ act1, const float* __restrict__ act2,
-                                                       const float* __restrict__ gy, int rows, float* __restrict__ g) {
-  extern __shared__ float smem_f[];
-  float(*sW2)[kH + 1] = reinterpret_cast<float(*)[kH + 1]>(smem_f);
-  float(*h1)[kH + 1] = reinterpret_cast<float(*)[kH + 1]>(smem_f + kH * (kH + 1));
-  float(*h2)[kH + 1] = reinterpret_cast<float(*)[kH + 1]>(smem_f + (kH + kRows) * (kH + 1));
-  float(*ga2)[kH + 1] = reinterpret_cast<float(*)[kH + 1]>(smem_f + (kH + 2 * kRows) * (kH + 1));
-  float(*ga1)[kH + 1] = reinterpret_cast<float(*)[kH + 1]>(smem_f + (kH + 3 * kRows) * (kH + 1));
-  float(*sx)[kIn] = reinterpret_cast<float(*)[kIn]>(smem_f + (kH + 4 * kRows) * (kH + 1));
-  float(*sgy)[kOut] = reinterpret_cast<float(*)[kOut]>(smem_f + (kH + 4 * kRows) * (kH + 1) + kRows * kIn);
-  const int j = threadIdx.x;
-  const int r0 = blockIdx.x * kRows;
-  for (int e = j; e < kH * kH; e += kThr) sW2[e / kH][e % kH] = __bfloat162float(wb[kOffW2 + e]);
-  for (int e = j; e < kRows * kIn; e += kThr) {
-    const int r = e / kIn, i = e % kIn;
-    sx[r][i] = (r0 + r < rows) ? x[(size_t)(r0 + r) * kIn + i] : 0.f;
-  }
-  if (j < kRows * kOut) {
-    const int r = j / kOut, o = j % kOut;
-    sgy[r][o] = (r0 + r < rows) ? gy[(size_t)(r0 + r) * kOut + o] : 0.f;
-  }
-  for (int r = 0; r < kRows; ++r) {
-    const bool ok = r0 + r < rows;
-    h1[r][j] = ok ? act1[(size_t)(r0 + r) * kH + j] : 0.f;
-    h2[r][j] = ok ? act2[(size_t)(r0 + r) * kH + j] : 0.f;
-  }
+  if (!TRAIN) return;
   __syncthreads();
-  // output layer
+  if (j == 0) loss_part[blockIdx.x] = (sloss[0] + sloss[1]) + (sloss[2] + sloss[3]);
   const float w30 = __bfloat162float(wb[kOffW3 + j]), w31 = __bfloat162float(wb[kOffW3 + kH + j]);
-  float gw30 = 0.f, gw31 = 0.f;
+  const size_t plane = (size_t)rows * kH;  // act: h1, h2, ga1, ga2, rows x 128 each
+  float g2[kRows];
+#pragma unroll
   for (int r = 0; r < kRows; ++r) {
-    gw30 = fmaf(sgy[r][0], h2[r][j], gw30);
-    gw31 = fmaf(sgy[r][1], h2[r][j], gw31);
-    const float gh2 = w30 * sgy[r][0] + w31 * sgy[r][1];
-    ga2[r][j] = gh2 * (1.f - h2[r][j] * h2[r][j]);
-  }
-  atomicAdd(&g[kOffW3 + j], gw30);
-  atomicAdd(&g[kOffW3 + kH + j], gw31);
-  if (j < kOut) {
-    float gb = 0.f;
-    for (int r = 0; r < kRows; ++r) gb += sgy[r][j];
-    atomicAdd(&g[kOffB3 + j], gb);
-  }
-  __syncthreads();
-  // hidden layer 2: gW2[j][k] = sum_r ga2[r][j] h1[r][k]; gb2[j]; gh1[r][k] = sum_j W2[j][k] ga2[r][j]
-  {
-    float gb = 0.f;
-    for (int r = 0; r < kRows; ++r) gb += ga2[r][j];
-    atomicAdd(&g[kOffB2 + j], gb);
-    for (int k = 0; k < kH; ++k) {
-      float a = 0.f;
-      for (int r = 0; r < kRows; ++r) a = fmaf(ga2[r][j], h1[r][k], a);
-      atomicAdd(&g[kOffW2 + j * kH + k], a);
+    g2[r] = (w30 * sgy[r][0] + w31 * sgy[r][1]) * (1.f - h2[r] * h2[r]);
+    if (r < nr) {
+      float* row = act + (size_t)(r0 + r) * kH + j;
+      row[0] = h1[r];
+      row[plane] = h2[r];
+      row[3 * plane] = g2[r];
     }
   }
-  for (int r = 0; r < kRows; ++r) {
-    float a = 0.f;
-#pragma unroll 8
-    for (int jj = 0; jj < kH; ++jj) a = fmaf(sW2[jj][j], ga2[r][jj], a);
-    ga1[r][j] = a * (1.f - h1[r][j] * h1[r][j]);
+  g2s[j] = make_float4(g2[0], g2[1], g2[2], g2[3]);
+  __syncthreads();
+  float g1[kRows] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 16
+  for (int k = 0; k < kH; ++k) {  // column j of W2
+    const float w = __bfloat162float(wb[kOffW2 + k * kH + j]);
+    const float4 u = g2s[k];
+    g1[0] = fmaf(w, u.x, g1[0]);
+    g1[1] = fmaf(w, u.y, g1[1]);
+    g1[2] = fmaf(w, u.z, g1[2]);
+    g1[3] = fmaf(w, u.w, g1[3]);
+  }
+#pragma unroll
+  for (int r = 0; r < kRows; ++r)
+    if (r < nr) act[2 * plane + (size_t)(r0 + r) * kH + j] = g1[r] * (1.f - h1[r] * h1[r]);
+}
+
+// Parameter gradients: CTA (u, chunk) sums kGradRows rows for two hidden units: 128 x 2 entries of
+// gW2 by four row groups of threads (added in order), the other parameters of the two units by a
+// warp each. Every entry is written once, so nothing is cleared and no atomics are needed; with
+// one chunk g is the result, else chunk c goes to its own copy and k_mlp_chunks adds them.
+__global__ void __launch_bounds__(kGradThr) k_mlp_grad(const float* __restrict__ x, const float* __restrict__ act,
+                                                       const float* __restrict__ gy, int rows, float* __restrict__ g_all,
+                                                       const float* __restrict__ loss_part, int loss_parts,
+                                                       float* __restrict__ loss) {
+  __shared__ float part[4][kGradUnits][kH];
+  float* g = g_all + (size_t)blockIdx.y * kParams;
+  const size_t plane = (size_t)rows * kH;
+  const float *h1 = act, *h2 = act + plane, *ga1 = act + 2 * plane, *ga2 = act + 3 * plane;
+  const int j0 = blockIdx.x * kGradUnits;
+  const int ra = blockIdx.y * kGradRows, rb = min(rows, ra + kGradRows);
+  const int k = threadIdx.x & (kH - 1), u = (threadIdx.x >> 7) & 1, grp = threadIdx.x >> 8;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float a = 0.f;
+#pragma unroll 16
+  for (int r = ra + grp; r < rb; r += 4) a = fmaf(ga2[(size_t)r * kH + j0 + u], h1[(size_t)r * kH + k], a);
+  part[grp][u][k] = a;
+  // warps 0..19: bias, input and output weights of the units; 20, 21: output biases; 22: the loss
+  if (warp < 20) {
+    const int uu = warp / 10, item = warp % 10, j = j0 + uu;
+    float s = 0.f;
+    for (int r = ra + lane; r < rb; r += 32) {
+      if (item < 6) s = fmaf(ga1[(size_t)r * kH + j], x[(size_t)r * kIn + item], s);
+      else if (item == 6) s += ga1[(size_t)r * kH + j];
+      else if (item == 7) s += ga2[(size_t)r * kH + j];
+      else s = fmaf(gy[(size_t)r * kOut + item - 8], h2[(size_t)r * kH + j], s);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+      const int at = item < 6 ? kOffW1 + j * kIn + item : item == 6 ? kOffB1 + j : item == 7 ? kOffB2 + j : kOffW3 + (item - 8) * kH + j;
+      g[at] = s;
+    }
+  } else if (warp < 22 && blockIdx.x == 0) {
+    float s = 0.f;
+    for (int r = ra + lane; r < rb; r += 32) s += gy[(size_t)r * kOut + warp - 20];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) g[kOffB3 + warp - 20] = s;
+  } else if (warp == 22 && blockIdx.x == 0 && blockIdx.y == 0) {
+    float s = 0.f;
+    for (int q = lane; q < loss_parts; q += 32) s += loss_part[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) loss[0] = s;
   }
   __syncthreads();
-  // hidden layer 1
-  {
-    float gb = 0.f, gw[kIn] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int r = 0; r < kRows; ++r) {
-      gb += ga1[r][j];
-#pragma unroll
-      for (int i = 0; i < kIn; ++i) gw[i] = fmaf(ga1[r][j], sx[r][i], gw[i]);
-    }
-    atomicAdd(&g[kOffB1 + j], gb);
-#pragma unroll
-    for (int i = 0; i < kIn; ++i) atomicAdd(&g[kOffW1 + j * kIn + i], gw[i]);
+  if (grp == 0)
+    g[kOffW2 + (j0 + u) * kH + k] = (part[0][u][k] + part[1][u][k]) + (part[2][u][k] + part[3][u][k]);
+}
+
+__global__ void k_mlp_chunks(const float* __restrict__ g_all, int chunks, float* __restrict__ g) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < kParams; e += gridDim.x * blockDim.x) {
+    float s = g_all[e];
+    for (int c = 1; c < chunks; ++c) s += g_all[(size_t)c * kParams + e];
+    g[e] = s;
   }
 }
 
@@ -199,12 +247,11 @@ struct hhl_mlp_s {
   float* p = nullptr;           // FP32 master parameters
   float* m = nullptr;           // Adam moments
   float* v = nullptr;
-  float* g = nullptr;           // gradient accumulator
+  float* g = nullptr;           // gradients of a training step
   __nv_bfloat16* wb = nullptr;  // BF16 copy used by forward / backward
-  float* act = nullptr;         // activations (2 x cap x 128)
-  float* y = nullptr;           // outputs (cap x 2)
-  float* gy = nullptr;
-  int cap = 0;
+  float* act = nullptr;         // activations and their gradients (4 x cap x 128), gy (cap x 2), loss partials
+  float* gc = nullptr;          // per-chunk gradients of batches over kGradRows rows
+  int cap = 0, cap_chunks = 0;
   int64_t step = 0;
 };
 
@@ -212,41 +259,48 @@ namespace hhl {
 namespace {
 
 hhl_status mlp_reserve(hhl_mlp_s* n, int rows) {
-  if (rows <= n->cap) return HHL_OK;
-  if (n->act) cudaFree(n->act);
-  if (n->y) cudaFree(n->y);
-  if (n->gy) cudaFree(n->gy);
-  n->act = nullptr;
-  n->y = nullptr;
-  n->gy = nullptr;
-  if (cudaMalloc(&n->act, (size_t)2 * rows * kH * sizeof(float)) != cudaSuccess ||
-      cudaMalloc(&n->y, (size_t)rows * kOut * sizeof(float)) != cudaSuccess ||
-      cudaMalloc(&n->gy, (size_t)rows * kOut * sizeof(float)) != cudaSuccess) {
-    cudaGetLastError();
+  const int chunks = (rows + kGradRows - 1) / kGradRows;
+  if (rows > n->cap) {
+    if (n->act) cudaFree(n->act);
+    n->act = nullptr;
     n->cap = 0;
-    return fail(HHL_ERR_OOM, "MLP activation buffers");
+    if (cudaMalloc(&n->act, (size_t)rows * (4 * kH + kOut + 1) * sizeof(float)) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(HHL_ERR_OOM, "MLP activation buffers");
+    }
+    n->cap = rows;
   }
-  n->cap = rows;
+  if (chunks > 1 && chunks > n->cap_chunks) {
+    if (n->gc) cudaFree(n->gc);
+    n->gc = nullptr;
+    n->cap_chunks = 0;
+    if (cudaMalloc(&n->gc, (size_t)chunks * kParams * sizeof(float)) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(HHL_ERR_OOM, "MLP gradient buffers");
+    }
+    n->cap_chunks = chunks;
+  }
   return HHL_OK;
 }
 
-hhl_status mlp_grad(hhl_mlp_s* n, const float* x, const float* t, int rows, float* loss, cudaStream_t st) {
+hhl_status mlp_grad(hhl_mlp_s* n, const float* x, const float* t, int rows, float* g, float* loss, cudaStream_t st) {
   hhl_status s = mlp_reserve(n, rows);
   if (s != HHL_OK) return s;
-  const int blocks = (rows + kRows - 1) / kRows;
-  HHL_CUDA_TRY(cudaMemsetAsync(n->g, 0, kParams * sizeof(float), st));
-  HHL_CUDA_TRY(cudaMemsetAsync(loss, 0, sizeof(float), st));
-  float* a1 = n->act;
-  float* a2 = n->act + (size_t)n->cap * kH;
+  const int blocks = (rows + kRows - 1) / kRows, chunks = (rows + kGradRows - 1) / kGradRows;
+  float* gy = n->act + (size_t)rows * 4 * kH;
+  float* loss_part = gy + (size_t)rows * kOut;
   HHL_PROF_BEGIN(st);
-  k_mlp_forward<<<blocks, kThr, kFwdSmem, st>>>(n->wb, n->p, x, rows, n->y, a1, a2);
-  HHL_LAUNCH_CHECK("k_mlp_forward");
+  k_mlp_rows<true><<<blocks, kThr, 0, st>>>(n->wb, n->p, x, t, rows, nullptr, n->act, gy, loss_part);
+  HHL_LAUNCH_CHECK("k_mlp_rows");
   HHL_PROF_BEGIN(st);
-  k_mlp_loss<<<std::min(64, (rows * kOut + 255) / 256), 256, 0, st>>>(n->y, t, rows, n->gy, loss);
-  HHL_LAUNCH_CHECK("k_mlp_loss");
-  HHL_PROF_BEGIN(st);
-  k_mlp_backward<<<blocks, kThr, kBwdSmem, st>>>(n->wb, x, a1, a2, n->gy, rows, n->g);
-  HHL_LAUNCH_CHECK("k_mlp_backward");
+  k_mlp_grad<<<dim3(kH / kGradUnits, chunks), kGradThr, 0, st>>>(x, n->act, gy, rows, chunks > 1 ? n->gc : g, loss_part, blocks,
+                                                                loss);
+  HHL_LAUNCH_CHECK("k_mlp_grad");
+  if (chunks > 1) {
+    HHL_PROF_BEGIN(st);
+    k_mlp_chunks<<<(kParams + 255) / 256, 256, 0, st>>>(n->gc, chunks, g);
+    HHL_LAUNCH_CHECK("k_mlp_chunks");
+  }
   return HHL_OK;
 }
 
@@ -267,12 +321,6 @@ hhl_status hhl_mlp_create(hhl_mlp_t* out) {
     hhl_mlp_destroy(n);
     return fail(HHL_ERR_OOM, "MLP parameter buffers");
   }
-  if (cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdSmem) != cudaSuccess) {
-    cudaGetLastError();
-    hhl_mlp_destroy(n);
-    return fail(HHL_ERR_CUDA, "MLP kernel attributes");
-  }
   cudaMemset(n->p, 0, kParams * sizeof(float));
   cudaMemset(n->m, 0, kParams * sizeof(float));
   cudaMemset(n->v, 0, kParams * sizeof(float));
@@ -283,7 +331,7 @@ hhl_status hhl_mlp_create(hhl_mlp_t* out) {
 
 void hhl_mlp_destroy(hhl_mlp_t n) {
   if (n == nullptr) return;
-  void* ptrs[] = {n->p, n->m, n->v, n->g, n->wb, n->act, n->y, n->gy};
+  void* ptrs[] = {n->p, n->m, n->v, n->g, n->wb, n->act, n->gc};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   delete n;
@@ -318,8 +366,9 @@ hhl_status hhl_mlp_forward(hhl_mlp_t n, const float* x_dev, int32_t rows, float*
   if (n == nullptr || x_dev == nullptr || y_dev == nullptr || rows < 1) return fail(HHL_ERR_INVALID_ARG, "bad argument");
   cudaStream_t st = (cudaStream_t)stream;
   HHL_PROF_BEGIN(st);
-  k_mlp_forward<<<(rows + kRows - 1) / kRows, kThr, kFwdSmem, st>>>(n->wb, n->p, x_dev, rows, y_dev, nullptr, nullptr);
-  HHL_LAUNCH_CHECK("k_mlp_forward");
+  k_mlp_rows<false><<<(rows + kRows - 1) / kRows, kThr, 0, st>>>(n->wb, n->p, x_dev, nullptr, rows, y_dev, nullptr, nullptr,
+                                                                nullptr);
+  HHL_LAUNCH_CHECK("k_mlp_rows");
   return HHL_OK;
 }
 
@@ -333,10 +382,7 @@ hhl_status hhl_mlp_gradients(hhl_mlp_t n, const float* x_dev, const float* t_dev
   if (n == nullptr || x_dev == nullptr || t_dev == nullptr || grad_dev == nullptr || loss_dev == nullptr || rows < 1)
     return fail(HHL_ERR_INVALID_ARG, "bad argument");
   cudaStream_t st = (cudaStream_t)stream;
-  hhl_status s = mlp_grad(n, x_dev, t_dev, rows, loss_dev, st);
-  if (s != HHL_OK) return s;
-  HHL_CUDA_TRY(cudaMemcpyAsync(grad_dev, n->g, kParams * sizeof(float), cudaMemcpyDeviceToDevice, st));
-  return HHL_OK;
+  return mlp_grad(n, x_dev, t_dev, rows, grad_dev, loss_dev, st);
 }
 
 hhl_status hhl_mlp_train_step(hhl_mlp_t n, const float* x_dev, const float* t_dev, int32_t rows, float lr,
@@ -345,7 +391,7 @@ hhl_status hhl_mlp_train_step(hhl_mlp_t n, const float* x_dev, const float* t_de
   if (n == nullptr || x_dev == nullptr || t_dev == nullptr || loss_dev == nullptr || rows < 1 || !(lr > 0.f))
     return fail(HHL_ERR_INVALID_ARG, "bad argument");
   cudaStream_t st = (cudaStream_t)stream;
-  hhl_status s = mlp_grad(n, x_dev, t_dev, rows, loss_dev, st);
+  hhl_status s = mlp_grad(n, x_dev, t_dev, rows, n->g, loss_dev, st);
   if (s != HHL_OK) return s;
   n->step += 1;
   const float b1c = 1.f - powf(0.9f, (float)n->step), b2c = 1.f - powf(0.999f, (float)n->step);
