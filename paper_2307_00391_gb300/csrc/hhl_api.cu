@@ -596,6 +596,11 @@ hhl_status hhl_plan_create(const hhl_problem* prob, const hhl_params* params, hh
       hhl_plan_destroy(h);
       return fail(HHL_ERR_UNSUPPORTED, "tcgen05 GEMM not available for this size/precision");
     }
+    // The library's choice of product in complex128: the whole circuit and the postselected solve in
+    // the eigenbasis of A where that is real (hhl_spectral.cu); the stages keep the gate products.
+    if (params->gemm_impl == HHL_GEMM_AUTO && p.prec == HHL_PREC_C128 && prob->kind != HHL_MATRIX_UNITARY &&
+        eg.vi.empty() && clock_spec_fits(p))
+      HHL_PLAN_TRY(spec_create(p, eg.lam, eg.toeplitz ? nullptr : &eg.vr, st));
     const size_t mat = (size_t)N * N;
     // CUDA-core operands: every k (SIMT plans), or the k whose tree steps of the postselected
     // solve have fewer rows than one tcgen05 tile (2^k < 128) (tcgen05 plans)
@@ -776,6 +781,7 @@ void hhl_plan_destroy(hhl_plan_t plan) {
   for (void* q : ptrs)
     if (q) cudaFree(q);
   hhl::tc_free(p);
+  hhl::spec_free(p);
   delete plan;
 }
 
@@ -910,6 +916,10 @@ hhl_status hhl_apply_stage(hhl_plan_t plan, int32_t stage, void* state_dev, void
 }
 
 hhl_status hhl_apply_circuit(hhl_plan_t plan, void* state_dev, void* stream) {
+  if (plan != nullptr && state_dev != nullptr && plan->p.spec != nullptr) {
+    if (hhl::fault("launch")) return fail(HHL_ERR_CUDA, "injected launch failure (HHL_FAULT=launch)");
+    return hhl::launch_spec_circuit(plan->p, state_dev, (cudaStream_t)stream);
+  }
   for (int stage = HHL_STAGE_QPE_U; stage <= HHL_STAGE_FINAL_H; ++stage) {
     hhl_status s = hhl_apply_stage(plan, stage, state_dev, stream);
     if (s != HHL_OK) return s;
@@ -929,6 +939,7 @@ hhl_status hhl_solve_postselected(hhl_plan_t plan, const double* b_dev, void* st
   cudaStream_t st = (cudaStream_t)stream;
   char* s0 = (char*)state_dev;
   char* s1 = s0 + (size_t)(p.R * p.N) * p.amp_bytes();
+  if (p.spec != nullptr) return hhl::launch_spec_solve(p, b_dev, (double2*)s1, out_dev, eps_dev, st);
   // the trees as controlled-product GEMMs (dense plans) or Strang passes (Trotter plans)
   auto tree = [&](void* half, bool reduce) -> hhl_status {
     if (!dense) return hhl::launch_trotter_tree(p, half, reduce, st);

@@ -243,6 +243,8 @@ struct TrotPassDesc {
   int64_t list_off = 0;
 };
 
+struct SpecState;  // hhl_spectral.cu: the eigenbasis tables of a complex128 dense plan
+
 struct Plan {
   int n_s = 0, n_c = 0, n = 0;
   int prec = HHL_PREC_C64;
@@ -263,6 +265,7 @@ struct Plan {
   double* d_b = nullptr;      // N complex128: host-prepared b
   void* d_bs = nullptr;       // N amplitudes: b / (|b| 2^(n_c/2)), one anc = 0 row
   void* d_scratch = nullptr;  // GEMM output rows: 2^(n_c-1) * N amplitudes
+  SpecState* spec = nullptr;  // complex128 dense plans with the library's choice of product
   float4* d_gdf = nullptr;    // Toeplitz A, complex64: per k the 2N+2 double-float g_k values
   // Trotter (Toeplitz tridiagonal): per k the step count and the 2x2 blocks
   std::vector<int> trot_r;
@@ -351,6 +354,19 @@ hhl_status launch_toeplitz_rows(float2* half, int n_s, const float4* g, int adjo
 size_t trotter_build_passes(Plan& p, std::vector<unsigned char>* table);
 int64_t trotter_side_amps(int64_t N, int64_t R);  // side-buffer amplitudes of a Trotter plan
 hhl_status launch_interleave(const double* re, const double* im, int64_t n, double* out, cudaStream_t st);
+
+// Complex128 dense plans in the eigenbasis of A (hhl_spectral.cu): lam the eigenvalues, vec the real
+// eigenvectors (N x N row-major, columns the vectors) or NULL for the sine basis of a Toeplitz A.
+hhl_status spec_create(Plan& p, const std::vector<double>& lam, const std::vector<double>* vec, cudaStream_t st);
+void spec_free(Plan& p);
+hhl_status launch_spec_circuit(const Plan& p, void* state, cudaStream_t st);
+hhl_status launch_spec_solve(const Plan& p, const double* b, double2* v_row, double* out, double* eps, cudaStream_t st);
+// Its middle part: phases, the clock block, the conjugate phases and the Hadamards, column by column
+// (hhl_fft.cu). ph_lo / ph_hi: e^{i phi_j c} for c < 32 and c = 32 q, per eigenvector; tw: the
+// 2^n_c roots e^{-2 pi i q / 2^n_c}.
+bool clock_spec_fits(const Plan& p);
+hhl_status launch_clock_spec(const Plan& p, void* state, const double2* ph_lo, const double2* ph_hi, const double2* tw,
+                             cudaStream_t st);
 
 // tcgen05 GEMM (hhl_gemm_tc.cu)
 bool tc_supported(const Plan& p);

@@ -473,6 +473,91 @@ __global__ void __launch_bounds__(kFftThreads, 2) k_clock_block(typename Cx<R>::
   if (FULL) store_block(S0 + row0 * N + j0, N, Y, Lp, Lc, W, inv, false, rank, m);
 }
 
+// The clock part of a complex128 circuit in the eigenbasis of A (hhl_spectral.cu): per column j of
+// the anc = 0 half the phases e^{i phi_j c}, the inverse QFT, the rotation, the QFT, the conjugate
+// phases and the Hadamards, in one pass over W columns held in shared memory (no cluster: the
+// FP64 pipe bounds it, not the row segments). Radix-2 stages with their roots read from the plan's
+// table: on that pipe a table read is cheaper than forming a root, and every butterfly is a
+// thread of its own, which at 2^6 clock rows matters more than the round trips it costs (radix-8
+// groups with composed roots took 30 us at 16 columns of 2^6 rows, this form 9).
+// OP 0: DIF inverse-QFT butterflies, 1: DIT QFT butterflies, 2: Hadamards.
+template <int OP>
+__device__ __forceinline__ void radix2_stages(double2* X, int Lp, int W, int m, const double2* __restrict__ roots) {
+  const int L = 1 << m, total = W << (m - 1);
+  for (int q = 0; q < m; ++q) {
+    const int hb = OP == 1 ? q : m - 1 - q, half = 1 << hb;
+    for (int u = threadIdx.x; u < total; u += kFftThreads) {
+      const int w = u >> (m - 1), e = u & (L / 2 - 1);
+      const int k = e & (half - 1), i0 = ((e >> hb) << (hb + 1)) + k;
+      double2* a = X + w * Lp + pad16(i0);
+      double2* b = X + w * Lp + pad16(i0 + half);
+      const double2 av = *a, bv = *b;
+      if (OP == 0) {
+        *a = cadd(av, bv);
+        *b = cmul(csub(av, bv), roots[k << (m - 1 - hb)]);
+      } else if (OP == 1) {
+        const double2 t = cconjmul(bv, roots[k << (m - 1 - hb)]);
+        *a = cadd(av, t);
+        *b = csub(av, t);
+      } else {
+        *a = cadd(av, bv);
+        *b = csub(av, bv);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+template <bool FULL>
+__global__ void __launch_bounds__(kFftThreads) k_clock_spec(double2* __restrict__ S, const double2* __restrict__ rot,
+                                                         const double2* __restrict__ ph_lo,
+                                                         const double2* __restrict__ ph_hi,
+                                                         const double2* __restrict__ roots, int n_s, int m, int W) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int L = 1 << m, Lp = L + L / 16 + 1, nh = L > 32 ? L / 32 : 1;
+  const int64_t N = 1LL << n_s;
+  double2* X = reinterpret_cast<double2*>(smem_raw);
+  double2* Y = X + (size_t)W * Lp;
+  const int64_t j0 = (int64_t)blockIdx.x * W;
+  double2* S0 = S + j0;
+  double2* S1 = S0 + (N << m);
+  auto phase = [&](int w, int c) {
+    return cmul(ph_hi[(size_t)(j0 + w) * nh + (c >> 5)], ph_lo[(size_t)(j0 + w) * 32 + (c & 31)]);
+  };
+  const double inv = 1.0 / sqrt((double)L);
+  for (int u = threadIdx.x; u < L * W; u += kFftThreads) {
+    const int c = u / W, w = u - c * W;
+    X[w * Lp + pad16(c)] = cmul(S0[(int64_t)c * N + w], phase(w, c));
+  }
+  __syncthreads();
+  radix2_stages<0>(X, Lp, W, m, roots);  // inverse QFT, bit-reversed result
+  for (int u = threadIdx.x; u < L * W; u += kFftThreads) {
+    const int p = u / W, w = u - p * W;
+    const int y = bitrev_m(p, m), idx = w * Lp + pad16(p);
+    const double2 r = rot[y], x = cscale(X[idx], inv);
+    if (FULL) Y[idx] = cscale(x, r.x);
+    else S0[(int64_t)y * N + w] = cscale(x, r.x);  // every load of these columns is done
+    X[idx] = cscale(x, r.y);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < (FULL ? 2 : 1); ++h) {
+    double2* Z = h ? Y : X;
+    radix2_stages<1>(Z, Lp, W, m, roots);  // QFT
+    for (int u = threadIdx.x; u < L * W; u += kFftThreads) {
+      const int c = u / W, w = u - c * W, idx = w * Lp + pad16(c);
+      Z[idx] = cscale(cconjmul(Z[idx], phase(w, c)), inv);
+    }
+    __syncthreads();
+    radix2_stages<2>(Z, Lp, W, m, roots);  // Hadamards
+    double2* D = h ? S0 : S1;
+    for (int u = threadIdx.x; u < L * W; u += kFftThreads) {
+      const int c = u / W, w = u - c * W;
+      D[(int64_t)c * N + w] = cscale(Z[w * Lp + pad16(c)], inv);
+    }
+  }
+}
+
 // Register transform on bits [lo, lo+m): mode 0 = QFT, 1 = inverse QFT, 2 = Hadamards (DIF,
 // natural in; QFT / inverse QFT results are stored from bit-reversed positions), 3 = the QFT's
 // DIF stages left in bit-reversed order, 4 = the inverse QFT's DIT stages from bit-reversed
@@ -1896,7 +1981,29 @@ inline bool fp64_pipe() {
   return env != nullptr && atoi(env) != 0;
 }
 
+size_t clock_spec_smem(const Plan& p, int W) {
+  const size_t L = (size_t)p.R, Lp = L + L / 16 + 1;
+  return (p.full ? 2 : 1) * W * Lp * sizeof(double2);
+}
+
 }  // namespace
+
+bool clock_spec_fits(const Plan& p) { return clock_spec_smem(p, 1) <= kFftSmemCap; }
+
+hhl_status launch_clock_spec(const Plan& p, void* state, const double2* ph_lo, const double2* ph_hi, const double2* tw,
+                             cudaStream_t st) {
+  // columns per block: up to 64-byte row segments while two blocks fit an SM and every SM has one
+  int W = 4;
+  while (W > 1 && (clock_spec_smem(p, W) > 100 * 1024 || p.N / W < 2 * 152)) W /= 2;
+  const size_t smem = clock_spec_smem(p, W);
+  auto kern = p.full ? k_clock_spec<true> : k_clock_spec<false>;
+  HHL_CUDA_TRY(raise_dyn_smem((const void*)kern, smem));
+  HHL_PROF_BEGIN(st);
+  kern<<<(unsigned)(p.N / W), kFftThreads, smem, st>>>((double2*)state, (const double2*)p.d_rot, ph_lo, ph_hi, tw, p.n_s,
+                                                      p.n_c, W);
+  HHL_LAUNCH_CHECK("k_clock_spec");
+  return HHL_OK;
+}
 
 hhl_status launch_clock_block(const Plan& p, void* state, cudaStream_t st) {
   const long long half = p.R * p.N;
