@@ -558,6 +558,8 @@ hhl_status hhl_plan_create(const hhl_problem* prob, const hhl_params* params, hh
 
   HHL_ALLOC(p.d_scal, 16 * sizeof(double), &p.workspace_bytes);
   HHL_PLAN_CUDA(cudaMemsetAsync(p.d_scal, 0, 16 * sizeof(double), st));
+  HHL_ALLOC(p.d_part, (3 * kMeasureBlocks + 1) * sizeof(double), &p.workspace_bytes);
+  HHL_PLAN_CUDA(cudaMemsetAsync(p.d_part, 0, (3 * kMeasureBlocks + 1) * sizeof(double), st));
   HHL_ALLOC(p.d_b, (size_t)N * 2 * sizeof(double), &p.workspace_bytes);
   HHL_ALLOC(p.d_bs, (size_t)std::max<int64_t>(N, 2) * ab, &p.workspace_bytes);
   HHL_ALLOC(h->d_bsplit, (size_t)N * 2 * sizeof(double), &p.workspace_bytes);
@@ -776,7 +778,7 @@ hhl_status hhl_plan(const hhl_problem* prob, const hhl_params* params, hhl_plan_
 void hhl_plan_destroy(hhl_plan_t plan) {
   if (plan == nullptr) return;
   Plan& p = plan->p;
-  void* ptrs[] = {p.d_bfwd, p.d_badj, p.d_gdf, p.d_rot, p.d_scal, p.d_b, p.d_bs, p.d_scratch, p.d_trot,
+  void* ptrs[] = {p.d_bfwd, p.d_badj, p.d_gdf, p.d_rot, p.d_scal, p.d_part, p.d_b, p.d_bs, p.d_scratch, p.d_trot,
                   p.d_trot_lists, plan->d_meas, plan->d_u, plan->d_cdf, plan->d_bsplit, plan->d_qpp};
   for (void* q : ptrs)
     if (q) cudaFree(q);
@@ -818,12 +820,7 @@ uint64_t hhl_state_bytes(hhl_plan_t plan) {
 
 hhl_status hhl_prepare_rhs(hhl_plan_t plan, const double* b_dev, void* state_dev, void* stream) {
   if (plan == nullptr || b_dev == nullptr || state_dev == nullptr) return fail(HHL_ERR_INVALID_ARG, "NULL argument");
-  Plan& p = plan->p;
-  cudaStream_t st = (cudaStream_t)stream;
-  HHL_CUDA_TRY(cudaMemsetAsync(p.d_scal, 0, sizeof(double), st));
-  hhl_status s = hhl::launch_bnorm(b_dev, p.N, p.d_scal, st);
-  if (s != HHL_OK) return s;
-  return hhl::launch_prep_fill(p, b_dev, state_dev, st);
+  return hhl::launch_prep_fill(plan->p, b_dev, state_dev, (cudaStream_t)stream);
 }
 
 hhl_status hhl_prepare_rhs_host(hhl_plan_t plan, const double* b_re, const double* b_im, void* state_dev,
@@ -949,9 +946,7 @@ hhl_status hhl_solve_postselected(hhl_plan_t plan, const double* b_dev, void* st
     }
     return HHL_OK;
   };
-  HHL_CUDA_TRY(cudaMemsetAsync(p.d_scal, 0, sizeof(double), st));
   hhl_status s = hhl::tc_reset_error(p, st);
-  if (s == HHL_OK) s = hhl::launch_bnorm(b_dev, p.N, p.d_scal, st);
   if (s == HHL_OK) s = hhl::launch_prep_row(p, b_dev, s0, st);
   if (s == HHL_OK) s = tree(s0, false);                                // QPE by doubling
   // the clock block writes the whole anc = 1 half; the weights |S0|^2, |S1|^2 (= P(anc = 1))

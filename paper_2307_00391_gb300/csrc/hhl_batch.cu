@@ -197,11 +197,9 @@ hhl_status enqueue_instance(hhl_batch_s* B, int i) {
   char* s0 = (char*)state;
   char* s1 = s0 + (size_t)(p.R * p.N) * 8;
   const double* b = B->d_b + B->b_off[i];
-  HHL_CUDA_TRY(cudaMemsetAsync(p.d_scal, 0, 16 * sizeof(double), st));
-  hhl_status s = launch_bnorm(b, p.N, p.d_scal, st);
   // the postselected solve (the same circuit rearranged for its prepared input; see
   // hhl_solve_postselected): only the clock = 0 row of the anc = 0 half is prepared
-  if (s == HHL_OK) s = launch_prep_row(p, b, state, st);
+  hhl_status s = launch_prep_row(p, b, state, st);
   if (s != HHL_OK) return s;
   const int M = (int)(2 * p.N + 2);
   // tree step k: expansion (rows [2^k, 2^(k+1)) = U_k rows [0, 2^k), anc = 0 half) or

@@ -245,6 +245,8 @@ struct TrotPassDesc {
 
 struct SpecState;  // hhl_spectral.cu: the eigenbasis tables of a complex128 dense plan
 
+constexpr int kMeasureBlocks = 152 * 8;  // blocks of the sums over a state
+
 struct Plan {
   int n_s = 0, n_c = 0, n = 0;
   int prec = HHL_PREC_C64;
@@ -263,6 +265,7 @@ struct Plan {
   void* d_rot = nullptr;      // 2^n_c (cos(theta/2), sin(theta/2)) pairs, amplitude precision
   double* d_scal = nullptr;   // device scalars: [0] |b|^2, [1..3] measure sums, [4] eps sum, [5] p_anc1
   double* d_b = nullptr;      // N complex128: host-prepared b
+  double* d_part = nullptr;   // kMeasureBlocks x 3 partial sums and a ticket counter (zero between calls)
   void* d_bs = nullptr;       // N amplitudes: b / (|b| 2^(n_c/2)), one anc = 0 row
   void* d_scratch = nullptr;  // GEMM output rows: 2^(n_c-1) * N amplitudes
   SpecState* spec = nullptr;  // complex128 dense plans with the library's choice of product
@@ -291,6 +294,7 @@ hhl_status plan_scalars(const hhl_problem* prob, const hhl_params* params, Plan&
 
 // Launchers (host side of the kernels); all return HHL_OK or an error.
 hhl_status launch_bnorm(const double* b, int64_t N, double* acc, cudaStream_t st);
+// a1: |b|^2 into the plan scalars, then b / (|b| 2^(n_c/2)) into every clock row of the anc = 0 half.
 hhl_status launch_prep_fill(const Plan& p, const double* b, void* state, cudaStream_t st);
 hhl_status launch_ctrl_u_dense(const Plan& p, void* half, int k, bool adjoint, cudaStream_t st);
 // SIMT controlled product with an explicit operand B[m][n] (U^T forward, conj(U) adjoint).
@@ -314,7 +318,7 @@ hhl_status launch_measure(const Plan& p, const void* state, double* out, cudaStr
 // clock = 0 row of the anc = 1 half, then the measurement block as hhl_measure_async writes it).
 hhl_status launch_measure_sums(const Plan& p, const void* state, cudaStream_t st);
 hhl_status launch_measure_row(const Plan& p, const void* state, double* out, cudaStream_t st);
-// a1 for the postselected solve: b / (|b| 2^(n_c/2)) into the clock = 0 row of the anc = 0 half only.
+// a1 for the postselected solve: |b|^2, then b / (|b| 2^(n_c/2)) into the clock = 0 row of the anc = 0 half only.
 hhl_status launch_prep_row(const Plan& p, const double* b, void* state, cudaStream_t st);
 hhl_status launch_dissipation(const Plan& p, const void* state, double* eps, double* u_dev, cudaStream_t st);
 hhl_status launch_sample(const Plan& p, const void* state, const double* uniforms, int64_t shots, uint64_t* counts,

@@ -94,6 +94,90 @@ __global__ void k_prep_fill(const uint4* __restrict__ bs, uint4* __restrict__ st
     st[u] = u < half_units ? bs[u & (row_units - 1)] : zero;
 }
 
+// Sums of NV per-thread values over the block, returned to every thread (a fixed order).
+template <int NV>
+__device__ void block_sum_all(const double (&v)[NV], double (&total)[NV]) {
+  __shared__ double sh[NV][32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  __syncthreads();  // an earlier use may still be read
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const double s = warp_sum(v[i]);
+    if (lane == 0) sh[i][wid] = s;
+  }
+  __syncthreads();
+  if (wid == 0) {  // (not by every thread: an FP64 addition occupies the narrow pipe for 16 cycles a warp)
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const double s = warp_sum(lane < nw ? sh[i][lane] : 0.0);
+      if (lane == 0) sh[i][0] = s;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) total[i] = sh[i][0];
+}
+
+// The same for double-float values: shuffled and added on the FP32 pipe, one FP64 value per warp.
+template <int NV>
+__device__ void block_sum_all_df(df (&v)[NV], double (&total)[NV]) {
+  __shared__ double sh[NV][32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      v[i] = df_add(v[i], df(__shfl_down_sync(0xffffffffu, v[i].h, o), __shfl_down_sync(0xffffffffu, v[i].l, o)));
+    if (lane == 0) sh[i][wid] = (double)v[i].h + (double)v[i].l;
+  }
+  __syncthreads();
+  if (wid == 0) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const double s = warp_sum(lane < nw ? sh[i][lane] : 0.0);
+      if (lane == 0) sh[i][0] = s;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) total[i] = sh[i][0];
+}
+
+// Systems of at most kSmallN points: the norm, the scaled row and the fill in one launch instead of
+// four (memset, norm, scale, fill: 22 us back to back against 4 us on an 11-qubit state). Every
+// block forms |b|^2 and the row itself (at most 16 KiB of reads that hit L2); beyond kSmallN that
+// repetition would cost more than the launches. row_only: just the clock = 0 row (one block).
+constexpr int kSmallN = 1024;
+constexpr size_t kPrepOneLaunch = 4 << 20;  // larger states: the row by one block, then the fill over all SMs
+template <class R>
+__global__ void __launch_bounds__(kThreads) k_prep_small(const double2* __restrict__ b, int N, int n_c,
+                                                         double* __restrict__ scal, uint4* __restrict__ st,
+                                                         int64_t half_units, int row_only) {
+  using T = typename Cx<R>::T;
+  extern __shared__ __align__(16) unsigned char prep_smem[];
+  T* row = reinterpret_cast<T*>(prep_smem);
+  double s[1] = {0.0}, nb2[1];
+  for (int i = threadIdx.x; i < N; i += kThreads) {
+    const double2 z = b[i];
+    s[0] += z.x * z.x + z.y * z.y;
+  }
+  block_sum_all(s, nb2);
+  if (blockIdx.x == 0 && threadIdx.x == 0) scal[0] = nb2[0];
+  const double scale = nb2[0] > 0.0 ? 1.0 / sqrt(nb2[0] * (double)(1LL << n_c)) : 0.0;
+  for (int i = threadIdx.x; i < N; i += kThreads) {
+    const double2 z = b[i];
+    row[i] = mk<R>((R)(z.x * scale), (R)(z.y * scale));
+  }
+  __syncthreads();
+  const int64_t row_units = (int64_t)N * (int)sizeof(T) / 16;
+  const uint4* src = reinterpret_cast<const uint4*>(row);
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  const int64_t units = row_only ? row_units : 2 * half_units;
+  for (int64_t u = blockIdx.x * (int64_t)kThreads + threadIdx.x; u < units; u += (int64_t)gridDim.x * kThreads)
+    st[u] = u < half_units ? src[u & (row_units - 1)] : zero;
+}
+
 // ------------------------------------------------------------------------------ SIMT GEMM
 // out[i][n] = sum_m S[row(i)][m] * B[m][n] for the M_sub = 2^(n_c-1) rows with clock bit k
 // set; B = U_k^T (forward) or conj(U_k) (adjoint) so that out row = U row.
@@ -198,7 +282,7 @@ __device__ __forceinline__ void kahan_add(R& s, R& c, R p) {
 // Complex128 form on the FP32 pipe: the FP64 amplitudes split into double-float with integer
 // operations, |z|^2 and the running sums in double-float (about 48 significant bits per
 // partial; the block and grid totals in FP64).
-__global__ void k_measure_sums_df(const double2* __restrict__ S, int64_t half, int64_t N, double* acc) {
+__device__ __forceinline__ void measure_thread_df(const double2* __restrict__ S, int64_t half, int64_t N, df (&a)[3]) {
   const int64_t units = 2 * half;
   constexpr int U = 4;  // loads in flight per thread
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -222,12 +306,13 @@ __global__ void k_measure_sums_df(const double2* __restrict__ S, int64_t half, i
       }
     }
   }
-  double a[3] = {df_to_double(s[0]), df_to_double(s[1]), df_to_double(s[2])};
-  block_sum_atomic<3>(a, acc);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) a[i] = s[i];
 }
 
 template <class R>
-__global__ void k_measure_sums(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N, double* acc) {
+__device__ __forceinline__ void measure_thread(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
+                                               typename std::conditional<sizeof(R) == 4, df, double>::type (&a)[3]) {
   constexpr int per = 16 / sizeof(typename Cx<R>::T);  // amplitudes per 16-byte unit
   using V = typename std::conditional<sizeof(R) == 4, float4, double2>::type;
   const V* u = reinterpret_cast<const V*>(S);
@@ -262,8 +347,98 @@ __global__ void k_measure_sums(const typename Cx<R>::T* __restrict__ S, int64_t 
       }
     }
   }
-  double a[3] = {(double)s[0] - (double)c[0], (double)s[1] - (double)c[1], (double)s[2] - (double)c[2]};
-  block_sum_atomic<3>(a, acc);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    if constexpr (sizeof(R) == 4) a[i] = df(s[i], -c[i]);
+    else a[i] = s[i] - c[i];
+  }
+}
+// The block's totals: from double-float partials (complex64, and complex128 on the FP32 pipe) or FP64.
+template <class R, bool DF>
+__device__ __forceinline__ void measure_block(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
+                                              double (&t)[3]) {
+  if constexpr (DF) {
+    df a[3];
+    measure_thread_df(S, half, N, a);
+    block_sum_all_df(a, t);
+  } else if constexpr (sizeof(R) == 4) {
+    df a[3];
+    measure_thread<R>(S, half, N, a);
+    block_sum_all_df(a, t);
+  } else {
+    double a[3];
+    measure_thread<R>(S, half, N, a);
+    block_sum_all(a, t);
+  }
+}
+template <class R, bool DF>
+__global__ void k_measure_sums(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N, double* acc) {
+  double t[3];
+  measure_block<R, DF>(S, half, N, t);
+  if (threadIdx.x < 3) atomicAdd(acc + threadIdx.x, threadIdx.x == 0 ? t[0] : threadIdx.x == 1 ? t[1] : t[2]);
+}
+
+// out = [p_success, p_anc1, norm, |b|, xhat] by one block from the totals (w0, w1, |v|^2).
+template <class R>
+__device__ void measure_write(const typename Cx<R>::T* __restrict__ v, int64_t N, double w0, double w1, double ps,
+                              double nb2, double* __restrict__ out) {
+  if (threadIdx.x == 0) {
+    out[0] = ps;
+    out[1] = w1;
+    out[2] = w0 + w1;
+    out[3] = sqrt(nb2);
+  }
+  const double inv = ps > 0.0 ? 1.0 / sqrt(ps) : 0.0;
+  for (int64_t j = threadIdx.x; j < N; j += blockDim.x) {
+    const typename Cx<R>::T z = v[j];
+    out[4 + 2 * j] = (double)z.x * inv;
+    out[5 + 2 * j] = (double)z.y * inv;
+  }
+}
+
+// Systems of at most kSmallN points: the sums over the state and the measurement block in one
+// launch. Every block leaves its three partial sums in `part`; the block that draws the last
+// ticket adds them in block order (the same total on every run), writes the block and returns
+// the ticket counter to zero. Saves a memset and a launch (5 us of 13 on a 2 MiB state).
+template <class R, bool DF>
+__global__ void __launch_bounds__(kThreads) k_measure_small(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
+                                                            double* __restrict__ scal, double* __restrict__ part,
+                                                            unsigned* __restrict__ ticket, double* __restrict__ out) {
+  __shared__ bool last;
+  double a[3], t[3];
+  measure_block<R, DF>(S, half, N, t);
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 3; ++i) part[3 * blockIdx.x + i] = t[i];
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();  // the other blocks' partials are visible
+  a[0] = a[1] = a[2] = 0.0;
+  for (int g = threadIdx.x; g < (int)gridDim.x; g += kThreads)
+    for (int i = 0; i < 3; ++i) a[i] += __ldcg(part + 3 * g + i);
+  block_sum_all(a, t);
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 3; ++i) scal[1 + i] = t[i];
+    *ticket = 0;
+  }
+  measure_write<R>(S + half, N, t[0], t[1], t[2], scal[0], out);
+}
+
+// The postselected row's norm and the measurement block from the weights already in scal[1..2]
+// (one block; at most kSmallN points).
+template <class R>
+__global__ void __launch_bounds__(kThreads) k_row_finish_small(const typename Cx<R>::T* __restrict__ v, int64_t N,
+                                                               double* __restrict__ scal, double* __restrict__ out) {
+  double s[1] = {0.0}, t[1];
+  for (int64_t j = threadIdx.x; j < N; j += kThreads) {
+    const double re = (double)v[j].x, im = (double)v[j].y;
+    s[0] += re * re + im * im;
+  }
+  block_sum_all(s, t);
+  if (threadIdx.x == 0) scal[3] = t[0];
+  measure_write<R>(v, N, scal[1], scal[2], t[0], scal[0], out);
 }
 
 // |v|^2 of one row of N amplitudes (the postselected row), FP64.
@@ -453,6 +628,28 @@ __global__ void k_diss_sum(const typename Cx<R>::T* __restrict__ S, int64_t half
   block_sum_atomic<1>(s, acc);
 }
 
+// The whole read-out by one block (at most kSmallN points): no memset, no second launch.
+template <class R>
+__global__ void __launch_bounds__(kThreads) k_diss_small(const typename Cx<R>::T* __restrict__ v, int N,
+                                                         double* __restrict__ scal, double inv_c_lam, double wlo, double whi,
+                                                         double nu_over_h, double* __restrict__ eps,
+                                                         double* __restrict__ u_out) {
+  const double scale = sqrt(scal[0]) * inv_c_lam;
+  double s[1] = {0.0}, t[1];
+  for (int i = threadIdx.x; i <= N; i += kThreads) {
+    const double left = (i == 0) ? wlo : scale * (double)v[i - 1].x;
+    const double right = (i == N) ? whi : scale * (double)v[i].x;
+    const double d = right - left;
+    s[0] += d * d;
+    if (u_out != nullptr && i < N) u_out[i] = right;
+  }
+  block_sum_all(s, t);
+  if (threadIdx.x == 0) {
+    scal[4] = t[0];
+    eps[0] = nu_over_h * t[0];
+  }
+}
+
 __global__ void k_diss_finish(const double* __restrict__ acc, double nu_over_h, double* eps) {
   if (threadIdx.x == 0 && blockIdx.x == 0) eps[0] = nu_over_h * acc[0];
 }
@@ -569,16 +766,37 @@ hhl_status launch_bnorm(const double* b, int64_t N, double* acc, cudaStream_t st
   return HHL_OK;
 }
 
+namespace {
+template <class R>
+hhl_status prep_small(const Plan& p, const double* b, void* state, bool row_only, cudaStream_t st) {
+  const int64_t half_units = p.R * p.N * (int64_t)p.amp_bytes() / 16;
+  const int g = row_only ? 1 : grid_for(2 * half_units, kThreads, 152);  // the FP64 norm and scale: once per SM
+  HHL_PROF_BEGIN(st);
+  k_prep_small<R><<<g, kThreads, (size_t)p.N * p.amp_bytes(), st>>>((const double2*)b, (int)p.N, p.n_c, p.d_scal,
+                                                                   (uint4*)state, half_units, row_only);
+  HHL_LAUNCH_CHECK("k_prep_small");
+  return HHL_OK;
+}
+}  // namespace
+
 hhl_status launch_prep_fill(const Plan& p, const double* b, void* state, cudaStream_t st) {
-  const int gs = grid_for(p.N, kThreads, 152);
-  if (p.prec == HHL_PREC_C64) {
-    HHL_PROF_BEGIN(st);
-    k_prep_scale<float><<<gs, kThreads, 0, st>>>((const double2*)b, p.d_scal, (float2*)p.d_bs, p.N, p.n_c);
+  const bool small = p.N <= kSmallN, one = small && (size_t)(2 * p.R * p.N) * p.amp_bytes() <= kPrepOneLaunch;
+  if (small) {
+    hhl_status s = p.prec == HHL_PREC_C64 ? prep_small<float>(p, b, one ? state : p.d_bs, !one, st)
+                                          : prep_small<double>(p, b, one ? state : p.d_bs, !one, st);
+    if (s != HHL_OK || one) return s;
   } else {
+    HHL_CUDA_TRY(cudaMemsetAsync(p.d_scal, 0, sizeof(double), st));
+    hhl_status bs = launch_bnorm(b, p.N, p.d_scal, st);
+    if (bs != HHL_OK) return bs;
+    const int gs = grid_for(p.N, kThreads, 152);
     HHL_PROF_BEGIN(st);
-    k_prep_scale<double><<<gs, kThreads, 0, st>>>((const double2*)b, p.d_scal, (double2*)p.d_bs, p.N, p.n_c);
+    if (p.prec == HHL_PREC_C64)
+      k_prep_scale<float><<<gs, kThreads, 0, st>>>((const double2*)b, p.d_scal, (float2*)p.d_bs, p.N, p.n_c);
+    else
+      k_prep_scale<double><<<gs, kThreads, 0, st>>>((const double2*)b, p.d_scal, (double2*)p.d_bs, p.N, p.n_c);
+    HHL_LAUNCH_CHECK("k_prep_scale");
   }
-  HHL_LAUNCH_CHECK("k_prep_scale");
   const int64_t row_units = p.N * (int64_t)p.amp_bytes() / 16;
   const int64_t half_units = p.R * row_units;
   const int g = grid_for(2 * half_units, kThreads, 152 * 16);
@@ -656,17 +874,24 @@ hhl_status launch_measure_sums(const Plan& p, const void* state, cudaStream_t st
   const char* env = getenv("HHL_FP64_PIPE");
   HHL_PROF_BEGIN(st);
   if (p.prec == HHL_PREC_C64)
-    k_measure_sums<float><<<g, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal + 1);
+    k_measure_sums<float, false><<<g, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal + 1);
   else if (env != nullptr && atoi(env) != 0)
-    k_measure_sums<double><<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
+    k_measure_sums<double, false><<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
   else
-    k_measure_sums_df<<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
+    k_measure_sums<double, true><<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
   HHL_LAUNCH_CHECK("k_measure_sums");
   return HHL_OK;
 }
 
 hhl_status launch_measure_row(const Plan& p, const void* state, double* out, cudaStream_t st) {
   const int64_t half = p.R * p.N;
+  if (p.N <= kSmallN) {
+    HHL_PROF_BEGIN(st);
+    if (p.prec == HHL_PREC_C64) k_row_finish_small<float><<<1, kThreads, 0, st>>>((const float2*)state + half, p.N, p.d_scal, out);
+    else k_row_finish_small<double><<<1, kThreads, 0, st>>>((const double2*)state + half, p.N, p.d_scal, out);
+    HHL_LAUNCH_CHECK("k_row_finish_small");
+    return HHL_OK;
+  }
   HHL_CUDA_TRY(cudaMemsetAsync(p.d_scal + 3, 0, sizeof(double), st));
   const int gf = grid_for(p.N, kThreads, 152 * 4);
   HHL_PROF_BEGIN(st);
@@ -685,6 +910,11 @@ hhl_status launch_measure_row(const Plan& p, const void* state, double* out, cud
 }
 
 hhl_status launch_prep_row(const Plan& p, const double* b, void* state, cudaStream_t st) {
+  if (p.N <= kSmallN)
+    return p.prec == HHL_PREC_C64 ? prep_small<float>(p, b, state, true, st) : prep_small<double>(p, b, state, true, st);
+  HHL_CUDA_TRY(cudaMemsetAsync(p.d_scal, 0, sizeof(double), st));
+  hhl_status bs = launch_bnorm(b, p.N, p.d_scal, st);
+  if (bs != HHL_OK) return bs;
   const int gs = grid_for(p.N, kThreads, 152);
   HHL_PROF_BEGIN(st);
   if (p.prec == HHL_PREC_C64)
@@ -698,12 +928,26 @@ hhl_status launch_prep_row(const Plan& p, const double* b, void* state, cudaStre
 
 hhl_status launch_measure(const Plan& p, const void* state, double* out, cudaStream_t st) {
   const int64_t half = p.R * p.N;
+  if (p.N <= kSmallN && p.d_part != nullptr) {
+    const char* env = getenv("HHL_FP64_PIPE");
+    const int gm = grid_for(2 * half, kThreads, kMeasureBlocks);
+    unsigned* ticket = reinterpret_cast<unsigned*>(p.d_part + 3 * kMeasureBlocks);
+    HHL_PROF_BEGIN(st);
+    if (p.prec == HHL_PREC_C64)
+      k_measure_small<float, false><<<gm, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal, p.d_part, ticket, out);
+    else if (env != nullptr && atoi(env) != 0)
+      k_measure_small<double, false><<<gm, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal, p.d_part, ticket, out);
+    else
+      k_measure_small<double, true><<<gm, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal, p.d_part, ticket, out);
+    HHL_LAUNCH_CHECK("k_measure_small");
+    return HHL_OK;
+  }
   HHL_CUDA_TRY(cudaMemsetAsync(p.d_scal + 1, 0, 3 * sizeof(double), st));
   const int g = grid_for(2 * half, kThreads, 152 * 8);
   const int gf = grid_for(p.N, kThreads, 152 * 4);
   if (p.prec == HHL_PREC_C64) {
     HHL_PROF_BEGIN(st);
-    k_measure_sums<float><<<g, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal + 1);
+    k_measure_sums<float, false><<<g, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal + 1);
     HHL_LAUNCH_CHECK("k_measure_sums");
     HHL_PROF_BEGIN(st);
     k_measure_finish<float><<<gf, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal, out);
@@ -711,9 +955,9 @@ hhl_status launch_measure(const Plan& p, const void* state, double* out, cudaStr
     const char* env = getenv("HHL_FP64_PIPE");
     HHL_PROF_BEGIN(st);
     if (env != nullptr && atoi(env) != 0)
-      k_measure_sums<double><<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
+      k_measure_sums<double, false><<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
     else
-      k_measure_sums_df<<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
+      k_measure_sums<double, true><<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
     HHL_LAUNCH_CHECK("k_measure_sums");
     HHL_PROF_BEGIN(st);
     k_measure_finish<double><<<gf, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal, out);
@@ -830,9 +1074,20 @@ hhl_status launch_sample(const Plan& p, const void* state, const double* uniform
 
 hhl_status launch_dissipation(const Plan& p, const void* state, double* eps, double* u_dev, cudaStream_t st) {
   const int64_t half = p.R * p.N;
+  const double inv_c_lam = 1.0 / (p.C * p.lam_ub);
+  if (p.N <= kSmallN) {
+    HHL_PROF_BEGIN(st);
+    if (p.prec == HHL_PREC_C64)
+      k_diss_small<float><<<1, kThreads, 0, st>>>((const float2*)state + half, (int)p.N, p.d_scal, inv_c_lam, p.wall_lo,
+                                                  p.wall_hi, p.nu * (double)(p.N + 1), eps, u_dev);
+    else
+      k_diss_small<double><<<1, kThreads, 0, st>>>((const double2*)state + half, (int)p.N, p.d_scal, inv_c_lam, p.wall_lo,
+                                                   p.wall_hi, p.nu * (double)(p.N + 1), eps, u_dev);
+    HHL_LAUNCH_CHECK("k_diss_small");
+    return HHL_OK;
+  }
   HHL_CUDA_TRY(cudaMemsetAsync(p.d_scal + 4, 0, sizeof(double), st));
   const int g = grid_for(p.N + 1, kThreads, 152 * 4);
-  const double inv_c_lam = 1.0 / (p.C * p.lam_ub);
   if (p.prec == HHL_PREC_C64) {
     HHL_PROF_BEGIN(st);
     k_diss_sum<float><<<g, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal, inv_c_lam, p.wall_lo,
