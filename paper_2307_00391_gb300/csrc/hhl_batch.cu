@@ -34,7 +34,7 @@
 
 #include <cuda_fp16.h>
 
-#include "hhl_common.cuh"
+#include "hhl_fft_core.cuh"
 
 namespace hhl {
 namespace {
@@ -118,6 +118,226 @@ __global__ void k_ugen_embed_simt(int n_s, const float4* __restrict__ g, int adj
   }
 }
 
+// ------------------------------------------------------------------ one-block solves
+// Instances whose clock and system registers fit one block's shared memory (n_c <= 7, N <= 128): the
+// whole postselected solve in one launch for all of them, a block each, instead of about 17
+// launches per instance (384 instances of 2^3..2^6 points: 6,900 launches of 0.6 us each on 8
+// streams, 3.9 ms; now one launch). Bound by the latency of the 2 n_c dependent products. The
+// arithmetic is that of the launches it replaces, operation for operation: U_k from its g table,
+// every output of a product as 32 partial sums over m (mod 32) added in the order of
+// k_toeplitz_rows' shuffles and warps, the transform stages of k_clock_block, the squares of
+// k_measure_sums.
+struct SmallInst {
+  int n_s, n_c;
+  long long b_off, out_off;  // doubles into the packed arrays
+  const float4* g;           // n_c x (2N + 2)
+  const float2* rot;         // R: (cos, sin)(theta_y / 2)
+  double inv_c_lam, wall_lo, wall_hi, nu_over_h;
+  int index, pad;            // position of the dissipation rate
+};
+
+constexpr int kSmallBits = 7;       // n_s and n_c at most
+constexpr int kSmallThreads = 256;
+
+__host__ __device__ constexpr int small_column(int n_c) { return (1 << n_c) + (1 << n_c) / 16 + 1; }
+size_t small_smem(int n_s, int n_c) {
+  return ((size_t)twiddle_entries(n_c) + ((size_t)small_column(n_c) << n_s)) * sizeof(float2) +
+         2 * (2 * ((size_t)1 << n_s) + 2) * sizeof(float4) + 16;
+}
+
+// The partial sums of output (n; rows in0 ..) whose parts lie in warp w of k_toeplitz_rows: parts
+// 4w .. 4w + 3 (columns m = part mod 32), added as its shuffles add them.
+template <int RB>
+__device__ __forceinline__ void small_parts(const float2* __restrict__ X, int Lp, const float4* __restrict__ g, int N, int n,
+                                            int in0, int w, bool adjoint, float2 (&y)[RB]) {
+  float2 a[4][RB];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+#pragma unroll
+    for (int r = 0; r < RB; ++r) a[q][r] = make_float2(0.f, 0.f);
+    for (int c = 4 * w + q; c < N; c += 32) {
+      float2 u = toeplitz_u(g, n, c);
+      if (adjoint) u.y = -u.y;
+#pragma unroll
+      for (int r = 0; r < RB; ++r) {
+        const float2 x = X[c * Lp + pad16(in0 + r)];
+        a[q][r].x = fmaf(u.x, x.x, fmaf(-u.y, x.y, a[q][r].x));
+        a[q][r].y = fmaf(u.x, x.y, fmaf(u.y, x.x, a[q][r].y));
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < RB; ++r) y[r] = cadd(cadd(a[0][r], a[1][r]), cadd(a[2][r], a[3][r]));
+}
+
+__device__ __forceinline__ void small_store(float2* X, int Lp, int n, int row, float2 y, bool accumulate, float scale,
+                                            bool scaled) {
+  float2* d = X + n * Lp + pad16(row);
+  if (accumulate) {
+    y.x += d->x;
+    y.y += d->y;
+    if (scaled) {
+      y.x *= scale;
+      y.y *= scale;
+    }
+  }
+  *d = y;
+}
+
+// m output rows from out0 on, each U (or U^dagger) applied to its row from in0 on. With few outputs
+// eight threads share one (a warp's parts each), else a thread takes four rows of one column.
+__device__ void small_product(float2* X, int Lp, const float4* __restrict__ g, int n_s, int m, int in0, int out0,
+                              bool adjoint, bool accumulate, float scale, bool scaled) {
+  const int N = 1 << n_s;
+  if (m < 4 || (m << n_s) < 4 * kSmallThreads) {
+    const int items = m << n_s, lane8 = threadIdx.x & 7;
+    for (int i0 = 0; i0 < items; i0 += kSmallThreads / 8) {  // (whole warps take part in the shuffles)
+      const int it = i0 + (threadIdx.x >> 3);
+      const int n = it & (N - 1), r = it >> n_s;
+      float2 part[1] = {make_float2(0.f, 0.f)};
+      if (it < items && 4 * lane8 < N) small_parts<1>(X, Lp, g, N, n, in0 + r, lane8, adjoint, part);
+      float2 y = part[0];
+      const int base = threadIdx.x & 24;
+#pragma unroll
+      for (int w = 1; w < 8; ++w) {
+        const float px = __shfl_sync(0xffffffffu, part[0].x, base + w);
+        const float py = __shfl_sync(0xffffffffu, part[0].y, base + w);
+        y.x += px;
+        y.y += py;
+      }
+      if (it < items && lane8 == 0) small_store(X, Lp, n, out0 + r, y, accumulate, scale, scaled);
+    }
+  } else {
+    const int items = (m / 4) << n_s;
+    for (int it = threadIdx.x; it < items; it += kSmallThreads) {
+      const int n = it & (N - 1), r = (it >> n_s) * 4;
+      float2 y[4], p[4];
+      small_parts<4>(X, Lp, g, N, n, in0 + r, 0, adjoint, y);
+      for (int w = 1; 4 * w < N && w < 8; ++w) {
+        small_parts<4>(X, Lp, g, N, n, in0 + r, w, adjoint, p);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) y[q] = cadd(y[q], p[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) small_store(X, Lp, n, out0 + r + q, y[q], accumulate, scale, scaled);
+    }
+  }
+}
+
+__device__ __forceinline__ float small_square(float2 a, float2 b) {
+  return fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(b.x, b.x, b.y * b.y)));
+}
+
+__global__ void __launch_bounds__(kSmallThreads) k_batch_small(const SmallInst* __restrict__ inst,
+                                                               const double* __restrict__ b_all, double* __restrict__ b_copy,
+                                                               double* __restrict__ out_all, double* __restrict__ eps) {
+  extern __shared__ __align__(16) unsigned char small_raw[];
+  const SmallInst d = inst[blockIdx.x];
+  const int N = 1 << d.n_s, L = 1 << d.n_c, m = d.n_c, Lp = small_column(d.n_c), M = 2 * N + 2;
+  float4* gk = reinterpret_cast<float4*>(small_raw);  // two tables: the next step's loads under this one
+  float2* t0 = reinterpret_cast<float2*>(gk + 2 * M);
+  float2* t1 = t0 + 64;
+  float2* X = t0 + twiddle_entries(m);
+  const double2* b = reinterpret_cast<const double2*>(b_all + d.b_off);
+  auto load_g = [&](int k, int buf) {
+    for (int q = threadIdx.x; q < M; q += kSmallThreads) gk[buf * M + q] = d.g[(size_t)k * M + q];
+  };
+  fill_twiddles<float>(t0, t1, m);
+  load_g(0, 0);
+  // the scaled right-hand side in clock row 0
+  double nb2[1], s[1] = {0.0};
+  double2 z = make_double2(0.0, 0.0);
+  if (threadIdx.x < N) {
+    z = b[threadIdx.x];
+    s[0] = z.x * z.x + z.y * z.y;
+    if (b_copy != nullptr) reinterpret_cast<double2*>(b_copy + d.b_off)[threadIdx.x] = z;
+  }
+  block_sum_all(s, nb2);
+  const double scale = nb2[0] > 0.0 ? 1.0 / sqrt(nb2[0] * (double)L) : 0.0;
+  if (threadIdx.x < N) X[threadIdx.x * Lp] = make_float2((float)(z.x * scale), (float)(z.y * scale));
+  __syncthreads();
+  // QPE by doubling
+  for (int k = 0; k < m; ++k) {
+    load_g(k + 1 < m ? k + 1 : m - 1, (k + 1) & 1);  // (the last load is the first reduction step's)
+    small_product(X, Lp, gk + (k & 1) * M, d.n_s, 1 << k, 0, 1 << k, false, false, 1.f, false);
+    __syncthreads();
+  }
+  // inverse QFT, rotation (the anc = 0 half is only weighed), QFT
+  const Twiddle<float2> tw{t0, t1};
+  local_stages<float2, false, 0, true>(X, Lp, N, tw, m, m, false);
+  const float inv = (float)(1.0 / sqrt((double)L));
+  df w[2] = {df(0), df(0)};
+  for (int u = threadIdx.x; u < L * (N / 2); u += kSmallThreads) {
+    const int p = u & (L - 1), j = (u >> m) * 2;
+    const float2 r = d.rot[bitrev_m(p, m)];
+    float2 kt[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int idx = (j + q) * Lp + pad16(p);
+      const float2 x = cscale(X[idx], inv);
+      kt[q] = cscale(x, r.x);
+      X[idx] = cscale(x, r.y);
+    }
+    w[0] = df_add(w[0], df(small_square(kt[0], kt[1]), 0.f));
+  }
+  __syncthreads();
+  local_stages<float2, true, 0, true>(X, Lp, N, tw, m, m, true);
+  for (int u = threadIdx.x; u < L * (N / 2); u += kSmallThreads) {
+    const int p = u & (L - 1), j = (u >> m) * 2;
+    float2 v[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int idx = (j + q) * Lp + pad16(p);
+      v[q] = cscale(X[idx], inv);
+      X[idx] = v[q];
+    }
+    w[1] = df_add(w[1], df(small_square(v[0], v[1]), 0.f));
+  }
+  double wt[2];
+  block_sum_all_df(w, wt);
+  __syncthreads();
+  // uncompute, Hadamards and postselection by halving: the table of step k is in buffer k & 1 or,
+  // for the first, in the one the last expansion step loaded
+  int buf = m & 1;
+  for (int k = m - 1; k >= 0; --k) {
+    if (k > 0) load_g(k - 1, buf ^ 1);
+    small_product(X, Lp, gk + buf * M, d.n_s, 1 << k, 1 << k, 0, true, true, inv, k == 0);
+    __syncthreads();
+    buf ^= 1;
+  }
+  // the measurement block and the dissipation rate
+  double a[2] = {0.0, 0.0}, t[2];
+  const double us = sqrt(nb2[0]) * d.inv_c_lam;
+  float2 v = make_float2(0.f, 0.f);
+  if (threadIdx.x < N) {
+    const int i = threadIdx.x;
+    v = X[i * Lp];
+    a[0] = (double)v.x * (double)v.x + (double)v.y * (double)v.y;
+    const double left = i == 0 ? d.wall_lo : us * (double)X[(i - 1) * Lp].x, right = us * (double)v.x;
+    a[1] = (right - left) * (right - left);
+    if (i == N - 1) a[1] += (d.wall_hi - right) * (d.wall_hi - right);
+  }
+  block_sum_all(a, t);
+  double* out = out_all + d.out_off;
+  if (threadIdx.x == 0) {
+    out[0] = t[0];
+    out[1] = wt[1];
+    out[2] = wt[0] + wt[1];
+    out[3] = sqrt(nb2[0]);
+    eps[d.index] = d.nu_over_h * t[1];
+  }
+  if (threadIdx.x < N) {
+    const double iv = t[0] > 0.0 ? 1.0 / sqrt(t[0]) : 0.0;
+    out[4 + 2 * threadIdx.x] = (double)v.x * iv;
+    out[5 + 2 * threadIdx.x] = (double)v.y * iv;
+  }
+}
+
+struct SmallClass {  // instances of similar shared-memory need: one launch
+  int first = 0, count = 0;
+  size_t smem = 0;
+};
+
 struct Work {
   cudaStream_t s = nullptr;
   cudaEvent_t done = nullptr;
@@ -144,6 +364,10 @@ struct hhl_batch_s {
   int count = 0;
   std::vector<Plan> plans;
   std::vector<int> gemm;       // 0 SIMT, 128 / 256 tcgen05 tile width
+  std::vector<int> large;      // the instances that the graph runs
+  std::vector<hhl::SmallClass> small;  // the others: one-block solves, by shared memory
+  hhl::SmallInst* d_small = nullptr;
+  int streams = 0;
   std::vector<int> stream_of;
   std::vector<size_t> state_off, b_off, out_off, ph_off, cos_off, g_off, rot_off;
   std::vector<CUtensorMap> maps;  // 4 per instance (tc): A_hi, A_lo, B_hi, B_lo
@@ -163,7 +387,8 @@ struct hhl_batch_s {
   double gemm_flops = 0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
-  uint64_t graph_launches = 0;
+  uint64_t graph_launches = 0;  // kernels of one run (0 before the first)
+  uint64_t captured = 0;        // those of them in the graph
   std::vector<double> host_b;  // staging for hhl_batch_run_host
 };
 
@@ -182,7 +407,7 @@ void free_batch(hhl_batch_s* b) {
     if (w.done) cudaEventDestroy(w.done);
     if (w.s) cudaStreamDestroy(w.s);
   }
-  void* ptrs[] = {b->arena, b->d_b, b->d_out, b->d_eps, b->d_scal, b->d_bs, b->d_rot, b->d_ph, b->d_cos, b->d_g, b->d_err};
+  void* ptrs[] = {b->arena, b->d_b, b->d_out, b->d_eps, b->d_scal, b->d_bs, b->d_rot, b->d_ph, b->d_cos, b->d_g, b->d_err, b->d_small};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   delete b;
@@ -242,8 +467,22 @@ hhl_status enqueue_instance(hhl_batch_s* B, int i) {
   return s;
 }
 
-hhl_status capture(hhl_batch_s* B, cudaStream_t origin) {
-  if (B->exec) return HHL_OK;
+// The one-block solves, on the caller's stream.
+hhl_status run_small(const hhl_batch_s* B, const double* b, double* b_copy, double* out, double* eps, cudaStream_t st) {
+  for (const SmallClass& c : B->small) {
+    HHL_CUDA_TRY(raise_dyn_smem((const void*)k_batch_small, c.smem));
+    HHL_PROF_BEGIN(st);
+    k_batch_small<<<(unsigned)c.count, kSmallThreads, c.smem, st>>>(B->d_small + c.first, b, b_copy, out, eps);
+    HHL_LAUNCH_CHECK("k_batch_small");
+  }
+  return HHL_OK;
+}
+
+hhl_status capture(hhl_batch_s* B) {
+  if (B->exec || B->large.empty()) {
+    B->graph_launches = B->captured + B->small.size();
+    return HHL_OK;
+  }
   cudaStream_t cap = nullptr;
   HHL_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
   cudaEvent_t fork = nullptr;
@@ -256,9 +495,7 @@ hhl_status capture(hhl_batch_s* B, cudaStream_t origin) {
   if (e == cudaSuccess) e = cudaEventRecord(fork, cap);
   for (auto& w : B->work)
     if (e == cudaSuccess) e = cudaStreamWaitEvent(w.s, fork, 0);
-  std::vector<int> order(B->count);
-  std::iota(order.begin(), order.end(), 0);
-  for (int i : order)
+  for (int i : B->large)
     if (e == cudaSuccess && s == HHL_OK) s = enqueue_instance(B, i);
   for (auto& w : B->work) {
     if (e == cudaSuccess) e = cudaEventRecord(w.done, w.s);
@@ -276,8 +513,8 @@ hhl_status capture(hhl_batch_s* B, cudaStream_t origin) {
   if (e2 != cudaSuccess) return cuda_fail(e2, "cudaStreamEndCapture");
   B->graph = graph;
   HHL_CUDA_TRY(cudaGraphInstantiate(&B->exec, graph, 0));
-  B->graph_launches = g_launches.load() - l0;
-  (void)origin;
+  B->captured = g_launches.load() - l0;
+  B->graph_launches = B->captured + B->small.size();
   return HHL_OK;
 }
 
@@ -327,13 +564,18 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
     if (gsel != 0 && (p.R / 2 < 128 || 2 * p.N < gsel)) gsel = 0;  // tile does not fit
     B->gemm[i] = gsel;
     p.gemm_impl = gsel ? HHL_GEMM_TCGEN05 : HHL_GEMM_SIMT;
+    // one-block solves: every tree step of n_c <= 7 is a Toeplitz product (fewer than 128 rows) whose
+    // blocks take 8 outputs at N <= 128, which is the summation order the block repeats
+    if (gsel != 0 || p.n_c > kSmallBits || p.n_s > kSmallBits || toeplitz_rows_limit() < 128) B->large.push_back(i);
     // the two trees: sum over k of 2^k rows each (expansion and reduction)
     B->gemm_flops += 2.0 * 8.0 * (double)(p.R - 1) * (double)p.N * (double)p.N;
   }
   // LPT assignment of instances to worker streams by GEMM work
-  streams = std::min(streams, count);
-  std::vector<int> order(count);
-  std::iota(order.begin(), order.end(), 0);
+  B->streams = std::min(streams, count);
+  streams = std::min<int>(streams, (int)B->large.size());
+  std::vector<int> order = B->large;
+  std::vector<char> is_large(count, 0);
+  for (int i : B->large) is_large[i] = 1;
   // work of an instance: the GEMM rows of its two trees (2^n_c) and its 2 n_c operand
   // generations, each over N^2 entries
   auto cost = [&](int i) {
@@ -356,7 +598,7 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
   B->cos_off.resize(count); B->g_off.resize(count); B->rot_off.resize(count);
   for (int i = 0; i < count; ++i) {
     const Plan& p = B->plans[i];
-    B->state_off[i] = so; so += (size_t)(2 * p.R * p.N) * 8;
+    B->state_off[i] = so; so += is_large[i] ? (size_t)(2 * p.R * p.N) * 8 : 0;
     B->b_off[i] = bo;     bo += (size_t)2 * p.N;
     B->out_off[i] = oo;   oo += (size_t)(4 + 2 * p.N);
     B->ph_off[i] = po;    po += (size_t)p.n_c * p.N;
@@ -378,7 +620,8 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
             alloc((void**)&B->d_scal, (size_t)count * 16 * sizeof(double)) &&
             alloc(&B->d_bs, (bo / 2) * sizeof(float2)) && alloc(&B->d_rot, ro * sizeof(float2)) &&
             alloc((void**)&B->d_ph, po * sizeof(double2)) && alloc((void**)&B->d_cos, co * sizeof(double)) &&
-            alloc((void**)&B->d_g, go * sizeof(float4)) && alloc((void**)&B->d_err, sizeof(int));
+            alloc((void**)&B->d_g, go * sizeof(float4)) && alloc((void**)&B->d_err, sizeof(int)) &&
+            alloc((void**)&B->d_small, (count - B->large.size()) * sizeof(SmallInst));
   for (auto& w : B->work) {
     if (!ok) break;
     const int64_t N2 = 2 * w.capN;
@@ -415,6 +658,10 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
     cudaMemcpy(B->d_ph + B->ph_off[i], ph.data(), ph.size() * sizeof(double2), cudaMemcpyHostToDevice);
     cudaMemcpy(B->d_cos + B->cos_off[i], cs.data(), cs.size() * sizeof(double), cudaMemcpyHostToDevice);
     cudaMemcpy((float2*)B->d_rot + B->rot_off[i], rot.data(), rot.size() * sizeof(float2), cudaMemcpyHostToDevice);
+    if (!is_large[i]) {
+      B->maps.insert(B->maps.end(), 4, CUtensorMap{});
+      continue;
+    }
     // device pointers of the per-instance plan view
     Work& w = B->work[B->stream_of[i]];
     p.d_scal = B->d_scal + (size_t)16 * i;
@@ -452,9 +699,39 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
     const Plan& p = B->plans[i];
     const int M = (int)(2 * p.N + 2);
     dim3 grid((unsigned)((M + 255) / 256), (unsigned)p.n_c);
-    k_ugen_g<<<grid, 256, p.N * sizeof(double2), B->work[B->stream_of[i]].s>>>(
+    k_ugen_g<<<grid, 256, p.N * sizeof(double2), is_large[i] ? B->work[B->stream_of[i]].s : (cudaStream_t)0>>>(
         (int)p.N, B->d_ph + B->ph_off[i], B->d_cos + B->cos_off[i], B->d_g + B->g_off[i]);
     if (cudaError_t le = cudaGetLastError(); le != cudaSuccess) s = cuda_fail(le, "k_ugen_g");
+  }
+  if (s == HHL_OK && (int)B->large.size() < count) {
+    // the one-block solves, largest first, in at most three launches (the shared memory of a launch is
+    // its largest instance's: beyond 16 KiB a quarter of it starts the next)
+    std::vector<SmallInst> small;
+    std::vector<int> idx;
+    for (int i = 0; i < count; ++i)
+      if (!is_large[i]) idx.push_back(i);
+    auto need = [&](int i) { return small_smem(B->plans[i].n_s, B->plans[i].n_c); };
+    std::stable_sort(idx.begin(), idx.end(), [&](int a, int c) { return need(a) > need(c); });
+    for (int i : idx) {
+      const Plan& p = B->plans[i];
+      SmallInst d = {};
+      d.n_s = p.n_s;
+      d.n_c = p.n_c;
+      d.b_off = (long long)B->b_off[i];
+      d.out_off = (long long)B->out_off[i];
+      d.g = B->d_g + B->g_off[i];
+      d.rot = (const float2*)B->d_rot + B->rot_off[i];
+      d.inv_c_lam = 1.0 / (p.C * p.lam_ub);
+      d.wall_lo = p.wall_lo;
+      d.wall_hi = p.wall_hi;
+      d.nu_over_h = p.nu * (double)(p.N + 1);
+      d.index = i;
+      if (B->small.empty() || (4 * need(i) < B->small.back().smem && B->small.back().smem > (16 << 10))) B->small.push_back({(int)small.size(), 0, need(i)});
+      ++B->small.back().count;
+      small.push_back(d);
+    }
+    cudaError_t e = cudaMemcpy(B->d_small, small.data(), small.size() * sizeof(SmallInst), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) s = cuda_fail(e, "batch setup");
   }
   if (s == HHL_OK) {
     cudaError_t e = cudaDeviceSynchronize();
@@ -478,7 +755,7 @@ hhl_status hhl_batch_get_info(hhl_batch_t b, hhl_batch_info* info) {
   if (b == nullptr || info == nullptr) return fail(HHL_ERR_INVALID_ARG, "NULL batch or info");
   memset(info, 0, sizeof(*info));
   info->count = b->count;
-  info->streams = (int32_t)b->work.size();
+  info->streams = b->streams;
   info->state_bytes = b->state_bytes;
   info->workspace_bytes = b->work_bytes;
   info->gemm_flops = b->gemm_flops;
@@ -514,11 +791,15 @@ hhl_status hhl_batch_run(hhl_batch_t b, const double* b_dev, double* out_dev, do
     bo += 2 * b->plans[i].N;
     oo += 4 + 2 * b->plans[i].N;
   }
-  hhl_status s = capture(b, st);
+  hhl_status s = capture(b);
   if (s != HHL_OK) return s;
+  if (b->exec == nullptr)  // one-block solves only (they keep the right-hand sides for hhl_batch_run_eager)
+    return run_small(b, b_dev, b->d_b, out_dev, eps_dev, st);
   HHL_CUDA_TRY(cudaMemcpyAsync(b->d_b, b_dev, bo * sizeof(double), cudaMemcpyDeviceToDevice, st));
   HHL_CUDA_TRY(cudaGraphLaunch(b->exec, st));
-  g_launches.fetch_add(b->graph_launches, std::memory_order_relaxed);
+  g_launches.fetch_add(b->captured, std::memory_order_relaxed);
+  s = run_small(b, b->d_b, nullptr, b->d_out, b->d_eps, st);
+  if (s != HHL_OK) return s;
   HHL_CUDA_TRY(cudaMemcpyAsync(out_dev, b->d_out, oo * sizeof(double), cudaMemcpyDeviceToDevice, st));
   HHL_CUDA_TRY(cudaMemcpyAsync(eps_dev, b->d_eps, b->count * sizeof(double), cudaMemcpyDeviceToDevice, st));
   return HHL_OK;
@@ -534,7 +815,8 @@ hhl_status hhl_batch_run_eager(hhl_batch_t b, void* stream) {
   HHL_CUDA_TRY(cudaEventRecord(fork, st));
   for (auto& w : b->work) HHL_CUDA_TRY(cudaStreamWaitEvent(w.s, fork, 0));
   hhl_status s = HHL_OK;
-  for (int i = 0; i < b->count && s == HHL_OK; ++i) s = enqueue_instance(b, i);
+  for (size_t q = 0; q < b->large.size() && s == HHL_OK; ++q) s = enqueue_instance(b, b->large[q]);
+  if (s == HHL_OK) s = run_small(b, b->d_b, nullptr, b->d_out, b->d_eps, st);
   for (auto& w : b->work) {
     HHL_CUDA_TRY(cudaEventRecord(w.done, w.s));
     HHL_CUDA_TRY(cudaStreamWaitEvent(st, w.done, 0));
@@ -553,11 +835,15 @@ hhl_status hhl_batch_run_host(hhl_batch_t b, const double* b_host, double* out_h
     bo += 2 * b->plans[i].N;
     oo += 4 + 2 * b->plans[i].N;
   }
-  hhl_status s = capture(b, st);
+  hhl_status s = capture(b);
   if (s != HHL_OK) return s;
   HHL_CUDA_TRY(cudaMemcpyAsync(b->d_b, b_host, bo * sizeof(double), cudaMemcpyHostToDevice, st));
-  HHL_CUDA_TRY(cudaGraphLaunch(b->exec, st));
-  g_launches.fetch_add(b->graph_launches, std::memory_order_relaxed);
+  if (b->exec != nullptr) {
+    HHL_CUDA_TRY(cudaGraphLaunch(b->exec, st));
+    g_launches.fetch_add(b->captured, std::memory_order_relaxed);
+  }
+  s = run_small(b, b->d_b, nullptr, b->d_out, b->d_eps, st);
+  if (s != HHL_OK) return s;
   HHL_CUDA_TRY(cudaMemcpyAsync(out_host, b->d_out, oo * sizeof(double), cudaMemcpyDeviceToHost, st));
   HHL_CUDA_TRY(cudaMemcpyAsync(eps_host, b->d_eps, b->count * sizeof(double), cudaMemcpyDeviceToHost, st));
   return hhl_batch_status(b, stream);

@@ -22,12 +22,6 @@ namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Sum NV per-thread values over the block and add them to dst[0..NV) with one atomic each.
 template <int NV>
 __device__ void block_sum_atomic(const double (&v)[NV], double* dst) {
@@ -92,56 +86,6 @@ __global__ void k_prep_fill(const uint4* __restrict__ bs, uint4* __restrict__ st
   for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < 2 * half_units;
        u += (int64_t)gridDim.x * blockDim.x)
     st[u] = u < half_units ? bs[u & (row_units - 1)] : zero;
-}
-
-// Sums of NV per-thread values over the block, returned to every thread (a fixed order).
-template <int NV>
-__device__ void block_sum_all(const double (&v)[NV], double (&total)[NV]) {
-  __shared__ double sh[NV][32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __syncthreads();  // an earlier use may still be read
-#pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    const double s = warp_sum(v[i]);
-    if (lane == 0) sh[i][wid] = s;
-  }
-  __syncthreads();
-  if (wid == 0) {  // (not by every thread: an FP64 addition occupies the narrow pipe for 16 cycles a warp)
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const double s = warp_sum(lane < nw ? sh[i][lane] : 0.0);
-      if (lane == 0) sh[i][0] = s;
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NV; ++i) total[i] = sh[i][0];
-}
-
-// The same for double-float values: shuffled and added on the FP32 pipe, one FP64 value per warp.
-template <int NV>
-__device__ void block_sum_all_df(df (&v)[NV], double (&total)[NV]) {
-  __shared__ double sh[NV][32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NV; ++i) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      v[i] = df_add(v[i], df(__shfl_down_sync(0xffffffffu, v[i].h, o), __shfl_down_sync(0xffffffffu, v[i].l, o)));
-    if (lane == 0) sh[i][wid] = (double)v[i].h + (double)v[i].l;
-  }
-  __syncthreads();
-  if (wid == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const double s = warp_sum(lane < nw ? sh[i][lane] : 0.0);
-      if (lane == 0) sh[i][0] = s;
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NV; ++i) total[i] = sh[i][0];
 }
 
 // Systems of at most kSmallN points: the norm, the scaled row and the fill in one launch instead of

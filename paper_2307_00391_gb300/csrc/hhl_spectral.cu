@@ -52,28 +52,6 @@ constexpr size_t kSpecRowSmem = 128 * 1024;  // system rows of one block of the 
 constexpr int kClockThreads = 128;
 constexpr int kClockBits = 7;                // log2 of the threads of one column (at most)
 
-// Total of per-thread values over the block, in a fixed order, returned to every thread.
-template <int K>
-__device__ void block_totals(const double (&v)[K], double (&total)[K]) {
-  __shared__ double sh[K][32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __syncthreads();  // an earlier use may still be read
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    double s = v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) sh[k][wid] = s;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    double t = 0.0;
-    for (int w = 0; w < nw; ++w) t += sh[k][w];
-    total[k] = t;
-  }
-}
-
 // ------------------------------------------------------------------ plan tables
 // V of the sine basis from its table w sin(q pi / (N + 1)), q < 2N + 2.
 __global__ void k_spec_sine_basis(int N, const double* __restrict__ tab, double* __restrict__ V) {
@@ -180,7 +158,7 @@ __global__ void __launch_bounds__(kSpecThreads) k_spec_prep(const double2* __res
     const double2 z = b[i];
     s[0] += z.x * z.x + z.y * z.y;
   }
-  block_totals(s, nb2);
+  block_sum_all(s, nb2);
   if (threadIdx.x == 0) scal[0] = nb2[0];
   const double scale = nb2[0] > 0.0 ? 1.0 / sqrt(nb2[0]) : 0.0;
   for (int i = threadIdx.x; i < N; i += kSpecThreads) x[i] = make_double2(b[i].x * scale, b[i].y * scale);
@@ -322,7 +300,7 @@ __global__ void __launch_bounds__(kSpecThreads) k_spec_finish(const double2* __r
       }
     }
   }
-  block_totals(s, tot);
+  block_sum_all(s, tot);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     scal[1] = tot[1];
     scal[2] = tot[2];
