@@ -389,6 +389,9 @@ hhl_status launch_qft_register(void* state, int n, int lo, int m, bool inverse, 
 // Whole-register QFT (direction 0, output in bit-reversed order) or inverse QFT (direction 1,
 // input in bit-reversed order) of `outer` consecutive n-qubit states.
 hhl_status launch_qft_whole(void* state, int n, int outer, int direction, int prec, cudaStream_t st);
+// Its large complex64 form (hhl_qft.cu), where qft_whole_tiles says so.
+bool qft_whole_tiles(int n, int log_states);
+hhl_status launch_qft_whole_tiles(void* state, int n, int log_states, int direction, cudaStream_t st);
 hhl_status launch_expm_eigen(int N, int J, const double* d_vr, const double* d_vi, const double* d_cos,
                              const double* d_sin, double wgt, double2* d_u, cudaStream_t st);
 hhl_status launch_store_operands(const Plan& p, const double2* d_u, int k, cudaStream_t st);

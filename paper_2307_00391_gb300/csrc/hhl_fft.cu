@@ -1888,6 +1888,9 @@ hhl_status launch_final_h(const Plan& p, void* state, cudaStream_t st) {
 }
 
 hhl_status launch_qft_whole(void* state, int n, int outer, int direction, int prec, cudaStream_t st) {
+  int log_states = 0;
+  while ((1 << log_states) < outer) ++log_states;
+  if (prec == HHL_PREC_C64 && qft_whole_tiles(n, log_states)) return launch_qft_whole_tiles(state, n, log_states, direction, st);
   return prec == HHL_PREC_C64 ? whole_register_impl<float>(state, n, outer, direction, st)
                               : whole_register_impl<double>(state, n, outer, direction, st);
 }
