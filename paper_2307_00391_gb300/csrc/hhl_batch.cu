@@ -152,17 +152,22 @@ __device__ __forceinline__ void small_parts(const float2* __restrict__ X, int Lp
                                             int in0, int w, bool adjoint, float2 (&y)[RB]) {
   float2 a[4][RB];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
+  for (int q = 0; q < 4; ++q)
 #pragma unroll
     for (int r = 0; r < RB; ++r) a[q][r] = make_float2(0.f, 0.f);
-    for (int c = 4 * w + q; c < N; c += 32) {
-      float2 u = toeplitz_u(g, n, c);
-      if (adjoint) u.y = -u.y;
+  for (int t = 4 * w; t < N; t += 32) {  // (four independent chains of each row)
 #pragma unroll
-      for (int r = 0; r < RB; ++r) {
-        const float2 x = X[c * Lp + pad16(in0 + r)];
-        a[q][r].x = fmaf(u.x, x.x, fmaf(-u.y, x.y, a[q][r].x));
-        a[q][r].y = fmaf(u.x, x.y, fmaf(u.y, x.x, a[q][r].y));
+    for (int q = 0; q < 4; ++q) {
+      const int c = t + q;
+      if (c < N) {
+        float2 u = toeplitz_u(g, n, c);
+        if (adjoint) u.y = -u.y;
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+          const float2 x = X[c * Lp + pad16(in0 + r)];
+          a[q][r].x = fmaf(u.x, x.x, fmaf(-u.y, x.y, a[q][r].x));
+          a[q][r].y = fmaf(u.x, x.y, fmaf(u.y, x.x, a[q][r].y));
+        }
       }
     }
   }
@@ -184,51 +189,63 @@ __device__ __forceinline__ void small_store(float2* X, int Lp, int n, int row, f
   *d = y;
 }
 
-// m output rows from out0 on, each U (or U^dagger) applied to its row from in0 on. With few outputs
-// eight threads share one (a warp's parts each), else a thread takes four rows of one column.
-__device__ void small_product(float2* X, int Lp, const float4* __restrict__ g, int n_s, int m, int in0, int out0,
-                              bool adjoint, bool accumulate, float scale, bool scaled) {
-  const int N = 1 << n_s;
-  if (m < 4 || (m << n_s) < 4 * kSmallThreads) {
-    const int items = m << n_s, lane8 = threadIdx.x & 7;
+// m output rows from out0 on, each U (or U^dagger) applied to its row from in0 on: a thread takes RB
+// rows of one column; while those are fewer than the block's threads, eight threads share them (the
+// parts of one warp each) and add their sums in the order of the warps.
+template <int RB>
+__device__ __forceinline__ void small_rows(float2* X, int Lp, const float4* __restrict__ g, int n_s, int m, int in0, int out0,
+                                           bool adjoint, bool accumulate, float scale, bool scaled) {
+  const int N = 1 << n_s, items = (m / RB) << n_s;
+  float2 y[RB], p[RB];
+  if (items < kSmallThreads) {
+    const int w8 = threadIdx.x & 7, base = threadIdx.x & 24;
     for (int i0 = 0; i0 < items; i0 += kSmallThreads / 8) {  // (whole warps take part in the shuffles)
-      const int it = i0 + (threadIdx.x >> 3);
-      const int n = it & (N - 1), r = it >> n_s;
-      float2 part[1] = {make_float2(0.f, 0.f)};
-      if (it < items && 4 * lane8 < N) small_parts<1>(X, Lp, g, N, n, in0 + r, lane8, adjoint, part);
-      float2 y = part[0];
-      const int base = threadIdx.x & 24;
+      const int it = i0 + (threadIdx.x >> 3), n = it & (N - 1), r = (it >> n_s) * RB;
+#pragma unroll
+      for (int q = 0; q < RB; ++q) p[q] = make_float2(0.f, 0.f);
+      if (it < items && 4 * w8 < N) small_parts<RB>(X, Lp, g, N, n, in0 + r, w8, adjoint, p);
+#pragma unroll
+      for (int q = 0; q < RB; ++q) y[q] = p[q];
 #pragma unroll
       for (int w = 1; w < 8; ++w) {
-        const float px = __shfl_sync(0xffffffffu, part[0].x, base + w);
-        const float py = __shfl_sync(0xffffffffu, part[0].y, base + w);
-        y.x += px;
-        y.y += py;
+#pragma unroll
+        for (int q = 0; q < RB; ++q) {
+          y[q].x += __shfl_sync(0xffffffffu, p[q].x, base + w);
+          y[q].y += __shfl_sync(0xffffffffu, p[q].y, base + w);
+        }
       }
-      if (it < items && lane8 == 0) small_store(X, Lp, n, out0 + r, y, accumulate, scale, scaled);
+      if (it < items && w8 == 0) {
+#pragma unroll
+        for (int q = 0; q < RB; ++q) small_store(X, Lp, n, out0 + r + q, y[q], accumulate, scale, scaled);
+      }
     }
   } else {
-    const int items = (m / 4) << n_s;
     for (int it = threadIdx.x; it < items; it += kSmallThreads) {
-      const int n = it & (N - 1), r = (it >> n_s) * 4;
-      float2 y[4], p[4];
-      small_parts<4>(X, Lp, g, N, n, in0 + r, 0, adjoint, y);
+      const int n = it & (N - 1), r = (it >> n_s) * RB;
+      small_parts<RB>(X, Lp, g, N, n, in0 + r, 0, adjoint, y);
       for (int w = 1; 4 * w < N && w < 8; ++w) {
-        small_parts<4>(X, Lp, g, N, n, in0 + r, w, adjoint, p);
+        small_parts<RB>(X, Lp, g, N, n, in0 + r, w, adjoint, p);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) y[q] = cadd(y[q], p[q]);
+        for (int q = 0; q < RB; ++q) y[q] = cadd(y[q], p[q]);
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) small_store(X, Lp, n, out0 + r + q, y[q], accumulate, scale, scaled);
+      for (int q = 0; q < RB; ++q) small_store(X, Lp, n, out0 + r + q, y[q], accumulate, scale, scaled);
     }
   }
+}
+
+__device__ void small_product(float2* X, int Lp, const float4* __restrict__ g, int n_s, int m, int in0, int out0,
+                              bool adjoint, bool accumulate, float scale, bool scaled) {
+  if (m >= 4) small_rows<4>(X, Lp, g, n_s, m, in0, out0, adjoint, accumulate, scale, scaled);
+  else if (m == 2) small_rows<2>(X, Lp, g, n_s, m, in0, out0, adjoint, accumulate, scale, scaled);
+  else small_rows<1>(X, Lp, g, n_s, m, in0, out0, adjoint, accumulate, scale, scaled);
 }
 
 __device__ __forceinline__ float small_square(float2 a, float2 b) {
   return fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(b.x, b.x, b.y * b.y)));
 }
 
-__global__ void __launch_bounds__(kSmallThreads) k_batch_small(const SmallInst* __restrict__ inst,
+__global__ void __launch_bounds__(kSmallThreads, 3) k_batch_small(const SmallInst* __restrict__ inst,
                                                                const double* __restrict__ b_all, double* __restrict__ b_copy,
                                                                double* __restrict__ out_all, double* __restrict__ eps) {
   extern __shared__ __align__(16) unsigned char small_raw[];
@@ -705,7 +722,7 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
   }
   if (s == HHL_OK && (int)B->large.size() < count) {
     // the one-block solves, largest first, in at most three launches (the shared memory of a launch is
-    // its largest instance's: beyond 16 KiB a quarter of it starts the next)
+    // its largest instance's; past 72 KiB, fewer than three blocks an SM, a quarter of it starts the next)
     std::vector<SmallInst> small;
     std::vector<int> idx;
     for (int i = 0; i < count; ++i)
@@ -726,7 +743,7 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
       d.wall_hi = p.wall_hi;
       d.nu_over_h = p.nu * (double)(p.N + 1);
       d.index = i;
-      if (B->small.empty() || (4 * need(i) < B->small.back().smem && B->small.back().smem > (16 << 10))) B->small.push_back({(int)small.size(), 0, need(i)});
+      if (B->small.empty() || (4 * need(i) < B->small.back().smem && B->small.back().smem > (72 << 10))) B->small.push_back({(int)small.size(), 0, need(i)});
       ++B->small.back().count;
       small.push_back(d);
     }
