@@ -246,6 +246,7 @@ template <class R, bool FULL, int CB>
 __global__ void __launch_bounds__(kFftThreads, 2) k_clock_block(typename Cx<R>::T* __restrict__ S,
                                                              const typename Cx<R>::T* __restrict__ rot, int n_s,
                                                              int n_c, int W) {
+  dep_begin();
   using T = typename Cx<R>::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cg::cluster_group cl = cg::this_cluster();
@@ -343,6 +344,7 @@ __global__ void __launch_bounds__(kFftThreads) k_clock_spec(double2* __restrict_
                                                          const double2* __restrict__ ph_lo,
                                                          const double2* __restrict__ ph_hi,
                                                          const double2* __restrict__ roots, int n_s, int m, int W) {
+  dep_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int L = 1 << m, Lp = L + L / 16 + 1, nh = L > 32 ? L / 32 : 1;
   const int64_t N = 1LL << n_s;
@@ -396,6 +398,7 @@ __global__ void __launch_bounds__(kFftThreads) k_clock_spec(double2* __restrict_
 template <class R, int CB>
 __global__ void __launch_bounds__(kFftThreads, 2) k_register_transform(typename Cx<R>::T* __restrict__ S, int lo, int m,
                                                                     int W, int mode, R scale) {
+  dep_begin();
   using T = typename Cx<R>::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cg::cluster_group cl = cg::this_cluster();
@@ -551,13 +554,14 @@ hhl_status launch_cluster(Kern kernel, int grid, int cb, size_t smem, cudaStream
   cfg.blockDim = dim3(kFftThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 1u << cb;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  attr[1] = dep_attribute();
+  cfg.numAttrs = dep_allowed(st) ? 2 : 1;
   HHL_PROF_BEGIN(st);
   cudaError_t e = cudaLaunchKernelExC(&cfg, (const void*)kernel, args);
   if (e != cudaSuccess) {
@@ -1829,7 +1833,7 @@ hhl_status launch_clock_spec(const Plan& p, void* state, const double2* ph_lo, c
   auto kern = p.full ? k_clock_spec<true> : k_clock_spec<false>;
   HHL_CUDA_TRY(raise_dyn_smem((const void*)kern, smem));
   HHL_PROF_BEGIN(st);
-  kern<<<(unsigned)(p.N / W), kFftThreads, smem, st>>>((double2*)state, (const double2*)p.d_rot, ph_lo, ph_hi, tw, p.n_s,
+  launch_dep(kern, (unsigned)(p.N / W), kFftThreads, smem, st, (double2*)state, (const double2*)p.d_rot, ph_lo, ph_hi, tw, p.n_s,
                                                       p.n_c, W);
   HHL_LAUNCH_CHECK("k_clock_spec");
   return HHL_OK;

@@ -301,6 +301,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (CL > 1) cluster_sync_all();  // every CTA's barriers are initialised before any remote signal
   const uint32_t tmem = tmem_slot;
+  dep_begin();  // (after the set-up; no thread has touched global memory yet)
 
   if (warp == 0) {
     if (lane == 0) {
@@ -463,6 +464,7 @@ template <int BN>
 __global__ void __launch_bounds__(256) k_tc_fixup(const float4* __restrict__ ws, float* __restrict__ state_half,
                                                   int n_s, RowMap rows, int k_iters, int tiles_n, int64_t units,
                                                   int64_t G, int* err) {
+  dep_begin();
   constexpr int kQ = BN / 4;  // float4 per tile row
   const int64_t t = blockIdx.y;
   const int64_t t0u = t * k_iters;
@@ -491,6 +493,7 @@ __global__ void __launch_bounds__(256) k_tc_fixup(const float4* __restrict__ ws,
 // An amplitude component of magnitude >= 2 cannot be represented: error flag 4.
 __global__ void k_tc_split_rows(const float4* __restrict__ half, uint2* __restrict__ a_hi, uint2* __restrict__ a_lo,
                                 int n_s, RowMap rows, int64_t m_sub, int* err) {
+  dep_begin();
   const int row4_bits = n_s - 1;  // float4 per row = 2N/4 = 2^(n_s-1)
   const int64_t total = m_sub << row4_bits;
   constexpr int U = 4;  // loads in flight per thread
@@ -689,7 +692,7 @@ hhl_status launch_tc_gemm_map(int n_s, int64_t m_sub, const RowMap& k, void* hal
   int g = (int)((total4 + 255) / 256);
   if (g > 152 * 16) g = 152 * 16;
   HHL_PROF_BEGIN(st);
-  k_tc_split_rows<<<g, 256, 0, st>>>((const float4*)half, (uint2*)a_hi, (uint2*)a_lo, n_s, k, m_sub, err);
+  launch_dep(k_tc_split_rows, g, 256, 0, st, (const float4*)half, (uint2*)a_hi, (uint2*)a_lo, n_s, k, m_sub, err);
   HHL_LAUNCH_CHECK("k_tc_split_rows");
   // grid: one CTA per tile when the tiles fill at least three quarters of the SMs (or the
   // caller asks for it: the batch, whose streams fill the GPU together); otherwise stream-K,
@@ -717,13 +720,14 @@ hhl_status launch_tc_gemm_map(int n_s, int64_t m_sub, const RowMap& k, void* hal
     cfg.gridDim = dim3((unsigned)G);
     cfg.blockDim = dim3(kThreadsTc);
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 4;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1] = dep_attribute();
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = dep_allowed(st) ? 2 : 1;
     float* sh = (float*)half;
     float* wsp = w.ws;
     const int ti = (int)tiles_n;
@@ -739,11 +743,11 @@ hhl_status launch_tc_gemm_map(int n_s, int64_t m_sub, const RowMap& k, void* hal
     }
     if (e != cudaSuccess) return cuda_fail(e, "k_ctrl_gemm_tc (cluster launch)");
   } else if (bn == 256) {
-    k_ctrl_gemm_tc<256, 1><<<(unsigned)G, kThreadsTc, TcShape<256>::kSmemBytes, st>>>(
+    launch_dep(k_ctrl_gemm_tc<256, 1>, (unsigned)G, kThreadsTc, TcShape<256>::kSmemBytes, st, 
         map_ahi, map_alo, map_bhi, map_blo, (float*)half, n_s, k, k_iters, (int)tiles_n, units, w.ws, err,
         wait_cycles, fault);
   } else {
-    k_ctrl_gemm_tc<128, 1><<<(unsigned)G, kThreadsTc, TcShape<128>::kSmemBytes, st>>>(
+    launch_dep(k_ctrl_gemm_tc<128, 1>, (unsigned)G, kThreadsTc, TcShape<128>::kSmemBytes, st, 
         map_ahi, map_alo, map_bhi, map_blo, (float*)half, n_s, k, k_iters, (int)tiles_n, units, w.ws, err,
         wait_cycles, fault);
   }
@@ -755,10 +759,10 @@ hhl_status launch_tc_gemm_map(int n_s, int64_t m_sub, const RowMap& k, void* hal
   const dim3 fgrid((unsigned)(kBM * (bn / 4) / 256), (unsigned)tiles);
   HHL_PROF_BEGIN(st);
   if (bn == 256)
-    k_tc_fixup<256><<<fgrid, 256, 0, st>>>((const float4*)w.ws, (float*)half, n_s, k, k_iters, (int)tiles_n, units, G,
+    launch_dep(k_tc_fixup<256>, fgrid, 256, 0, st, (const float4*)w.ws, (float*)half, n_s, k, k_iters, (int)tiles_n, units, G,
                                            err);
   else
-    k_tc_fixup<128><<<fgrid, 256, 0, st>>>((const float4*)w.ws, (float*)half, n_s, k, k_iters, (int)tiles_n, units, G,
+    launch_dep(k_tc_fixup<128>, fgrid, 256, 0, st, (const float4*)w.ws, (float*)half, n_s, k, k_iters, (int)tiles_n, units, G,
                                            err);
   HHL_LAUNCH_CHECK("k_tc_fixup");
   return HHL_OK;

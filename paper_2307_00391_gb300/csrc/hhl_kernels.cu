@@ -82,6 +82,7 @@ __global__ void k_prep_scale(const double2* __restrict__ b, const double* __rest
 // Every clock row of the anc = 0 half gets bs, the anc = 1 half is zeroed: 16-byte stores.
 __global__ void k_prep_fill(const uint4* __restrict__ bs, uint4* __restrict__ st, int64_t row_units,
                             int64_t half_units) {
+  dep_begin();
   const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
   for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < 2 * half_units;
        u += (int64_t)gridDim.x * blockDim.x)
@@ -98,6 +99,7 @@ template <class R>
 __global__ void __launch_bounds__(kThreads) k_prep_small(const double2* __restrict__ b, int N, int n_c,
                                                          double* __restrict__ scal, uint4* __restrict__ st,
                                                          int64_t half_units, int row_only) {
+  dep_begin();
   using T = typename Cx<R>::T;
   extern __shared__ __align__(16) unsigned char prep_smem[];
   T* row = reinterpret_cast<T*>(prep_smem);
@@ -130,6 +132,7 @@ __global__ void __launch_bounds__(256) k_ctrl_gemm_simt(const typename Cx<R>::T*
                                                         typename Cx<R>::T* __restrict__ out,
                                                         const typename Cx<R>::T* __restrict__ B,
                                                         int n_s, RowMap rows, int64_t m_sub) {
+  dep_begin();
   using T = typename Cx<R>::T;
   constexpr int TM = BM / 16, TN = BN / 16;
   __shared__ T As[BK][BM + 1];
@@ -195,6 +198,7 @@ __global__ void __launch_bounds__(256) k_ctrl_gemm_simt(const typename Cx<R>::T*
 template <class R>
 __global__ void k_rows_scatter(typename Cx<R>::T* __restrict__ S, const typename Cx<R>::T* __restrict__ out,
                                int n_s, RowMap rows, int64_t m_sub) {
+  dep_begin();
   const int64_t N = 1LL << n_s;
   const int64_t total = m_sub * N;
   const R sc = (R)rows.scale;
@@ -317,6 +321,7 @@ __device__ __forceinline__ void measure_block(const typename Cx<R>::T* __restric
 }
 template <class R, bool DF>
 __global__ void k_measure_sums(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N, double* acc) {
+  dep_begin();
   double t[3];
   measure_block<R, DF>(S, half, N, t);
   if (threadIdx.x < 3) atomicAdd(acc + threadIdx.x, threadIdx.x == 0 ? t[0] : threadIdx.x == 1 ? t[1] : t[2]);
@@ -348,6 +353,7 @@ template <class R, bool DF>
 __global__ void __launch_bounds__(kThreads) k_measure_small(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
                                                             double* __restrict__ scal, double* __restrict__ part,
                                                             unsigned* __restrict__ ticket, double* __restrict__ out) {
+  dep_begin();
   __shared__ bool last;
   double a[3], t[3];
   measure_block<R, DF>(S, half, N, t);
@@ -375,6 +381,7 @@ __global__ void __launch_bounds__(kThreads) k_measure_small(const typename Cx<R>
 template <class R>
 __global__ void __launch_bounds__(kThreads) k_row_finish_small(const typename Cx<R>::T* __restrict__ v, int64_t N,
                                                                double* __restrict__ scal, double* __restrict__ out) {
+  dep_begin();
   double s[1] = {0.0}, t[1];
   for (int64_t j = threadIdx.x; j < N; j += kThreads) {
     const double re = (double)v[j].x, im = (double)v[j].y;
@@ -578,6 +585,7 @@ __global__ void __launch_bounds__(kThreads) k_diss_small(const typename Cx<R>::T
                                                          double* __restrict__ scal, double inv_c_lam, double wlo, double whi,
                                                          double nu_over_h, double* __restrict__ eps,
                                                          double* __restrict__ u_out) {
+  dep_begin();
   const double scale = sqrt(scal[0]) * inv_c_lam;
   double s[1] = {0.0}, t[1];
   for (int i = threadIdx.x; i <= N; i += kThreads) {
@@ -716,7 +724,7 @@ hhl_status prep_small(const Plan& p, const double* b, void* state, bool row_only
   const int64_t half_units = p.R * p.N * (int64_t)p.amp_bytes() / 16;
   const int g = row_only ? 1 : grid_for(2 * half_units, kThreads, 152);  // the FP64 norm and scale: once per SM
   HHL_PROF_BEGIN(st);
-  k_prep_small<R><<<g, kThreads, (size_t)p.N * p.amp_bytes(), st>>>((const double2*)b, (int)p.N, p.n_c, p.d_scal,
+  launch_dep(k_prep_small<R>, g, kThreads, (size_t)p.N * p.amp_bytes(), st, (const double2*)b, (int)p.N, p.n_c, p.d_scal,
                                                                    (uint4*)state, half_units, row_only);
   HHL_LAUNCH_CHECK("k_prep_small");
   return HHL_OK;
@@ -745,7 +753,7 @@ hhl_status launch_prep_fill(const Plan& p, const double* b, void* state, cudaStr
   const int64_t half_units = p.R * row_units;
   const int g = grid_for(2 * half_units, kThreads, 152 * 16);
   HHL_PROF_BEGIN(st);
-  k_prep_fill<<<g, kThreads, 0, st>>>((const uint4*)p.d_bs, (uint4*)state, row_units, half_units);
+  launch_dep(k_prep_fill, g, kThreads, 0, st, (const uint4*)p.d_bs, (uint4*)state, row_units, half_units);
   HHL_LAUNCH_CHECK("k_prep_fill");
   return HHL_OK;
 }
@@ -794,18 +802,18 @@ hhl_status launch_ctrl_u_simt_map(const Plan& p, void* half, const RowMap& k, in
   const int sg = grid_for(m_sub * N, kThreads, 152 * 32);
   if (p.prec == HHL_PREC_C64) {
     HHL_PROF_BEGIN(st);
-    k_ctrl_gemm_simt<float, 64, 64, 16><<<grid, 256, 0, st>>>((const float2*)half, (float2*)p.d_scratch,
+    launch_dep(k_ctrl_gemm_simt<float, 64, 64, 16>, grid, 256, 0, st, (const float2*)half, (float2*)p.d_scratch,
                                                               (const float2*)B, p.n_s, k, m_sub);
     HHL_LAUNCH_CHECK("k_ctrl_gemm_simt<f32>");
     HHL_PROF_BEGIN(st);
-    k_rows_scatter<float><<<sg, kThreads, 0, st>>>((float2*)half, (const float2*)p.d_scratch, p.n_s, k, m_sub);
+    launch_dep(k_rows_scatter<float>, sg, kThreads, 0, st, (float2*)half, (const float2*)p.d_scratch, p.n_s, k, m_sub);
   } else {
     HHL_PROF_BEGIN(st);
-    k_ctrl_gemm_simt<double, 64, 64, 8><<<grid, 256, 0, st>>>((const double2*)half, (double2*)p.d_scratch,
+    launch_dep(k_ctrl_gemm_simt<double, 64, 64, 8>, grid, 256, 0, st, (const double2*)half, (double2*)p.d_scratch,
                                                               (const double2*)B, p.n_s, k, m_sub);
     HHL_LAUNCH_CHECK("k_ctrl_gemm_simt<f64>");
     HHL_PROF_BEGIN(st);
-    k_rows_scatter<double><<<sg, kThreads, 0, st>>>((double2*)half, (const double2*)p.d_scratch, p.n_s, k, m_sub);
+    launch_dep(k_rows_scatter<double>, sg, kThreads, 0, st, (double2*)half, (const double2*)p.d_scratch, p.n_s, k, m_sub);
   }
   HHL_LAUNCH_CHECK("k_rows_scatter");
   return HHL_OK;
@@ -818,11 +826,11 @@ hhl_status launch_measure_sums(const Plan& p, const void* state, cudaStream_t st
   const char* env = getenv("HHL_FP64_PIPE");
   HHL_PROF_BEGIN(st);
   if (p.prec == HHL_PREC_C64)
-    k_measure_sums<float, false><<<g, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal + 1);
+    launch_dep(k_measure_sums<float, false>, g, kThreads, 0, st, (const float2*)state, half, p.N, p.d_scal + 1);
   else if (env != nullptr && atoi(env) != 0)
-    k_measure_sums<double, false><<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
+    launch_dep(k_measure_sums<double, false>, g, kThreads, 0, st, (const double2*)state, half, p.N, p.d_scal + 1);
   else
-    k_measure_sums<double, true><<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
+    launch_dep(k_measure_sums<double, true>, g, kThreads, 0, st, (const double2*)state, half, p.N, p.d_scal + 1);
   HHL_LAUNCH_CHECK("k_measure_sums");
   return HHL_OK;
 }
@@ -831,8 +839,8 @@ hhl_status launch_measure_row(const Plan& p, const void* state, double* out, cud
   const int64_t half = p.R * p.N;
   if (p.N <= kSmallN) {
     HHL_PROF_BEGIN(st);
-    if (p.prec == HHL_PREC_C64) k_row_finish_small<float><<<1, kThreads, 0, st>>>((const float2*)state + half, p.N, p.d_scal, out);
-    else k_row_finish_small<double><<<1, kThreads, 0, st>>>((const double2*)state + half, p.N, p.d_scal, out);
+    if (p.prec == HHL_PREC_C64) launch_dep(k_row_finish_small<float>, 1, kThreads, 0, st, (const float2*)state + half, p.N, p.d_scal, out);
+    else launch_dep(k_row_finish_small<double>, 1, kThreads, 0, st, (const double2*)state + half, p.N, p.d_scal, out);
     HHL_LAUNCH_CHECK("k_row_finish_small");
     return HHL_OK;
   }
@@ -878,11 +886,11 @@ hhl_status launch_measure(const Plan& p, const void* state, double* out, cudaStr
     unsigned* ticket = reinterpret_cast<unsigned*>(p.d_part + 3 * kMeasureBlocks);
     HHL_PROF_BEGIN(st);
     if (p.prec == HHL_PREC_C64)
-      k_measure_small<float, false><<<gm, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal, p.d_part, ticket, out);
+      launch_dep(k_measure_small<float, false>, gm, kThreads, 0, st, (const float2*)state, half, p.N, p.d_scal, p.d_part, ticket, out);
     else if (env != nullptr && atoi(env) != 0)
-      k_measure_small<double, false><<<gm, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal, p.d_part, ticket, out);
+      launch_dep(k_measure_small<double, false>, gm, kThreads, 0, st, (const double2*)state, half, p.N, p.d_scal, p.d_part, ticket, out);
     else
-      k_measure_small<double, true><<<gm, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal, p.d_part, ticket, out);
+      launch_dep(k_measure_small<double, true>, gm, kThreads, 0, st, (const double2*)state, half, p.N, p.d_scal, p.d_part, ticket, out);
     HHL_LAUNCH_CHECK("k_measure_small");
     return HHL_OK;
   }
@@ -891,7 +899,7 @@ hhl_status launch_measure(const Plan& p, const void* state, double* out, cudaStr
   const int gf = grid_for(p.N, kThreads, 152 * 4);
   if (p.prec == HHL_PREC_C64) {
     HHL_PROF_BEGIN(st);
-    k_measure_sums<float, false><<<g, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal + 1);
+    launch_dep(k_measure_sums<float, false>, g, kThreads, 0, st, (const float2*)state, half, p.N, p.d_scal + 1);
     HHL_LAUNCH_CHECK("k_measure_sums");
     HHL_PROF_BEGIN(st);
     k_measure_finish<float><<<gf, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal, out);
@@ -899,9 +907,9 @@ hhl_status launch_measure(const Plan& p, const void* state, double* out, cudaStr
     const char* env = getenv("HHL_FP64_PIPE");
     HHL_PROF_BEGIN(st);
     if (env != nullptr && atoi(env) != 0)
-      k_measure_sums<double, false><<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
+      launch_dep(k_measure_sums<double, false>, g, kThreads, 0, st, (const double2*)state, half, p.N, p.d_scal + 1);
     else
-      k_measure_sums<double, true><<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal + 1);
+      launch_dep(k_measure_sums<double, true>, g, kThreads, 0, st, (const double2*)state, half, p.N, p.d_scal + 1);
     HHL_LAUNCH_CHECK("k_measure_sums");
     HHL_PROF_BEGIN(st);
     k_measure_finish<double><<<gf, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal, out);
@@ -939,7 +947,7 @@ hhl_status launch_prep_qsp1(const Plan& p, const double* b, double* tree, double
   const int64_t row_units = p.N * (int64_t)p.amp_bytes() / 16;
   const int64_t half_units = p.R * row_units;
   HHL_PROF_BEGIN(st);
-  k_prep_fill<<<grid_for(2 * half_units, kThreads, 152 * 16), kThreads, 0, st>>>((const uint4*)p.d_bs, (uint4*)state,
+  launch_dep(k_prep_fill, grid_for(2 * half_units, kThreads, 152 * 16), kThreads, 0, st, (const uint4*)p.d_bs, (uint4*)state,
                                                                                 row_units, half_units);
   HHL_LAUNCH_CHECK("k_prep_fill");
   return HHL_OK;
@@ -993,7 +1001,7 @@ hhl_status launch_prep_qsp2(const Plan& p, const int64_t* idx, const double* val
   const int64_t row_units = p.N * (int64_t)p.amp_bytes() / 16;
   const int64_t half_units = p.R * row_units;
   HHL_PROF_BEGIN(st);
-  k_prep_fill<<<grid_for(2 * half_units, kThreads, 152 * 16), kThreads, 0, st>>>((const uint4*)p.d_bs, (uint4*)state,
+  launch_dep(k_prep_fill, grid_for(2 * half_units, kThreads, 152 * 16), kThreads, 0, st, (const uint4*)p.d_bs, (uint4*)state,
                                                                                 row_units, half_units);
   HHL_LAUNCH_CHECK("k_prep_fill");
   return HHL_OK;
@@ -1022,10 +1030,10 @@ hhl_status launch_dissipation(const Plan& p, const void* state, double* eps, dou
   if (p.N <= kSmallN) {
     HHL_PROF_BEGIN(st);
     if (p.prec == HHL_PREC_C64)
-      k_diss_small<float><<<1, kThreads, 0, st>>>((const float2*)state + half, (int)p.N, p.d_scal, inv_c_lam, p.wall_lo,
+      launch_dep(k_diss_small<float>, 1, kThreads, 0, st, (const float2*)state + half, (int)p.N, p.d_scal, inv_c_lam, p.wall_lo,
                                                   p.wall_hi, p.nu * (double)(p.N + 1), eps, u_dev);
     else
-      k_diss_small<double><<<1, kThreads, 0, st>>>((const double2*)state + half, (int)p.N, p.d_scal, inv_c_lam, p.wall_lo,
+      launch_dep(k_diss_small<double>, 1, kThreads, 0, st, (const double2*)state + half, (int)p.N, p.d_scal, inv_c_lam, p.wall_lo,
                                                    p.wall_hi, p.nu * (double)(p.N + 1), eps, u_dev);
     HHL_LAUNCH_CHECK("k_diss_small");
     return HHL_OK;
@@ -1154,6 +1162,7 @@ int64_t toeplitz_rows_limit() {
 template <int MT, int TN>
 __global__ void __launch_bounds__(256) k_toeplitz_rows(float2* __restrict__ half, int n_s, const float4* __restrict__ g,
                                                        int adjoint, RowMap rows, int64_t m_rows) {
+  dep_begin();
   constexpr int P = 256 / TN;                      // parts of each output
   constexpr int CH = toep_chunk<MT>();             // columns per chunk
   constexpr int kXs = MT * CH;                     // staged x values per chunk
@@ -1280,6 +1289,7 @@ constexpr int kToepKs = 4;
 template <int MT, int TN>
 __global__ void __launch_bounds__(256) k_toeplitz_rows_ks(float2* __restrict__ half, int n_s, const float4* __restrict__ g,
                                                           int adjoint, RowMap rows, int64_t m_rows) {
+  dep_begin();
   namespace cg = cooperative_groups;
   constexpr int P = 256 / TN, CH = 256;
   constexpr int kXs = MT * CH, kLd = kXs / 256, kGl = (TN + CH + 255) / 256;
@@ -1408,13 +1418,14 @@ cudaError_t toeplitz_rows_ks_launch(dim3 grid, cudaStream_t st, float2* half, in
   cfg.gridDim = grid;
   cfg.blockDim = dim3(256);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = kToepKs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1] = dep_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = dep_allowed(st) ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k_toeplitz_rows_ks<MT, TN>, half, n_s, g, adjoint, rows, m);
 }
 
@@ -1432,7 +1443,7 @@ cudaError_t toeplitz_rows_launch(dim3 grid, cudaStream_t st, float2* half, int n
   constexpr int smem = toep_smem<MT, TN>();
   cudaError_t e = raise_dyn_smem((const void*)k_toeplitz_rows<MT, TN>, smem);
   if (e != cudaSuccess) return e;
-  k_toeplitz_rows<MT, TN><<<grid, 256, smem, st>>>(half, n_s, g, adjoint, rows, m);
+  launch_dep(k_toeplitz_rows<MT, TN>, grid, 256, smem, st, half, n_s, g, adjoint, rows, m);
   return cudaSuccess;
 }
 

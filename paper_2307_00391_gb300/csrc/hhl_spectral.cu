@@ -93,6 +93,7 @@ __global__ void k_spec_phases(int N, int R, const unsigned long long* __restrict
 template <int RPT>
 __global__ void __launch_bounds__(kSpecThreads) k_spec_rows(double2* __restrict__ X, const double* __restrict__ B, int N,
                                                             long long rows) {
+  dep_begin();
   extern __shared__ __align__(16) unsigned char spec_smem[];
   double2* xs = reinterpret_cast<double2*>(spec_smem);
   const int tn = N < kSpecThreads ? N : kSpecThreads, rg = kSpecThreads / tn, BM = RPT * rg;
@@ -130,7 +131,7 @@ hhl_status rows_launch(double2* X, const double* B, int N, long long rows, cudaS
   const size_t smem = (size_t)bm * N * sizeof(double2);
   HHL_CUDA_TRY(raise_dyn_smem((const void*)k_spec_rows<RPT>, smem));
   HHL_PROF_BEGIN(st);
-  k_spec_rows<RPT><<<(unsigned)((rows + bm - 1) / bm), kSpecThreads, smem, st>>>(X, B, N, rows);
+  launch_dep(k_spec_rows<RPT>, (unsigned)((rows + bm - 1) / bm), kSpecThreads, smem, st, X, B, N, rows);
   HHL_LAUNCH_CHECK("k_spec_rows");
   return HHL_OK;
 }
@@ -153,6 +154,7 @@ hhl_status spec_rows(double2* X, const double* B, int N, long long rows, cudaStr
 // |b|^2 and bhat = b / |b|; one block.
 __global__ void __launch_bounds__(kSpecThreads) k_spec_prep(const double2* __restrict__ b, int N,
                                                             double* __restrict__ scal, double2* __restrict__ x) {
+  dep_begin();
   double s[1] = {0.0}, nb2[1];
   for (int i = threadIdx.x; i < N; i += kSpecThreads) {
     const double2 z = b[i];
@@ -168,6 +170,7 @@ __global__ void __launch_bounds__(kSpecThreads) k_spec_prep(const double2* __res
 // 8 threads, whose partial sums are added in a fixed order.
 __global__ void __launch_bounds__(kSpecThreads) k_spec_matvec(const double* __restrict__ B, const double2* __restrict__ x,
                                                               int N, double2* __restrict__ y) {
+  dep_begin();
   __shared__ double2 part[kSpecThreads / 32][8];
   const int o = blockIdx.x * 8 + (threadIdx.x & 7), p = threadIdx.x >> 3;
   double2 acc = make_double2(0.0, 0.0);
@@ -201,6 +204,7 @@ __global__ void __launch_bounds__(kSpecThreads) k_spec_matvec(const double* __re
 __global__ void __launch_bounds__(kClockThreads) k_spec_tree(const unsigned long long* __restrict__ frac,
                                                              const double* __restrict__ rot, int n_c, int N,
                                                              double2* __restrict__ beta, double2* __restrict__ wts) {
+  dep_begin();
   __shared__ double red[4][3];
   const int nb = n_c < kClockBits ? n_c : kClockBits, lb = n_c - nb;
   const int tpc = 1 << nb, t = threadIdx.x & (tpc - 1);
@@ -284,6 +288,7 @@ __global__ void __launch_bounds__(kSpecThreads) k_spec_finish(const double2* __r
                                                               int N, double* __restrict__ scal, double inv_c_lam,
                                                               double wall_lo, double wall_hi, double nu_over_h,
                                                               double* __restrict__ out, double* __restrict__ eps) {
+  dep_begin();
   const double scale = sqrt(scal[0]) * inv_c_lam;  // u = |b| Re(v) / (C lambda_ub)
   double s[4] = {0.0, 0.0, 0.0, 0.0}, tot[4];
   for (int i = threadIdx.x; i < N; i += kSpecThreads) {
@@ -333,20 +338,20 @@ hhl_status launch_spec_solve(const Plan& p, const double* b, double2* v_row, dou
   const SpecState& s = *p.spec;
   const int N = (int)p.N;
   HHL_PROF_BEGIN(st);
-  k_spec_prep<<<1, kSpecThreads, 0, st>>>((const double2*)b, N, p.d_scal, s.x);
+  launch_dep(k_spec_prep, 1, kSpecThreads, 0, st, (const double2*)b, N, p.d_scal, s.x);
   HHL_LAUNCH_CHECK("k_spec_prep");
   HHL_PROF_BEGIN(st);
-  k_spec_matvec<<<(N + 7) / 8, kSpecThreads, 0, st>>>(s.basis, s.x, N, s.beta);
+  launch_dep(k_spec_matvec, (N + 7) / 8, kSpecThreads, 0, st, s.basis, s.x, N, s.beta);
   HHL_LAUNCH_CHECK("k_spec_matvec");
   const int cols = kClockThreads >> std::min(p.n_c, kClockBits);
   HHL_PROF_BEGIN(st);
-  k_spec_tree<<<(N + cols - 1) / cols, kClockThreads, 0, st>>>(s.frac, s.sin_half, p.n_c, N, s.beta, s.wts);
+  launch_dep(k_spec_tree, (N + cols - 1) / cols, kClockThreads, 0, st, s.frac, s.sin_half, p.n_c, N, s.beta, s.wts);
   HHL_LAUNCH_CHECK("k_spec_tree");
   HHL_PROF_BEGIN(st);
-  k_spec_matvec<<<(N + 7) / 8, kSpecThreads, 0, st>>>(s.basis_t, s.beta, N, v_row);
+  launch_dep(k_spec_matvec, (N + 7) / 8, kSpecThreads, 0, st, s.basis_t, s.beta, N, v_row);
   HHL_LAUNCH_CHECK("k_spec_matvec");
   HHL_PROF_BEGIN(st);
-  k_spec_finish<<<std::max(1, std::min(16, N / kSpecThreads)), kSpecThreads, 0, st>>>(
+  launch_dep(k_spec_finish, std::max(1, std::min(16, N / kSpecThreads)), kSpecThreads, 0, st, 
       v_row, s.wts, N, p.d_scal, 1.0 / (p.C * p.lam_ub), p.wall_lo, p.wall_hi, p.nu * (double)(p.N + 1), out, eps);
   HHL_LAUNCH_CHECK("k_spec_finish");
   return HHL_OK;
