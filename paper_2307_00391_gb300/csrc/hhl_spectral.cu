@@ -32,6 +32,7 @@
 namespace hhl {
 
 struct SpecState {
+  void* mem = nullptr;        // one allocation for everything below
   double* basis = nullptr;    // V, N x N row-major (column j: eigenvector j)
   double* basis_t = nullptr;  // V^T (the same buffer for the symmetric sine basis)
   unsigned long long* frac = nullptr;  // N: phi_j / (2 pi) mod 1 in units of 2^-64
@@ -358,79 +359,68 @@ hhl_status launch_spec_solve(const Plan& p, const double* b, double2* v_row, dou
 }
 
 void spec_free(Plan& p) {
-  SpecState* s = p.spec;
-  if (s == nullptr) return;
-  if (s->basis_t != s->basis && s->basis_t) cudaFree(s->basis_t);
-  void* ptrs[] = {s->basis, s->frac, s->ph_lo, s->ph_hi, s->tw, s->sin_half, s->x, s->beta, s->wts};
-  for (void* q : ptrs)
-    if (q) cudaFree(q);
-  delete s;
+  if (p.spec == nullptr) return;
+  if (p.spec->mem) cudaFree(p.spec->mem);
+  delete p.spec;
   p.spec = nullptr;
 }
 
 hhl_status spec_create(Plan& p, const std::vector<double>& lam, const std::vector<double>* vec, cudaStream_t st) {
-  const int N = (int)p.N, R = (int)p.R, nh = R > 32 ? R / 32 : 1;
-  const size_t mat = (size_t)N * N * sizeof(double);
+  const size_t N = (size_t)p.N, R = (size_t)p.R, nh = R > 32 ? R / 32 : 1, mat = N * N;
   SpecState* s = new SpecState();
   p.spec = s;  // the plan's destructor frees what a failure below leaves
-  double* d_sine = nullptr;
-  auto alloc = [&](auto** q, size_t bytes) {
-    p.table_bytes += bytes;
-    return cudaMalloc((void**)q, bytes) == cudaSuccess;
-  };
-  const bool ok = alloc(&s->basis, mat) && (vec == nullptr || alloc(&s->basis_t, mat)) &&
-                  alloc(&s->frac, (size_t)N * sizeof(unsigned long long)) && alloc(&s->ph_lo, (size_t)N * 32 * sizeof(double2)) &&
-                  alloc(&s->ph_hi, (size_t)N * nh * sizeof(double2)) && alloc(&s->tw, (size_t)R * sizeof(double2)) &&
-                  alloc(&s->sin_half, (size_t)R * sizeof(double)) && alloc(&s->x, (size_t)N * sizeof(double2)) &&
-                  alloc(&s->beta, (size_t)N * sizeof(double2)) && alloc(&s->wts, (size_t)N * sizeof(double2)) &&
-                  (vec != nullptr || cudaMalloc((void**)&d_sine, (2 * (size_t)N + 2) * sizeof(double)) == cudaSuccess);
-  if (!ok) {
-    cudaGetLastError();
-    if (d_sine) cudaFree(d_sine);
-    return fail(HHL_ERR_OOM, "eigenbasis tables");
-  }
-  if (vec == nullptr) s->basis_t = s->basis;
-  std::vector<unsigned long long> frac(N);
-  for (int j = 0; j < N; ++j) {
+  // What the host computes comes first and is copied at once (in units of 8 bytes): the phase
+  // fractions, sin(theta_y / 2), and V, V^T or the sine table.
+  std::vector<double> host(N + R + (vec != nullptr ? 2 * mat : 2 * N + 2));
+  unsigned long long* frac = reinterpret_cast<unsigned long long*>(host.data());
+  double *sh = host.data() + N, *basis = sh + R;
+  for (size_t j = 0; j < N; ++j) {
     double t = lam[j] / p.lam_ub * p.t0 / (2.0 * kPiS * (double)R);
     t -= floor(t);
     frac[j] = t < 1.0 ? (unsigned long long)(t * 18446744073709551616.0) : 0ULL;
   }
-  std::vector<double> sh(R), tab, vt;
-  for (int y = 0; y < R; ++y) sh[y] = sin(p.theta[y] / 2.0);
-  cudaError_t e = cudaMemcpyAsync(s->frac, frac.data(), N * sizeof(unsigned long long), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(s->sin_half, sh.data(), R * sizeof(double), cudaMemcpyHostToDevice, st);
-  if (vec == nullptr) {
-    tab.resize(2 * (size_t)N + 2);
-    const double w = sqrt(2.0 / (N + 1));
-    for (int q = 0; q < 2 * N + 2; ++q) tab[q] = w * sin((double)q * kPiS / (N + 1));
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_sine, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) {
-      HHL_PROF_BEGIN(st);
-      k_spec_sine_basis<<<(unsigned)std::min<long long>(((long long)N * N + 255) / 256, 152 * 16), 256, 0, st>>>(N, d_sine, s->basis);
-      g_launches.fetch_add(1, std::memory_order_relaxed);
-      if (g_prof_on.load(std::memory_order_relaxed)) prof_end("k_spec_sine_basis");
-      e = cudaGetLastError();
-    }
+  for (size_t y = 0; y < R; ++y) sh[y] = sin(p.theta[y] / 2.0);
+  if (vec != nullptr) {
+    std::copy(vec->begin(), vec->end(), basis);
+    for (size_t a = 0; a < N; ++a)
+      for (size_t c = 0; c < N; ++c) basis[mat + c * N + a] = (*vec)[a * N + c];
   } else {
-    vt.resize((size_t)N * N);
-    for (int a = 0; a < N; ++a)
-      for (int c = 0; c < N; ++c) vt[(size_t)c * N + a] = (*vec)[(size_t)a * N + c];
-    if (e == cudaSuccess) e = cudaMemcpyAsync(s->basis, vec->data(), mat, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(s->basis_t, vt.data(), mat, cudaMemcpyHostToDevice, st);
+    const double w = sqrt(2.0 / (double)(N + 1));
+    for (size_t q = 0; q < 2 * N + 2; ++q) basis[q] = w * sin((double)q * kPiS / (double)(N + 1));
   }
-  if (e == cudaSuccess) {
-    const long long total = (long long)N * (32 + nh) + R;
+  const size_t host_units = (host.size() + 1) & ~(size_t)1;  // (complex tables from a 16-byte boundary)
+  const size_t cplx = N * 32 + N * nh + R + 3 * N;
+  const size_t bytes = (host_units + (vec != nullptr ? 0 : mat) + 2 * cplx) * sizeof(double);
+  if (cudaMalloc(&s->mem, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    s->mem = nullptr;
+    return fail(HHL_ERR_OOM, "eigenbasis tables");
+  }
+  p.table_bytes += bytes;
+  double* d = static_cast<double*>(s->mem);
+  s->frac = reinterpret_cast<unsigned long long*>(d);
+  s->sin_half = d + N;
+  double2* z = reinterpret_cast<double2*>(d + host_units);
+  s->ph_lo = z;
+  s->ph_hi = s->ph_lo + N * 32;
+  s->tw = s->ph_hi + N * nh;
+  s->x = s->tw + R;
+  s->beta = s->x + N;
+  s->wts = s->beta + N;
+  s->basis = vec != nullptr ? d + N + R : reinterpret_cast<double*>(s->wts + N);
+  s->basis_t = vec != nullptr ? s->basis + mat : s->basis;  // (the sine basis is symmetric)
+  HHL_CUDA_TRY(cudaMemcpyAsync(d, host.data(), host.size() * sizeof(double), cudaMemcpyHostToDevice, st));
+  if (vec == nullptr) {
     HHL_PROF_BEGIN(st);
-    k_spec_phases<<<(unsigned)std::min<long long>((total + 255) / 256, 152 * 16), 256, 0, st>>>(N, R, s->frac, s->ph_lo,
-                                                                                            s->ph_hi, s->tw);
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    if (g_prof_on.load(std::memory_order_relaxed)) prof_end("k_spec_phases");
-    e = cudaGetLastError();
+    k_spec_sine_basis<<<(unsigned)std::min<size_t>((mat + 255) / 256, 152 * 16), 256, 0, st>>>((int)N, d + N + R, s->basis);
+    HHL_LAUNCH_CHECK("k_spec_sine_basis");
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the host tables go out of scope
-  if (d_sine) cudaFree(d_sine);
-  return e == cudaSuccess ? HHL_OK : cuda_fail(e, "eigenbasis tables");
+  HHL_PROF_BEGIN(st);
+  k_spec_phases<<<(unsigned)std::min<size_t>((N * (32 + nh) + R + 255) / 256, 152 * 16), 256, 0, st>>>(
+      (int)N, (int)R, s->frac, s->ph_lo, s->ph_hi, s->tw);
+  HHL_LAUNCH_CHECK("k_spec_phases");
+  HHL_CUDA_TRY(cudaStreamSynchronize(st));  // the host copy goes out of scope
+  return HHL_OK;
 }
 
 }  // namespace hhl
