@@ -873,8 +873,9 @@ hhl_status hhl_prepare_rhs_qsp2(hhl_plan_t plan, const int64_t* idx_dev, const d
   return hhl::launch_prep_qsp2(p, idx_dev, val_dev, count, (double2*)p.d_b, state_dev, (cudaStream_t)stream);
 }
 
-static hhl_status ctrl_u(const Plan& p, void* half, int k, bool adj, cudaStream_t st) {
-  if (p.gemm_impl == HHL_GEMM_TCGEN05) return hhl::launch_ctrl_u_tc(p, half, k, adj, st);
+// kn: the clock bit of the product that follows on the same half (-1: none), for tcgen05 chains
+static hhl_status ctrl_u(const Plan& p, void* half, int k, bool adj, int kn, hhl::TcChain* chain, cudaStream_t st) {
+  if (p.gemm_impl == HHL_GEMM_TCGEN05) return hhl::launch_ctrl_u_tc(p, half, k, adj, kn, chain, st);
   return hhl::launch_ctrl_u_dense(p, half, k, adj, st);
 }
 
@@ -886,11 +887,12 @@ hhl_status hhl_apply_stage(hhl_plan_t plan, int32_t stage, void* state_dev, void
   char* s0 = (char*)state_dev;
   char* s1 = s0 + (size_t)(p.R * p.N) * p.amp_bytes();
   hhl_status s = HHL_OK;
+  hhl::TcChain chain;
   switch (stage) {
     case HHL_STAGE_QPE_U:
       if (p.expm_mode == HHL_EXPM_TROTTER) return hhl::launch_trotter(p, s0, false, st);
       s = hhl::tc_reset_error(p, st);  // a new circuit: the GEMM status covers it alone
-      for (int k = 0; k < p.n_c && s == HHL_OK; ++k) s = ctrl_u(p, s0, k, false, st);
+      for (int k = 0; k < p.n_c && s == HHL_OK; ++k) s = ctrl_u(p, s0, k, false, k + 1 < p.n_c ? k + 1 : -1, &chain, st);
       return s;
     case HHL_STAGE_CLOCK_BLOCK:
       return hhl::launch_clock_block(p, state_dev, st);
@@ -901,8 +903,9 @@ hhl_status hhl_apply_stage(hhl_plan_t plan, int32_t stage, void* state_dev, void
         return s;
       }
       for (int k = p.n_c - 1; k >= 0 && s == HHL_OK; --k) {
-        s = ctrl_u(p, s1, k, true, st);
-        if (s == HHL_OK && p.full) s = ctrl_u(p, s0, k, true, st);
+        // (both halves: their products alternate, so no chain)
+        s = ctrl_u(p, s1, k, true, p.full ? -1 : k - 1, p.full ? nullptr : &chain, st);
+        if (s == HHL_OK && p.full) s = ctrl_u(p, s0, k, true, -1, nullptr, st);
       }
       return s;
     case HHL_STAGE_FINAL_H:
@@ -940,8 +943,9 @@ hhl_status hhl_solve_postselected(hhl_plan_t plan, const double* b_dev, void* st
   // the trees as controlled-product GEMMs (dense plans) or Strang passes (Trotter plans)
   auto tree = [&](void* half, bool reduce) -> hhl_status {
     if (!dense) return hhl::launch_trotter_tree(p, half, reduce, st);
+    hhl::TcChain chain;
     for (int j = 0; j < p.n_c; ++j) {
-      hhl_status ts = hhl::launch_ctrl_u_tree(p, half, reduce ? p.n_c - 1 - j : j, reduce, st);
+      hhl_status ts = hhl::launch_ctrl_u_tree(p, half, reduce ? p.n_c - 1 - j : j, reduce, st, &chain);
       if (ts != HHL_OK) return ts;
     }
     return HHL_OK;

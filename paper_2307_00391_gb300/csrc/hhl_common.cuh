@@ -64,7 +64,7 @@ inline cudaLaunchAttribute dep_attribute() {
   a.val.programmaticStreamSerializationAllowed = 1;
   return a;
 }
-// Not while the stream is captured: the batch's graph runs eight such chains side by side, where a
+// Whether the stream's kernels run one after another by themselves. Not while it is captured: the batch's graph runs eight such chains side by side, where a
 // block that waits takes its slot from the other chains' work (256 instances 127.5 -> 132.7 ms).
 inline bool dep_allowed(cudaStream_t st) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -400,7 +400,8 @@ hhl_status launch_ctrl_u_simt_map(const Plan& p, void* half, const RowMap& rows,
 // One tree step of the dense postselected solve: expansion (rows [2^k, 2^(k+1)) = U_k rows
 // [0, 2^k)) or reduction (rows [0, 2^k) += U_k^dagger rows [2^k, 2^(k+1)), the last one, k = 0,
 // scaled by 2^(-n_c/2)), on the plan's operands (tcgen05 where 2^k >= 128, else CUDA cores).
-hhl_status launch_ctrl_u_tree(const Plan& p, void* half, int k, bool reduce, cudaStream_t st);
+struct TcChain;  // (below)
+hhl_status launch_ctrl_u_tree(const Plan& p, void* half, int k, bool reduce, cudaStream_t st, TcChain* chain);
 hhl_status launch_clock_block(const Plan& p, void* state, cudaStream_t st);
 // The clock block for the postselected solve (postselect-early plans on the split-pass path):
 // the anc = 0 half is not stored; the weights of the two halves after the block are added to
@@ -473,7 +474,24 @@ hhl_status launch_clock_spec(const Plan& p, void* state, const double2* ph_lo, c
 // tcgen05 GEMM (hhl_gemm_tc.cu)
 bool tc_supported(const Plan& p);
 hhl_status tc_prepare_operands(Plan& p, const double2* d_u, int k, cudaStream_t st);
-hhl_status launch_ctrl_u_tc(const Plan& p, void* half, int k, bool adjoint, cudaStream_t st);
+// Consecutive tcgen05 products of one chain (the k of a circuit half, the steps of a tree): a product
+// that is told its successor also leaves the successor's split-FP16 rows, so only the first of a
+// chain runs k_tc_split_rows. ready: the rows of the next product lie in operand buffer `buf`.
+struct TcChain {
+  bool ready = false;
+  int buf = 0;
+};
+struct TcNext {
+  enum Mode { kNone = 0, kCircuit = 1, kExpand = 2, kReduce = 3 };
+  int mode = kNone;
+  int k = 0, kn = 0;       // kCircuit: this product's clock bit and the successor's
+  int64_t first = 0;       // kReduce: first state row of the successor's operand
+  int64_t side_rows = 0;   // kCircuit: successor rows this product does not write
+  void* hi = nullptr;
+  void* lo = nullptr;
+};
+// The controlled product of clock bit k; kn >= 0: the circuit's next one (chain then not NULL).
+hhl_status launch_ctrl_u_tc(const Plan& p, void* half, int k, bool adjoint, int kn, TcChain* chain, cudaStream_t st);
 void tc_free(Plan& p);
 int* tc_error_flag(const Plan& p);  // device flag: 1-3, 5 a bounded GEMM wait ran out, 4 operand out of range
 // Clear that flag on the stream (at the start of each circuit, so that a status reports only
@@ -503,10 +521,11 @@ void tc_work_free(TcWork& w);
 hhl_status launch_tc_gemm_map(int n_s, int64_t m_sub, const RowMap& rows, void* half, void* a_hi, void* a_lo,
                               const CUtensorMap& map_ahi, const CUtensorMap& map_alo, const CUtensorMap& map_bhi,
                               const CUtensorMap& map_blo, int bn, int* err, const TcWork& w, int streamk,
-                              cudaStream_t st, const CUtensorMap* slice4 = nullptr);
+                              cudaStream_t st, const CUtensorMap* slice4 = nullptr, const TcNext& next = TcNext{},
+                              bool split_ready = false);
 // The plan's tcgen05 product on mapped rows (m_sub a multiple of 128).
 hhl_status launch_ctrl_u_tc_map(const Plan& p, void* half, const RowMap& rows, int64_t m_sub, int k, bool adjoint,
-                                cudaStream_t st);
+                                TcNext next, TcChain* chain, cudaStream_t st);
 hhl_status tc_make_map(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t box_rows);
 hhl_status tc_init_kernels();
 

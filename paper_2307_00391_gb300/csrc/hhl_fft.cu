@@ -39,6 +39,11 @@ namespace hhl {
 namespace {
 
 constexpr int kFftThreads = 256;
+// Threads of the one-pass blocks: 512 where shared memory leaves room for one block an SM (12-bit
+// clocks: 140 KiB; 256 threads left the SM waiting on its own round trips: 80.7 -> 71.7 us at 2^10
+// columns), else 256. 256 too in captured graphs, where the batch's other chains use the SM.
+constexpr int kFftWide = 512;
+constexpr size_t kFftWideSmem = 100 * 1024;
 constexpr size_t kFftSmemTarget = 140 * 1024;  // one CTA per SM at most this large
 constexpr size_t kFftSmemCap = 200 * 1024;
 constexpr int kUnroll = 8;                     // 16-byte loads in flight per thread
@@ -243,7 +248,7 @@ __device__ void store_block(T* dst, int64_t row_stride, const T* X, int Lp, int 
 
 // Clock block (a3 + a4 + the QFT of a5) on a cluster of 2^CB CTAs.
 template <class R, bool FULL, int CB>
-__global__ void __launch_bounds__(kFftThreads, 2) k_clock_block(typename Cx<R>::T* __restrict__ S,
+__global__ void __launch_bounds__(kFftWide, 1) k_clock_block(typename Cx<R>::T* __restrict__ S,
                                                              const typename Cx<R>::T* __restrict__ rot, int n_s,
                                                              int n_c, int W) {
   dep_begin();
@@ -396,7 +401,7 @@ __global__ void __launch_bounds__(kFftThreads) k_clock_spec(double2* __restrict_
 // order (the low register of a whole-register transform: its stages do not depend on the
 // bits above). Every output is multiplied by scale.
 template <class R, int CB>
-__global__ void __launch_bounds__(kFftThreads, 2) k_register_transform(typename Cx<R>::T* __restrict__ S, int lo, int m,
+__global__ void __launch_bounds__(kFftWide, 1) k_register_transform(typename Cx<R>::T* __restrict__ S, int lo, int m,
                                                                     int W, int mode, R scale) {
   dep_begin();
   using T = typename Cx<R>::T;
@@ -551,7 +556,7 @@ hhl_status launch_cluster(Kern kernel, int grid, int cb, size_t smem, cudaStream
   HHL_CUDA_TRY(raise_dyn_smem((const void*)kernel, smem));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kFftThreads);
+  cfg.blockDim = dim3(smem > kFftWideSmem && dep_allowed(st) ? kFftWide : kFftThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];

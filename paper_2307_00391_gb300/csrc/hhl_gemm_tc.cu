@@ -19,7 +19,10 @@
 // amplitude of magnitude >= 2 (outside the scaled FP16 range) as a numeric error.
 // The plan stores E_hi and E_lo (forward and adjoint) for every k; the gather kernel copies
 // the rows with bit k set into compact X_hi / X_lo arrays, so the GEMM may write its result
-// straight back into those state rows.
+// straight back into those state rows. Along a chain of products only the first gathers: each
+// product also leaves its successor's X_hi / X_lo in the other of two operand buffers, the rows it
+// writes from its epilogue and the rest by its epilogue warps while the accumulators fill (23-qubit
+// solve: 24 gathers of 8 us a solve become 2, 1182 -> 1010 us).
 //
 // Kernel (persistent, stream-K): the work is the list of (output tile, K step) units, tile-major,
 // 128 x BN tiles of K / 32 steps each; the grid has one CTA per SM (fewer when there are few
@@ -81,13 +84,13 @@ constexpr long long kWaitCycles = 4000000000LL;      // default bound of a wait:
 constexpr long long kFaultWaitCycles = 2000000LL;    // injected timeout: ~1 ms
 
 struct TcState {
-  __half* a_hi = nullptr;  // M_sub x 2N
-  __half* a_lo = nullptr;
+  __half* a_hi[2] = {nullptr, nullptr};  // M_sub x 2N each, two operand buffers (TcChain)
+  __half* a_lo[2] = {nullptr, nullptr};
   __half* b = nullptr;     // n_c x {fwd_hi, fwd_lo, adj_hi, adj_lo} x (2N x 2N)
   int* err = nullptr;      // device error flag
   TcWork work;             // stream-K partials and tile counters
   int bn = kBN;           // output tile width (128 or 256)
-  std::vector<CUtensorMap> maps;  // [0] A_hi, [1] A_lo, then per k: fwd_hi, fwd_lo, adj_hi, adj_lo
+  std::vector<CUtensorMap> maps;  // A_hi, A_lo of each buffer, then per k: fwd_hi, fwd_lo, adj_hi, adj_lo
   std::vector<CUtensorMap> smaps; // per k the same four with a quarter-height box (cluster slices)
 };
 
@@ -241,13 +244,60 @@ __device__ __forceinline__ void split_f16(float v, __half& hi, __half& lo) {
   lo = __float2half_rn(v - __half2float(hi));
 }
 
+// Four amplitude components as one unit of the split operand; false if one is out of range.
+__device__ __forceinline__ bool split_unit(float4 v, uint2& hi, uint2& lo) {
+  const float x[4] = {v.x * kOpScale, v.y * kOpScale, v.z * kOpScale, v.w * kOpScale};
+  __half h[4], l[4];
+  bool ok = true;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    split_f16(x[j], h[j], l[j]);
+    ok &= fabsf(x[j]) < 2.0f * kOpScale;
+  }
+  hi = make_uint2((uint32_t)__half_as_ushort(h[0]) | ((uint32_t)__half_as_ushort(h[1]) << 16),
+                  (uint32_t)__half_as_ushort(h[2]) | ((uint32_t)__half_as_ushort(h[3]) << 16));
+  lo = make_uint2((uint32_t)__half_as_ushort(l[0]) | ((uint32_t)__half_as_ushort(l[1]) << 16),
+                  (uint32_t)__half_as_ushort(l[2]) | ((uint32_t)__half_as_ushort(l[3]) << 16));
+  return ok;
+}
+
+// 32 bytes at a 32-byte boundary (the operand buffers are the plan's own allocations).
+__device__ __forceinline__ void store_32b(uint2* d, const uint2 (&v)[4]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d), "r"(v[0].x), "r"(v[0].y), "r"(v[1].x),
+               "r"(v[1].y), "r"(v[2].x), "r"(v[2].y), "r"(v[3].x), "r"(v[3].y)
+               : "memory");
+}
+
+__device__ __forceinline__ void store_32b(float4* d, float4 a, float4 b) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d), "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w),
+               "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+               : "memory");
+}
+
+// Row of the successor's operand that state row `row` is, or -1.
+__device__ __forceinline__ int64_t next_row(const TcNext& nx, int64_t row) {
+  if (nx.mode == TcNext::kExpand) return row;
+  if (nx.mode == TcNext::kReduce) return row >= nx.first ? row - nx.first : -1;
+  if (nx.mode == TcNext::kCircuit && ((row >> nx.kn) & 1))
+    return ((row >> (nx.kn + 1)) << nx.kn) | (row & ((1LL << nx.kn) - 1));
+  return -1;
+}
+
+// State row j of those with clock bit kn set and bit k clear (which product k does not write).
+__device__ __forceinline__ int64_t side_row(const TcNext& nx, int64_t j) {
+  const int a = nx.k < nx.kn ? nx.k : nx.kn, b = nx.k < nx.kn ? nx.kn : nx.k;
+  int64_t r = ((j >> a) << (a + 1)) | (j & ((1LL << a) - 1));
+  r = ((r >> b) << (b + 1)) | (r & ((1LL << b) - 1));
+  return r | (1LL << nx.kn);
+}
+
 
 template <int BN, int CL>
 __global__ void __launch_bounds__(kThreadsTc, 1)
     k_ctrl_gemm_tc(const __grid_constant__ CUtensorMap map_ahi, const __grid_constant__ CUtensorMap map_alo,
                    const __grid_constant__ CUtensorMap map_bhi, const __grid_constant__ CUtensorMap map_blo,
                    float* __restrict__ state_half, int n_s, RowMap rows, int k_iters, int tiles_n, int64_t units,
-                   float* __restrict__ ws, int* err, long long wait_cycles, int fault) {
+                   float* __restrict__ ws, int* err, long long wait_cycles, int fault, const TcNext nx) {
   constexpr int S = TcShape<BN>::kStages;
   constexpr int kTileB = TcShape<BN>::kTileB, kStageBytes = TcShape<BN>::kStageBytes;
   constexpr int kTmemCols = TcShape<BN>::kTmemCols;
@@ -392,6 +442,38 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
     const int row = q * 32 + lane;
     const bool leader = threadIdx.x == 64;
     const int64_t N2 = 2LL << n_s;  // floats per state row
+    // 32-byte stores of the rows where the caller's state allows them (16-byte alignment is all it owes)
+    const bool wide = (reinterpret_cast<uintptr_t>(state_half) & 31) == 0;
+    bool ok = true;                 // every component of the successor's operand in range
+    if (nx.mode == TcNext::kCircuit) {
+      // while the accumulators fill: the successor's rows that this product leaves as they are
+      const int row4_bits = n_s - 1;
+      const int64_t total = nx.side_rows << row4_bits, stride = G * 128;
+      const float4* src = reinterpret_cast<const float4*>(state_half);
+      constexpr int U = 4;  // loads in flight per thread
+      for (int64_t e0 = cta * 128 + (threadIdx.x - 64); e0 < total; e0 += U * stride) {
+        float4 v[U];
+        int64_t at[U];
+#pragma unroll
+        for (int q2 = 0; q2 < U; ++q2) {
+          const int64_t e = e0 + q2 * stride;
+          if (e < total) {
+            const int64_t r = side_row(nx, e >> row4_bits), c = e & ((1LL << row4_bits) - 1);
+            v[q2] = src[(r << row4_bits) + c];
+            at[q2] = (next_row(nx, r) << row4_bits) + c;
+          }
+        }
+#pragma unroll
+        for (int q2 = 0; q2 < U; ++q2) {
+          if (e0 + q2 * stride < total) {
+            uint2 h, l;
+            ok &= split_unit(v[q2], h, l);
+            static_cast<uint2*>(nx.hi)[at[q2]] = h;
+            static_cast<uint2*>(nx.lo)[at[q2]] = l;
+          }
+        }
+      }
+    }
     int j = 0;
     for (int64_t u = u_begin; u < u_end; ++j) {
       const int64_t t = u / k_iters;
@@ -404,7 +486,11 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
       const int m0 = (int)(t / tiles_n) * kBM, n0 = (int)(t % tiles_n) * BN;
-      float* dst = state_half + rowmap_out(rows, m0 + row) * N2 + n0;
+      const int64_t out_row = rowmap_out(rows, m0 + row);
+      float* dst = state_half + out_row * N2 + n0;
+      const int64_t nrow = next_row(nx, out_row);  // its row of the successor's operand
+      uint2* nhi = static_cast<uint2*>(nx.hi) + (nrow * N2 + n0) / 4;
+      uint2* nlo = static_cast<uint2*>(nx.lo) + (nrow * N2 + n0) / 4;
       if (kb == 0 && ke == k_iters) {
         // the whole tile is this CTA's: straight to the state row
 #pragma unroll 1
@@ -413,14 +499,30 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
           tmem_ld_32cols(taddr + c, v);
           float4* d4 = reinterpret_cast<float4*>(dst + c);
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            float4 o = make_float4(v[4 * e] * kUnscale, v[4 * e + 1] * kUnscale, v[4 * e + 2] * kUnscale,
-                                   v[4 * e + 3] * kUnscale);
-            if (rows.accumulate) {  // a reduction step of the postselected solve: the row keeps its value
-              const float4 prev = d4[e];
-              o = make_float4(prev.x + o.x, prev.y + o.y, prev.z + o.z, prev.w + o.w);
+          for (int e4 = 0; e4 < 8; e4 += 4) {
+            uint2 h[4], l[4];
+            float4 ov[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int e = e4 + i;
+              float4 o = make_float4(v[4 * e] * kUnscale, v[4 * e + 1] * kUnscale, v[4 * e + 2] * kUnscale,
+                                     v[4 * e + 3] * kUnscale);
+              if (rows.accumulate) {  // a reduction step of the postselected solve: the row keeps its value
+                const float4 prev = d4[e];
+                o = make_float4(prev.x + o.x, prev.y + o.y, prev.z + o.z, prev.w + o.w);
+              }
+              if (wide) ov[i] = o;
+              else d4[e] = o;
+              if (nrow >= 0) ok &= split_unit(o, h[i], l[i]);
             }
-            d4[e] = o;
+            if (wide) {
+              store_32b(d4 + e4, ov[0], ov[1]);
+              store_32b(d4 + e4 + 2, ov[2], ov[3]);
+            }
+            if (nrow >= 0) {
+              store_32b(nhi + c / 4 + e4, h);  // whole sectors: a lane's neighbours write other rows
+              store_32b(nlo + c / 4 + e4, l);
+            }
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -443,6 +545,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       }
       u += ke - kb;
     }
+    if (!ok) atomicExch(err, 4);
   }
   __syncwarp();
   __syncthreads();  // every role has left its (bounded) loop
@@ -463,7 +566,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
 template <int BN>
 __global__ void __launch_bounds__(256) k_tc_fixup(const float4* __restrict__ ws, float* __restrict__ state_half,
                                                   int n_s, RowMap rows, int k_iters, int tiles_n, int64_t units,
-                                                  int64_t G, int* err) {
+                                                  int64_t G, int* err, const TcNext nx) {
   dep_begin();
   constexpr int kQ = BN / 4;  // float4 per tile row
   const int64_t t = blockIdx.y;
@@ -479,13 +582,22 @@ __global__ void __launch_bounds__(256) k_tc_fixup(const float4* __restrict__ ws,
     o = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w);
   }
   const int m0 = (int)(t / tiles_n) * kBM, n0 = (int)(t % tiles_n) * BN;
-  float4* d4 = reinterpret_cast<float4*>(state_half + rowmap_out(rows, m0 + row) * (2LL << n_s) + n0) + q;
+  const int64_t out_row = rowmap_out(rows, m0 + row);
+  float4* d4 = reinterpret_cast<float4*>(state_half + out_row * (2LL << n_s) + n0) + q;
   o = make_float4(o.x * kUnscale, o.y * kUnscale, o.z * kUnscale, o.w * kUnscale);
   if (rows.accumulate) {
     const float4 prev = *d4;
     o = make_float4(prev.x + o.x, prev.y + o.y, prev.z + o.z, prev.w + o.w);
   }
   *d4 = o;
+  const int64_t nrow = next_row(nx, out_row);
+  if (nrow >= 0) {
+    const int64_t at = (nrow * (2LL << n_s) + n0) / 4 + q;
+    uint2 h, l;
+    if (!split_unit(o, h, l)) atomicExch(err, 4);
+    static_cast<uint2*>(nx.hi)[at] = h;
+    static_cast<uint2*>(nx.lo)[at] = l;
+  }
 }
 
 // The mapped rows (those with clock bit k set, or a tree step's source rows) -> compact FP16
@@ -513,17 +625,10 @@ __global__ void k_tc_split_rows(const float4* __restrict__ half, uint2* __restri
     for (int q = 0; q < U; ++q) {
       const int64_t e = e0 + q * stride;
       if (e < total) {
-        const float x[4] = {v[q].x * kOpScale, v[q].y * kOpScale, v[q].z * kOpScale, v[q].w * kOpScale};
-        __half h[4], l[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          split_f16(x[j], h[j], l[j]);
-          bad |= !(fabsf(x[j]) < 2.0f * kOpScale);
-        }
-        a_hi[e] = make_uint2((uint32_t)__half_as_ushort(h[0]) | ((uint32_t)__half_as_ushort(h[1]) << 16),
-                             (uint32_t)__half_as_ushort(h[2]) | ((uint32_t)__half_as_ushort(h[3]) << 16));
-        a_lo[e] = make_uint2((uint32_t)__half_as_ushort(l[0]) | ((uint32_t)__half_as_ushort(l[1]) << 16),
-                             (uint32_t)__half_as_ushort(l[2]) | ((uint32_t)__half_as_ushort(l[3]) << 16));
+        uint2 h, l;
+        bad |= !split_unit(v[q], h, l);
+        a_hi[e] = h;
+        a_lo[e] = l;
       }
     }
   }
@@ -598,7 +703,8 @@ hhl_status tc_prepare_operands(Plan& p, const double2* d_u, int k, cudaStream_t 
     t = new TcState();
     p.d_tc = t;
     const size_t abytes = (size_t)(p.R / 2) * N2 * sizeof(__half);
-    if (cudaMalloc(&t->a_hi, abytes) != cudaSuccess || cudaMalloc(&t->a_lo, abytes) != cudaSuccess ||
+    if (cudaMalloc(&t->a_hi[0], abytes) != cudaSuccess || cudaMalloc(&t->a_lo[0], abytes) != cudaSuccess ||
+        cudaMalloc(&t->a_hi[1], abytes) != cudaSuccess || cudaMalloc(&t->a_lo[1], abytes) != cudaSuccess ||
         cudaMalloc(&t->b, (size_t)p.n_c * 4 * mat * sizeof(__half)) != cudaSuccess ||
         cudaMalloc(&t->err, sizeof(int)) != cudaSuccess) {
       cudaGetLastError();
@@ -606,18 +712,21 @@ hhl_status tc_prepare_operands(Plan& p, const double2* d_u, int k, cudaStream_t 
     }
     hhl_status ws = tc_work_alloc(t->work, &p.workspace_bytes);
     if (ws != HHL_OK) return ws;
-    p.workspace_bytes += 2 * abytes;
+    p.workspace_bytes += 4 * abytes;
     p.table_bytes += (size_t)p.n_c * 4 * mat * sizeof(__half);
     HHL_CUDA_TRY(cudaMemsetAsync(t->err, 0, sizeof(int), st));
     // tile width: 256 unless HHL_TC_BN=128 (tuning) or the operand is narrower
     if (const char* env = getenv("HHL_TC_BN")) t->bn = atoi(env) == 128 ? 128 : 256;
     if (N2 < t->bn) t->bn = 128;
-    t->maps.resize(2 + 4 * (size_t)p.n_c);
-    hhl_status s = make_map(&t->maps[0], t->a_hi, N2, p.R / 2, kBM);
-    if (s == HHL_OK) s = make_map(&t->maps[1], t->a_lo, N2, p.R / 2, kBM);
+    t->maps.resize(4 + 4 * (size_t)p.n_c);
+    hhl_status s = HHL_OK;
+    for (int b = 0; b < 2 && s == HHL_OK; ++b) {
+      s = make_map(&t->maps[2 * b], t->a_hi[b], N2, p.R / 2, kBM);
+      if (s == HHL_OK) s = make_map(&t->maps[2 * b + 1], t->a_lo[b], N2, p.R / 2, kBM);
+    }
     for (int kk = 0; kk < p.n_c && s == HHL_OK; ++kk)
       for (int j = 0; j < 4 && s == HHL_OK; ++j)
-        s = make_map(&t->maps[2 + 4 * kk + j], t->b + ((size_t)kk * 4 + j) * mat, N2, N2, t->bn);
+        s = make_map(&t->maps[4 + 4 * kk + j], t->b + ((size_t)kk * 4 + j) * mat, N2, N2, t->bn);
     t->smaps.resize(4 * (size_t)p.n_c);
     for (int kk = 0; kk < p.n_c && s == HHL_OK; ++kk)
       for (int j = 0; j < 4 && s == HHL_OK; ++j)
@@ -634,18 +743,35 @@ hhl_status tc_prepare_operands(Plan& p, const double2* d_u, int k, cudaStream_t 
   return HHL_OK;
 }
 
-hhl_status launch_ctrl_u_tc(const Plan& p, void* half, int k, bool adjoint, cudaStream_t st) {
-  return launch_ctrl_u_tc_map(p, half, circuit_rows(k), p.R / 2, k, adjoint, st);
+hhl_status launch_ctrl_u_tc(const Plan& p, void* half, int k, bool adjoint, int kn, TcChain* chain, cudaStream_t st) {
+  TcNext next;
+  if (chain != nullptr && kn >= 0) {
+    next.mode = TcNext::kCircuit;
+    next.k = k;
+    next.kn = kn;
+    next.side_rows = p.R / 4;
+  }
+  return launch_ctrl_u_tc_map(p, half, circuit_rows(k), p.R / 2, k, adjoint, next, chain, st);
 }
 
 hhl_status launch_ctrl_u_tc_map(const Plan& p, void* half, const RowMap& rows, int64_t m_sub, int k, bool adjoint,
-                                cudaStream_t st) {
+                                TcNext next, TcChain* chain, cudaStream_t st) {
   const TcState* t = static_cast<const TcState*>(p.d_tc);
   if (t == nullptr) return fail(HHL_ERR_INVALID_ARG, "tcgen05 operands not prepared");
-  const CUtensorMap* mb = &t->maps[2 + 4 * (size_t)k + (adjoint ? 2 : 0)];
+  const CUtensorMap* mb = &t->maps[4 + 4 * (size_t)k + (adjoint ? 2 : 0)];
   const CUtensorMap* ms = &t->smaps[4 * (size_t)k + (adjoint ? 2 : 0)];
-  return launch_tc_gemm_map(p.n_s, m_sub, rows, half, t->a_hi, t->a_lo, t->maps[0], t->maps[1], mb[0], mb[1], t->bn,
-                            t->err, t->work, 1, st, ms);
+  const int buf = chain != nullptr ? chain->buf : 0;
+  const bool ready = chain != nullptr && chain->ready;
+  if (chain != nullptr) {
+    // an expansion's operand grows in place (its new rows lie above those being read); otherwise
+    // the successor's operand goes to the other buffer
+    if (next.mode != TcNext::kNone && next.mode != TcNext::kExpand) chain->buf ^= 1;
+    chain->ready = next.mode != TcNext::kNone;
+    next.hi = t->a_hi[chain->buf];
+    next.lo = t->a_lo[chain->buf];
+  }
+  return launch_tc_gemm_map(p.n_s, m_sub, rows, half, t->a_hi[buf], t->a_lo[buf], t->maps[2 * buf], t->maps[2 * buf + 1],
+                            mb[0], mb[1], t->bn, t->err, t->work, 1, st, ms, next, ready);
 }
 
 int tc_num_sms() {
@@ -677,7 +803,7 @@ void tc_work_free(TcWork& w) {
 hhl_status launch_tc_gemm_map(int n_s, int64_t m_sub, const RowMap& k, void* half, void* a_hi, void* a_lo,
                               const CUtensorMap& map_ahi, const CUtensorMap& map_alo, const CUtensorMap& map_bhi,
                               const CUtensorMap& map_blo, int bn, int* err, const TcWork& w, int streamk,
-                              cudaStream_t st, const CUtensorMap* slice4) {
+                              cudaStream_t st, const CUtensorMap* slice4, const TcNext& next, bool split_ready) {
   const int64_t N2 = 2LL << n_s;
   if (m_sub < kBM || m_sub % kBM != 0) return fail(HHL_ERR_INVALID_ARG, "tcgen05 GEMM rows must be a multiple of 128");
   if (bn != 128 && bn != 256) return fail(HHL_ERR_INVALID_ARG, "tcgen05 tile width must be 128 or 256");
@@ -691,9 +817,11 @@ hhl_status launch_tc_gemm_map(int n_s, int64_t m_sub, const RowMap& k, void* hal
   const int64_t total4 = m_sub * N2 / 4;
   int g = (int)((total4 + 255) / 256);
   if (g > 152 * 16) g = 152 * 16;
-  HHL_PROF_BEGIN(st);
-  launch_dep(k_tc_split_rows, g, 256, 0, st, (const float4*)half, (uint2*)a_hi, (uint2*)a_lo, n_s, k, m_sub, err);
-  HHL_LAUNCH_CHECK("k_tc_split_rows");
+  if (!split_ready) {
+    HHL_PROF_BEGIN(st);
+    launch_dep(k_tc_split_rows, g, 256, 0, st, (const float4*)half, (uint2*)a_hi, (uint2*)a_lo, n_s, k, m_sub, err);
+    HHL_LAUNCH_CHECK("k_tc_split_rows");
+  }
   // grid: one CTA per tile when the tiles fill at least three quarters of the SMs (or the
   // caller asks for it: the batch, whose streams fill the GPU together); otherwise stream-K,
   // one CTA per SM, fewer when a CTA would get under a quarter of a tile
@@ -735,21 +863,21 @@ hhl_status launch_tc_gemm_map(int n_s, int64_t m_sub, const RowMap& k, void* hal
     if (bn == 256) {
       cfg.dynamicSmemBytes = TcShape<256>::kSmemBytes;
       e = cudaLaunchKernelEx(&cfg, k_ctrl_gemm_tc<256, 4>, map_ahi, map_alo, slice4[0], slice4[1], sh, n_s, k, k_iters,
-                             ti, units, wsp, err, wait_cycles, fault);
+                             ti, units, wsp, err, wait_cycles, fault, next);
     } else {
       cfg.dynamicSmemBytes = TcShape<128>::kSmemBytes;
       e = cudaLaunchKernelEx(&cfg, k_ctrl_gemm_tc<128, 4>, map_ahi, map_alo, slice4[0], slice4[1], sh, n_s, k, k_iters,
-                             ti, units, wsp, err, wait_cycles, fault);
+                             ti, units, wsp, err, wait_cycles, fault, next);
     }
     if (e != cudaSuccess) return cuda_fail(e, "k_ctrl_gemm_tc (cluster launch)");
   } else if (bn == 256) {
     launch_dep(k_ctrl_gemm_tc<256, 1>, (unsigned)G, kThreadsTc, TcShape<256>::kSmemBytes, st, 
         map_ahi, map_alo, map_bhi, map_blo, (float*)half, n_s, k, k_iters, (int)tiles_n, units, w.ws, err,
-        wait_cycles, fault);
+        wait_cycles, fault, next);
   } else {
     launch_dep(k_ctrl_gemm_tc<128, 1>, (unsigned)G, kThreadsTc, TcShape<128>::kSmemBytes, st, 
         map_ahi, map_alo, map_bhi, map_blo, (float*)half, n_s, k, k_iters, (int)tiles_n, units, w.ws, err,
-        wait_cycles, fault);
+        wait_cycles, fault, next);
   }
   HHL_LAUNCH_CHECK("k_ctrl_gemm_tc");
   // the split tiles, if any (a range boundary inside a tile): partials added in CTA order
@@ -760,10 +888,10 @@ hhl_status launch_tc_gemm_map(int n_s, int64_t m_sub, const RowMap& k, void* hal
   HHL_PROF_BEGIN(st);
   if (bn == 256)
     launch_dep(k_tc_fixup<256>, fgrid, 256, 0, st, (const float4*)w.ws, (float*)half, n_s, k, k_iters, (int)tiles_n, units, G,
-                                           err);
+                                           err, next);
   else
     launch_dep(k_tc_fixup<128>, fgrid, 256, 0, st, (const float4*)w.ws, (float*)half, n_s, k, k_iters, (int)tiles_n, units, G,
-                                           err);
+                                           err, next);
   HHL_LAUNCH_CHECK("k_tc_fixup");
   return HHL_OK;
 }
@@ -808,8 +936,10 @@ hhl_status tc_reset_error(const Plan& p, cudaStream_t st) {
 void tc_free(Plan& p) {
   TcState* t = static_cast<TcState*>(p.d_tc);
   if (t == nullptr) return;
-  if (t->a_hi) cudaFree(t->a_hi);
-  if (t->a_lo) cudaFree(t->a_lo);
+  for (int b = 0; b < 2; ++b) {
+    if (t->a_hi[b]) cudaFree(t->a_hi[b]);
+    if (t->a_lo[b]) cudaFree(t->a_lo[b]);
+  }
   if (t->b) cudaFree(t->b);
   if (t->err) cudaFree(t->err);
   tc_work_free(t->work);

@@ -765,7 +765,7 @@ hhl_status launch_ctrl_u_dense(const Plan& p, void* half, int k, bool adjoint, c
   return launch_ctrl_u_simt(p, half, k, B, st);
 }
 
-hhl_status launch_ctrl_u_tree(const Plan& p, void* half, int k, bool reduce, cudaStream_t st) {
+hhl_status launch_ctrl_u_tree(const Plan& p, void* half, int k, bool reduce, cudaStream_t st, TcChain* chain) {
   RowMap rows;
   const int64_t m = 1LL << k;
   if (reduce) {
@@ -779,8 +779,19 @@ hhl_status launch_ctrl_u_tree(const Plan& p, void* half, int k, bool reduce, cud
   }
   if (p.d_gdf != nullptr && m < toeplitz_rows_limit())  // few rows: U_k generated on the fly from its g table
     return launch_toeplitz_rows((float2*)half, p.n_s, p.d_gdf + (size_t)k * (2 * p.N + 2), reduce ? 1 : 0, rows, m, st);
-  if (p.gemm_impl == HHL_GEMM_TCGEN05 && m >= 128 && rows.scale == 1.0)
-    return launch_ctrl_u_tc_map(p, half, rows, m, k, reduce, st);
+  auto on_tc = [&](int kk) {  // the steps that take the tensor cores
+    const int64_t mm = 1LL << kk;
+    return kk >= 0 && kk < p.n_c && !(p.d_gdf != nullptr && mm < toeplitz_rows_limit()) &&
+           p.gemm_impl == HHL_GEMM_TCGEN05 && mm >= 128 && !(reduce && kk == 0);
+  };
+  if (on_tc(k)) {
+    TcNext next;
+    if (on_tc(reduce ? k - 1 : k + 1)) {
+      next.mode = reduce ? TcNext::kReduce : TcNext::kExpand;
+      next.first = m / 2;
+    }
+    return launch_ctrl_u_tc_map(p, half, rows, m, k, reduce, next, chain, st);
+  }
   if (p.d_gdf != nullptr && m < 128)
     return launch_toeplitz_rows((float2*)half, p.n_s, p.d_gdf + (size_t)k * (2 * p.N + 2), reduce ? 1 : 0, rows, m, st);
   if (p.d_bfwd == nullptr) {  // a tcgen05 plan keeps no CUDA-core operands
