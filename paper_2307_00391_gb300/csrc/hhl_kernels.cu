@@ -127,8 +127,10 @@ __global__ void __launch_bounds__(kThreads) k_prep_small(const double2* __restri
 // ------------------------------------------------------------------------------ SIMT GEMM
 // out[i][n] = sum_m S[row(i)][m] * B[m][n] for the M_sub = 2^(n_c-1) rows with clock bit k
 // set; B = U_k^T (forward) or conj(U_k) (adjoint) so that out row = U row.
-template <class R, int BM, int BN, int BK>
-__global__ void __launch_bounds__(256) k_ctrl_gemm_simt(const typename Cx<R>::T* __restrict__ S,
+// INPLACE (N <= BN: a block holds whole rows, and no other block reads them): the results go
+// straight to the mapped state rows, as k_rows_scatter would copy, add or scale them.
+template <class R, int BM, int BN, int BK, bool INPLACE>
+__global__ void __launch_bounds__(256) k_ctrl_gemm_simt(typename Cx<R>::T* S,
                                                         typename Cx<R>::T* __restrict__ out,
                                                         const typename Cx<R>::T* __restrict__ B,
                                                         int n_s, RowMap rows, int64_t m_sub) {
@@ -188,7 +190,18 @@ __global__ void __launch_bounds__(256) k_ctrl_gemm_simt(const typename Cx<R>::T*
 #pragma unroll
     for (int y = 0; y < TN; ++y) {
       const int64_t n = n0 + tx + 16 * y;
-      if (n < N) out[i * N + n] = mk<R>(accr[x][y], acci[x][y]);
+      if (n >= N) continue;
+      if constexpr (INPLACE) {  // (rows read by this block only, all of them by the last barrier above;
+        T* d = S + rowmap_out(rows, i) * N + n;  // a tree step's output rows are not read at all)
+        T v = mk<R>(accr[x][y], acci[x][y]);
+        if (rows.accumulate) {
+          v = cadd(*d, v);
+          if (rows.scale != 1.0) v = cscale(v, (R)rows.scale);
+        }
+        *d = v;
+      } else {
+        out[i * N + n] = mk<R>(accr[x][y], acci[x][y]);
+      }
     }
   }
 }
@@ -811,21 +824,20 @@ hhl_status launch_ctrl_u_simt_map(const Plan& p, void* half, const RowMap& k, in
   const int64_t N = p.N;
   dim3 grid((unsigned)((N + 63) / 64), (unsigned)((m_sub + 63) / 64));
   const int sg = grid_for(m_sub * N, kThreads, 152 * 32);
-  if (p.prec == HHL_PREC_C64) {
-    HHL_PROF_BEGIN(st);
-    launch_dep(k_ctrl_gemm_simt<float, 64, 64, 16>, grid, 256, 0, st, (const float2*)half, (float2*)p.d_scratch,
-                                                              (const float2*)B, p.n_s, k, m_sub);
-    HHL_LAUNCH_CHECK("k_ctrl_gemm_simt<f32>");
-    HHL_PROF_BEGIN(st);
-    launch_dep(k_rows_scatter<float>, sg, kThreads, 0, st, (float2*)half, (const float2*)p.d_scratch, p.n_s, k, m_sub);
+  const bool c64 = p.prec == HHL_PREC_C64, in_place = N <= 64;
+  HHL_PROF_BEGIN(st);
+  if (c64) {
+    auto kern = in_place ? k_ctrl_gemm_simt<float, 64, 64, 16, true> : k_ctrl_gemm_simt<float, 64, 64, 16, false>;
+    launch_dep(kern, grid, 256, 0, st, (float2*)half, (float2*)p.d_scratch, (const float2*)B, p.n_s, k, m_sub);
   } else {
-    HHL_PROF_BEGIN(st);
-    launch_dep(k_ctrl_gemm_simt<double, 64, 64, 8>, grid, 256, 0, st, (const double2*)half, (double2*)p.d_scratch,
-                                                              (const double2*)B, p.n_s, k, m_sub);
-    HHL_LAUNCH_CHECK("k_ctrl_gemm_simt<f64>");
-    HHL_PROF_BEGIN(st);
-    launch_dep(k_rows_scatter<double>, sg, kThreads, 0, st, (double2*)half, (const double2*)p.d_scratch, p.n_s, k, m_sub);
+    auto kern = in_place ? k_ctrl_gemm_simt<double, 64, 64, 8, true> : k_ctrl_gemm_simt<double, 64, 64, 8, false>;
+    launch_dep(kern, grid, 256, 0, st, (double2*)half, (double2*)p.d_scratch, (const double2*)B, p.n_s, k, m_sub);
   }
+  HHL_LAUNCH_CHECK(c64 ? "k_ctrl_gemm_simt<f32>" : "k_ctrl_gemm_simt<f64>");
+  if (in_place) return HHL_OK;
+  HHL_PROF_BEGIN(st);
+  if (c64) launch_dep(k_rows_scatter<float>, sg, kThreads, 0, st, (float2*)half, (const float2*)p.d_scratch, p.n_s, k, m_sub);
+  else launch_dep(k_rows_scatter<double>, sg, kThreads, 0, st, (double2*)half, (const double2*)p.d_scratch, p.n_s, k, m_sub);
   HHL_LAUNCH_CHECK("k_rows_scatter");
   return HHL_OK;
 }
