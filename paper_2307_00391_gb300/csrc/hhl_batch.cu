@@ -41,14 +41,21 @@ namespace {
 
 constexpr double kPiB = 3.14159265358979323846;
 
-// g_k(d) for d in [0, 2N+2) and every k: block (x = d chunk, y = k).
-__global__ void __launch_bounds__(256) k_ugen_g(int N, const double2* __restrict__ ph /* n_c x N */,
-                                               const double* __restrict__ cos_tab /* 2N+2 */,
-                                               float4* __restrict__ g /* n_c x (2N+2) */) {
+// g_k(d) for d in [0, 2N+2) and every k: block (x = d chunk, y = k, z = instance).
+struct GenInst {
+  int N, n_c;
+  const double2* ph;      // n_c x N
+  const double* cos_tab;  // 2N+2
+  float4* g;              // n_c x (2N+2)
+};
+__global__ void __launch_bounds__(256) k_ugen_g(const GenInst* __restrict__ inst) {
   extern __shared__ double2 sh_ph[];
-  const int k = blockIdx.y;
+  const GenInst in = inst[blockIdx.z];
+  const int N = in.N, k = blockIdx.y;
+  if (k >= in.n_c) return;  // block-uniform
+  const double* __restrict__ cos_tab = in.cos_tab;
   const int M = 2 * N + 2;
-  for (int j = threadIdx.x; j < N; j += blockDim.x) sh_ph[j] = ph[(size_t)k * N + j];
+  for (int j = threadIdx.x; j < N; j += blockDim.x) sh_ph[j] = in.ph[(size_t)k * N + j];
   __syncthreads();
   const double inv = 1.0 / (double)(N + 1);
   for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < M; d += gridDim.x * blockDim.x) {
@@ -65,7 +72,7 @@ __global__ void __launch_bounds__(256) k_ugen_g(int N, const double2* __restrict
     // double-float (hi + lo) in FP32, so that the expansion below runs in FP32 arithmetic
     const double gr = re * inv, gi = im * inv;
     const float rh = (float)gr, ih = (float)gi;
-    g[(size_t)k * M + d] = make_float4(rh, (float)(gr - (double)rh), ih, (float)(gi - (double)ih));
+    in.g[(size_t)k * M + d] = make_float4(rh, (float)(gr - (double)rh), ih, (float)(gi - (double)ih));
   }
 }
 
@@ -711,14 +718,38 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
                                          (int)std::max<int64_t>(maxN * (int64_t)sizeof(double2), 1024));
     if (e != cudaSuccess) s = cuda_fail(e, "cudaFuncSetAttribute(k_ugen_g)");
   }
-  // g_k for every k of every instance, once (they depend on A, T0 and k only)
-  for (int i = 0; i < count && s == HHL_OK; ++i) {
-    const Plan& p = B->plans[i];
-    const int M = (int)(2 * p.N + 2);
-    dim3 grid((unsigned)((M + 255) / 256), (unsigned)p.n_c);
-    k_ugen_g<<<grid, 256, p.N * sizeof(double2), is_large[i] ? B->work[B->stream_of[i]].s : (cudaStream_t)0>>>(
-        (int)p.N, B->d_ph + B->ph_off[i], B->d_cos + B->cos_off[i], B->d_g + B->g_off[i]);
-    if (cudaError_t le = cudaGetLastError(); le != cudaSuccess) s = cuda_fail(le, "k_ugen_g");
+  // g_k for every k of every instance, once (they depend on A, T0 and k only): one launch for the
+  // one-block solves, one each for the others on their worker streams
+  GenInst* d_gen = nullptr;
+  if (s == HHL_OK) {
+    std::vector<GenInst> gen;
+    std::vector<int> order_g;
+    int small_n = 0, small_k = 0;
+    for (int pass = 0; pass < 2; ++pass)
+      for (int i = 0; i < count; ++i) {
+        if ((int)is_large[i] != pass) continue;
+        const Plan& p = B->plans[i];
+        gen.push_back({(int)p.N, p.n_c, B->d_ph + B->ph_off[i], B->d_cos + B->cos_off[i], B->d_g + B->g_off[i]});
+        order_g.push_back(i);
+        if (pass == 0) {
+          small_n = std::max(small_n, (int)p.N);
+          small_k = std::max(small_k, p.n_c);
+        }
+      }
+    const int n_small = count - (int)B->large.size();
+    cudaError_t e = cudaMalloc((void**)&d_gen, gen.size() * sizeof(GenInst));
+    if (e == cudaSuccess) e = cudaMemcpy(d_gen, gen.data(), gen.size() * sizeof(GenInst), cudaMemcpyHostToDevice);
+    for (int z = 0; z < n_small && e == cudaSuccess; z += 65535) {
+      const dim3 grid((unsigned)((2 * small_n + 2 + 255) / 256), (unsigned)small_k, (unsigned)std::min(65535, n_small - z));
+      k_ugen_g<<<grid, 256, small_n * sizeof(double2)>>>(d_gen + z);
+      e = cudaGetLastError();
+    }
+    for (size_t q = n_small; q < gen.size() && e == cudaSuccess; ++q) {
+      const dim3 grid((unsigned)((2 * gen[q].N + 2 + 255) / 256), (unsigned)gen[q].n_c);
+      k_ugen_g<<<grid, 256, gen[q].N * sizeof(double2), B->work[B->stream_of[order_g[q]]].s>>>(d_gen + q);
+      e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) s = cuda_fail(e, "k_ugen_g");
   }
   if (s == HHL_OK && (int)B->large.size() < count) {
     // the one-block solves, largest first, in at most three launches (the shared memory of a launch is
@@ -754,6 +785,7 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) s = cuda_fail(e, "batch setup");
   }
+  if (d_gen) cudaFree(d_gen);
   if (s != HHL_OK) {
     free_batch(B);
     return s;
