@@ -59,6 +59,7 @@ __device__ __forceinline__ int64_t row_with_bit(int64_t i, int k) {
 // ------------------------------------------------------------------------------ prep
 
 __global__ void k_bnorm(const double2* __restrict__ b, int64_t n, double* acc) {
+  dep_begin();
   double s[1] = {0.0};
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double2 z = b[i];
@@ -71,6 +72,7 @@ __global__ void k_bnorm(const double2* __restrict__ b, int64_t n, double* acc) {
 template <class R>
 __global__ void k_prep_scale(const double2* __restrict__ b, const double* __restrict__ acc,
                              typename Cx<R>::T* __restrict__ bs, int64_t N, int n_c) {
+  dep_begin();
   const double nb2 = acc[0];
   const double scale = nb2 > 0.0 ? 1.0 / sqrt(nb2 * (double)(1LL << n_c)) : 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
@@ -408,6 +410,7 @@ __global__ void __launch_bounds__(kThreads) k_row_finish_small(const typename Cx
 // |v|^2 of one row of N amplitudes (the postselected row), FP64.
 template <class R>
 __global__ void k_row_norm(const typename Cx<R>::T* __restrict__ v, int64_t N, double* acc) {
+  dep_begin();
   double s[1] = {0.0};
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x) {
     const double re = (double)v[j].x, im = (double)v[j].y;
@@ -420,6 +423,7 @@ __global__ void k_row_norm(const typename Cx<R>::T* __restrict__ v, int64_t N, d
 template <class R>
 __global__ void k_measure_finish(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
                                  const double* __restrict__ scal, double* __restrict__ out) {
+  dep_begin();
   const double ps = scal[3];
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i == 0) {
@@ -580,6 +584,7 @@ template <class R>
 __global__ void k_diss_sum(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
                            const double* __restrict__ scal, double inv_c_lam, double wlo, double whi,
                            double* acc, double* __restrict__ u_out) {
+  dep_begin();
   const double scale = sqrt(scal[0]) * inv_c_lam;
   double s[1] = {0.0};
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= N; i += (int64_t)gridDim.x * blockDim.x) {
@@ -616,6 +621,7 @@ __global__ void __launch_bounds__(kThreads) k_diss_small(const typename Cx<R>::T
 }
 
 __global__ void k_diss_finish(const double* __restrict__ acc, double nu_over_h, double* eps) {
+  dep_begin();
   if (threadIdx.x == 0 && blockIdx.x == 0) eps[0] = nu_over_h * acc[0];
 }
 
@@ -726,7 +732,7 @@ __global__ void k_store_operands(const double2* __restrict__ U, int64_t N, typen
 
 hhl_status launch_bnorm(const double* b, int64_t N, double* acc, cudaStream_t st) {
   HHL_PROF_BEGIN(st);
-  k_bnorm<<<grid_for(N, kThreads, 152), kThreads, 0, st>>>((const double2*)b, N, acc);
+  launch_dep(k_bnorm, grid_for(N, kThreads, 152), kThreads, 0, st, (const double2*)b, N, acc);
   HHL_LAUNCH_CHECK("k_bnorm");
   return HHL_OK;
 }
@@ -757,9 +763,9 @@ hhl_status launch_prep_fill(const Plan& p, const double* b, void* state, cudaStr
     const int gs = grid_for(p.N, kThreads, 152);
     HHL_PROF_BEGIN(st);
     if (p.prec == HHL_PREC_C64)
-      k_prep_scale<float><<<gs, kThreads, 0, st>>>((const double2*)b, p.d_scal, (float2*)p.d_bs, p.N, p.n_c);
+      launch_dep(k_prep_scale<float>, gs, kThreads, 0, st, (const double2*)b, p.d_scal, (float2*)p.d_bs, p.N, p.n_c);
     else
-      k_prep_scale<double><<<gs, kThreads, 0, st>>>((const double2*)b, p.d_scal, (double2*)p.d_bs, p.N, p.n_c);
+      launch_dep(k_prep_scale<double>, gs, kThreads, 0, st, (const double2*)b, p.d_scal, (double2*)p.d_bs, p.N, p.n_c);
     HHL_LAUNCH_CHECK("k_prep_scale");
   }
   const int64_t row_units = p.N * (int64_t)p.amp_bytes() / 16;
@@ -822,15 +828,22 @@ hhl_status launch_ctrl_u_simt(const Plan& p, void* half, int k, const void* B, c
 hhl_status launch_ctrl_u_simt_map(const Plan& p, void* half, const RowMap& k, int64_t m_sub, const void* B,
                                   cudaStream_t st) {
   const int64_t N = p.N;
+  // 64 x 64 tiles; when those leave SMs idle, 16-row tiles as wide as the row (64 rows of 128 points:
+  // 2 blocks of 34 us become 4 of 9), which also write in place up to 256 points
   dim3 grid((unsigned)((N + 63) / 64), (unsigned)((m_sub + 63) / 64));
   const int sg = grid_for(m_sub * N, kThreads, 152 * 32);
-  const bool c64 = p.prec == HHL_PREC_C64, in_place = N <= 64;
+  const bool c64 = p.prec == HHL_PREC_C64, few = (int64_t)grid.x * grid.y < 152 && N <= (c64 ? 256 : 128);
+  const bool in_place = few || N <= 64;
+  if (few) grid = dim3(1, (unsigned)((m_sub + 15) / 16));
   HHL_PROF_BEGIN(st);
   if (c64) {
-    auto kern = in_place ? k_ctrl_gemm_simt<float, 64, 64, 16, true> : k_ctrl_gemm_simt<float, 64, 64, 16, false>;
+    auto kern = few ? (N <= 64 ? k_ctrl_gemm_simt<float, 16, 64, 16, true> : N <= 128 ? k_ctrl_gemm_simt<float, 16, 128, 16, true>
+                                                                                     : k_ctrl_gemm_simt<float, 16, 256, 16, true>)
+                : in_place ? k_ctrl_gemm_simt<float, 64, 64, 16, true> : k_ctrl_gemm_simt<float, 64, 64, 16, false>;
     launch_dep(kern, grid, 256, 0, st, (float2*)half, (float2*)p.d_scratch, (const float2*)B, p.n_s, k, m_sub);
   } else {
-    auto kern = in_place ? k_ctrl_gemm_simt<double, 64, 64, 8, true> : k_ctrl_gemm_simt<double, 64, 64, 8, false>;
+    auto kern = few ? (N <= 64 ? k_ctrl_gemm_simt<double, 16, 64, 8, true> : k_ctrl_gemm_simt<double, 16, 128, 8, true>)
+                : in_place ? k_ctrl_gemm_simt<double, 64, 64, 8, true> : k_ctrl_gemm_simt<double, 64, 64, 8, false>;
     launch_dep(kern, grid, 256, 0, st, (double2*)half, (double2*)p.d_scratch, (const double2*)B, p.n_s, k, m_sub);
   }
   HHL_LAUNCH_CHECK(c64 ? "k_ctrl_gemm_simt<f32>" : "k_ctrl_gemm_simt<f64>");
@@ -871,15 +884,15 @@ hhl_status launch_measure_row(const Plan& p, const void* state, double* out, cud
   const int gf = grid_for(p.N, kThreads, 152 * 4);
   HHL_PROF_BEGIN(st);
   if (p.prec == HHL_PREC_C64)
-    k_row_norm<float><<<gf, kThreads, 0, st>>>((const float2*)state + half, p.N, p.d_scal + 3);
+    launch_dep(k_row_norm<float>, gf, kThreads, 0, st, (const float2*)state + half, p.N, p.d_scal + 3);
   else
-    k_row_norm<double><<<gf, kThreads, 0, st>>>((const double2*)state + half, p.N, p.d_scal + 3);
+    launch_dep(k_row_norm<double>, gf, kThreads, 0, st, (const double2*)state + half, p.N, p.d_scal + 3);
   HHL_LAUNCH_CHECK("k_row_norm");
   HHL_PROF_BEGIN(st);
   if (p.prec == HHL_PREC_C64)
-    k_measure_finish<float><<<gf, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal, out);
+    launch_dep(k_measure_finish<float>, gf, kThreads, 0, st, (const float2*)state, half, p.N, p.d_scal, out);
   else
-    k_measure_finish<double><<<gf, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal, out);
+    launch_dep(k_measure_finish<double>, gf, kThreads, 0, st, (const double2*)state, half, p.N, p.d_scal, out);
   HHL_LAUNCH_CHECK("k_measure_finish");
   return HHL_OK;
 }
@@ -893,9 +906,9 @@ hhl_status launch_prep_row(const Plan& p, const double* b, void* state, cudaStre
   const int gs = grid_for(p.N, kThreads, 152);
   HHL_PROF_BEGIN(st);
   if (p.prec == HHL_PREC_C64)
-    k_prep_scale<float><<<gs, kThreads, 0, st>>>((const double2*)b, p.d_scal, (float2*)p.d_bs, p.N, p.n_c);
+    launch_dep(k_prep_scale<float>, gs, kThreads, 0, st, (const double2*)b, p.d_scal, (float2*)p.d_bs, p.N, p.n_c);
   else
-    k_prep_scale<double><<<gs, kThreads, 0, st>>>((const double2*)b, p.d_scal, (double2*)p.d_bs, p.N, p.n_c);
+    launch_dep(k_prep_scale<double>, gs, kThreads, 0, st, (const double2*)b, p.d_scal, (double2*)p.d_bs, p.N, p.n_c);
   HHL_LAUNCH_CHECK("k_prep_scale");
   HHL_CUDA_TRY(cudaMemcpyAsync(state, p.d_bs, (size_t)p.N * p.amp_bytes(), cudaMemcpyDeviceToDevice, st));
   return HHL_OK;
@@ -925,7 +938,7 @@ hhl_status launch_measure(const Plan& p, const void* state, double* out, cudaStr
     launch_dep(k_measure_sums<float, false>, g, kThreads, 0, st, (const float2*)state, half, p.N, p.d_scal + 1);
     HHL_LAUNCH_CHECK("k_measure_sums");
     HHL_PROF_BEGIN(st);
-    k_measure_finish<float><<<gf, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal, out);
+    launch_dep(k_measure_finish<float>, gf, kThreads, 0, st, (const float2*)state, half, p.N, p.d_scal, out);
   } else {
     const char* env = getenv("HHL_FP64_PIPE");
     HHL_PROF_BEGIN(st);
@@ -935,7 +948,7 @@ hhl_status launch_measure(const Plan& p, const void* state, double* out, cudaStr
       launch_dep(k_measure_sums<double, true>, g, kThreads, 0, st, (const double2*)state, half, p.N, p.d_scal + 1);
     HHL_LAUNCH_CHECK("k_measure_sums");
     HHL_PROF_BEGIN(st);
-    k_measure_finish<double><<<gf, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal, out);
+    launch_dep(k_measure_finish<double>, gf, kThreads, 0, st, (const double2*)state, half, p.N, p.d_scal, out);
   }
   HHL_LAUNCH_CHECK("k_measure_finish");
   return HHL_OK;
@@ -1065,16 +1078,16 @@ hhl_status launch_dissipation(const Plan& p, const void* state, double* eps, dou
   const int g = grid_for(p.N + 1, kThreads, 152 * 4);
   if (p.prec == HHL_PREC_C64) {
     HHL_PROF_BEGIN(st);
-    k_diss_sum<float><<<g, kThreads, 0, st>>>((const float2*)state, half, p.N, p.d_scal, inv_c_lam, p.wall_lo,
+    launch_dep(k_diss_sum<float>, g, kThreads, 0, st, (const float2*)state, half, p.N, p.d_scal, inv_c_lam, p.wall_lo,
                                               p.wall_hi, p.d_scal + 4, u_dev);
   } else {
     HHL_PROF_BEGIN(st);
-    k_diss_sum<double><<<g, kThreads, 0, st>>>((const double2*)state, half, p.N, p.d_scal, inv_c_lam, p.wall_lo,
+    launch_dep(k_diss_sum<double>, g, kThreads, 0, st, (const double2*)state, half, p.N, p.d_scal, inv_c_lam, p.wall_lo,
                                                p.wall_hi, p.d_scal + 4, u_dev);
   }
   HHL_LAUNCH_CHECK("k_diss_sum");
   HHL_PROF_BEGIN(st);
-  k_diss_finish<<<1, 32, 0, st>>>(p.d_scal + 4, p.nu * (double)(p.N + 1), eps);
+  launch_dep(k_diss_finish, 1, 32, 0, st, p.d_scal + 4, p.nu * (double)(p.N + 1), eps);
   HHL_LAUNCH_CHECK("k_diss_finish");
   return HHL_OK;
 }
