@@ -831,6 +831,76 @@ __device__ __forceinline__ void tile_stages(T* X, int b0, int lo_fixed, int m, c
   }
 }
 
+// The double-float passes read their twiddles from a table instead of forming them per group: a
+// complex product is about 32 FP32 operations there, and each group of 8 formed 7 factors with 7
+// products (three table look-ups, four roots) next to 12 butterflies of one product each. All lanes
+// of a warp work on the same rows, so a read is a broadcast. The stages of 2^NB rows have 2^NB - 1
+// factors in all: pass (TB, RB), in order, holds 2^RB - 1 for each value of its TB lower bits.
+template <class T, int NB, bool DIT, int Q = 0, int DONE = 0, class TW>
+__device__ __forceinline__ void build_factors(T* tab, int b0, int lo_fixed, int m, const TW& tw, bool conj) {
+  constexpr int MR = SplitGeom<T>::MR;
+  constexpr int NPASS = (NB + MR - 1) / MR;
+  using R = decltype(T().x);
+  if constexpr (Q < NPASS) {
+    constexpr int RB = (NB - DONE) / (NPASS - Q), TB = DIT ? DONE : NB - DONE - RB;
+    constexpr int F = (1 << RB) - 1, count = F << TB;
+    for (int e = threadIdx.x; e < count; e += blockDim.x) {
+      const int lo = e / F, i = e - lo * F;
+      const int t = 31 - __clz(i + 1), xr = i + 1 - (1 << t), s = t + 1 + b0 + TB;
+      T f = tw((lo_fixed + (lo << b0)) << (m - s), conj);
+      if (xr != 0) {
+        const int k16 = xr << (3 - t);
+        T w;
+        w.x = root16<R>(k16, 0);
+        w.y = conj ? -root16<R>(k16, 1) : root16<R>(k16, 1);
+        f = cmul(f, w);
+      }
+      tab[e] = f;
+    }
+    build_factors<T, NB, DIT, Q + 1, DONE + RB>(tab + count, b0, lo_fixed, m, tw, conj);
+  }
+}
+
+// tile_stages with those factors.
+template <class T, int NB, bool DIT, int LW, bool CV, int Q = 0, int DONE = 0>
+__device__ __forceinline__ void tile_stages_tab(T* X, const T* tab) {
+  constexpr int MR = SplitGeom<T>::MR;
+  constexpr int NPASS = (NB + MR - 1) / MR;
+  if constexpr (Q < NPASS) {
+    constexpr int RB = (NB - DONE) / (NPASS - Q), TB = DIT ? DONE : NB - DONE - RB;
+    constexpr int W = 1 << LW, G = 1 << RB, F = G - 1;
+#pragma unroll 1
+    for (int g = threadIdx.x; g < (W << (NB - RB)); g += blockDim.x) {
+      const int w = g & (W - 1), gg = g >> LW, lo = gg & ((1 << TB) - 1);
+      T* q = X + ((((gg >> TB) << (TB + RB)) + lo) << LW) + w;
+      const T* f = tab + lo * F;
+      T v[G];
+#pragma unroll
+      for (int x = 0; x < G; ++x) {
+        if constexpr (CV && Q == 0) v[x] = amp_in<T>(q, (long long)x << (TB + LW));
+        else v[x] = q[x << (TB + LW)];
+      }
+#pragma unroll
+      for (int tt = 0; tt < RB; ++tt) {
+        const int t = DIT ? tt : (RB - 1 - tt);
+#pragma unroll
+        for (int x = 0; x < G; ++x) {
+          if (x & (1 << t)) continue;
+          const int x1 = x | (1 << t);
+          const T fx = f[(1 << t) - 1 + (x & ((1 << t) - 1))];
+          const T a = v[x], b = DIT ? cmul(v[x1], fx) : v[x1];
+          v[x] = cadd(a, b);
+          v[x1] = DIT ? csub(a, b) : cmul(csub(a, b), fx);
+        }
+      }
+#pragma unroll
+      for (int x = 0; x < G; ++x) q[x << (TB + LW)] = v[x];
+    }
+    __syncthreads();
+    tile_stages_tab<T, NB, DIT, LW, CV, Q + 1, DONE + RB>(X, tab + (F << TB));
+  }
+}
+
 __device__ __forceinline__ void split_cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void split_cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
@@ -909,7 +979,7 @@ __device__ __forceinline__ TilePos tile_pos(const SplitArgs& a, long long t) {
 template <class R, int OP, bool FULL, int NB, bool WHOLE, bool CS = false, class TW>
 __device__ __forceinline__ void split_tile(const SplitArgs& a, const TilePos& q, typename Cx<R>::T* X,
                                            typename Cx<R>::T* Y, const TW& tw, int mt, long long row_units,
-                                           MidSums<R>* sums = nullptr) {
+                                           MidSums<R>* sums = nullptr, typename Cx<R>::T* tab = nullptr) {
   using T = typename Cx<R>::T;
   constexpr int upr = kSplitSegBytes / 16;
   constexpr int per = 16 / sizeof(T);
@@ -922,17 +992,20 @@ __device__ __forceinline__ void split_tile(const SplitArgs& a, const TilePos& q,
     else tile_stages<T, NB, true, 0>(X, a.b0, q.lo_fixed, mt, tw, false, q.inner_base, a.lo);
     tile_store<T, NB, CS>(dst, X, row_units, q.row0, a.b0, (R)1, false);
   } else if (OP == kSplitDif) {
-    tile_stages<T, NB, false, 0, LWT, 0, 0, CVT>(X, a.b0, q.lo_fixed, a.m, tw, false);
+    if constexpr (CVT) tile_stages_tab<T, NB, false, LWT, true>(X, tab);
+    else tile_stages<T, NB, false, 0, LWT, 0, 0, CVT>(X, a.b0, q.lo_fixed, a.m, tw, false);
     tile_store<T, NB, CS>(dst, X, row_units, q.row0, a.b0, (R)1, false);
   } else if (OP == kSplitDit) {
-    tile_stages<T, NB, true, 0, LWT, 0, 0, CVT>(X, a.b0, q.lo_fixed, a.m, tw, true);
+    if constexpr (CVT) tile_stages_tab<T, NB, true, LWT, true>(X, tab);
+    else tile_stages<T, NB, true, 0, LWT, 0, 0, CVT>(X, a.b0, q.lo_fixed, a.m, tw, true);
     tile_store<T, NB, CS>(dst, X, row_units, q.row0, a.b0, (R)1, false);
   } else if (OP == kSplitHad) {
     tile_stages<T, NB, false, 1, LWT, 0, 0, CVT>(X, a.b0, q.lo_fixed, a.m, tw, false);
     tile_store<T, NB, CS>(dst, X, row_units, q.row0, a.b0, split_scale<R>(a), a.scaled != 0);
   } else {  // kSplitMid(Sums): b0 = 0, the tile holds every low bit of the rows hi_fixed << NB
     constexpr bool SUMS = OP == kSplitMidSums;
-    tile_stages<T, NB, false, 0, LWT, 0, 0, CVT>(X, 0, 0, a.m, tw, false);
+    if constexpr (CVT) tile_stages_tab<T, NB, false, LWT, true>(X, tab);
+    else tile_stages<T, NB, false, 0, LWT, 0, 0, CVT>(X, 0, 0, a.m, tw, false);
     const R s = split_scale<R>(a);
     uint4* cos_out = reinterpret_cast<uint4*>(static_cast<T*>(a.dst_cos) + q.base_amp);
     for (int u = threadIdx.x; u < (upr << NB); u += kSplitThreads) {
@@ -965,8 +1038,13 @@ __device__ __forceinline__ void split_tile(const SplitArgs& a, const TilePos& q,
       }
     }
     __syncthreads();
-    tile_stages<T, NB, true, 0>(X, 0, 0, a.m, tw, true);
-    if (FULL) tile_stages<T, NB, true, 0>(Y, 0, 0, a.m, tw, true);
+    if constexpr (CVT) {
+      tile_stages_tab<T, NB, true, LWT, false>(X, tab + (1 << NB));
+      if (FULL) tile_stages_tab<T, NB, true, LWT, false>(Y, tab + (1 << NB));
+    } else {
+      tile_stages<T, NB, true, 0>(X, 0, 0, a.m, tw, true);
+      if (FULL) tile_stages<T, NB, true, 0>(Y, 0, 0, a.m, tw, true);
+    }
     tile_store<T, NB, CS>(dst, X, row_units, q.row0, 0, (R)1, false);
     if (FULL) tile_store<T, NB, CS>(reinterpret_cast<T*>(cos_out), Y, row_units, q.row0, 0, (R)1, false);
   }
@@ -994,6 +1072,8 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitMinBlocks<R, OP>) k_split
   T* t1 = t0 + 64;
   T* Xb = t0 + (WHOLE ? 1024 : twiddle_entries(a.m));  // two tile buffers (double buffering), then Y
   T* Y = Xb + 2 * tile_amps;
+  constexpr bool TAB = is_dfc<T>() && !WHOLE && OP != kSplitHad, MID = OP == kSplitMid || OP == kSplitMidSums;
+  T* tab = Y + (MID && FULL ? tile_amps : 0);  // (double-float) twiddles of the pass, 2^NB each way
   if (!WHOLE && OP != kSplitHad) fill_twiddles<R>(t0, t1, a.m);
   if constexpr (WHOLE) fill_twiddle4<R>(t0, a.lo + a.m);  // first read after the barrier of the first tile
   using TW = typename std::conditional<WHOLE, Twiddle4<T>, Twiddle<T>>::type;
@@ -1016,6 +1096,14 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitMinBlocks<R, OP>) k_split
     tile_issue<T, NB>(Xb, static_cast<const T*>(a.src) + q.base_amp, row_units, q.row0, a.b0);
   }
   split_cp_async_commit();
+  int tab_lo = -1;  // the fixed lower bits that the table holds
+  if constexpr (TAB) {
+    __syncthreads();  // the two-level tables are complete
+    if constexpr (MID) {
+      build_factors<T, NB, false>(tab, 0, 0, a.m, tw, false);
+      build_factors<T, NB, true>(tab + (1 << NB), 0, 0, a.m, tw, true);
+    }
+  }
   int buf = 0;
   for (; t < a.tiles; t += gridDim.x) {
     const long long tn = t + gridDim.x;
@@ -1025,10 +1113,16 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitMinBlocks<R, OP>) k_split
                         a.b0);
     }
     split_cp_async_commit();
+    const TilePos q = tile_pos<NB, LW>(a, t);
+    if constexpr (TAB && !MID) {  // (the previous tile's readers are past the barrier below)
+      if (q.lo_fixed != tab_lo) {  // block-uniform
+        tab_lo = q.lo_fixed;
+        build_factors<T, NB, OP == kSplitDit>(tab, a.b0, tab_lo, a.m, tw, OP == kSplitDit);
+      }
+    }
     split_cp_async_wait1();
     __syncthreads();  // the current tile has landed for every thread
-    const TilePos q = tile_pos<NB, LW>(a, t);
-    split_tile<R, OP, FULL, NB, WHOLE>(a, q, Xb + buf * tile_amps, Y, tw, mt, row_units, &sums);
+    split_tile<R, OP, FULL, NB, WHOLE>(a, q, Xb + buf * tile_amps, Y, tw, mt, row_units, &sums, tab);
     __syncthreads();  // this buffer is read out before it is refilled
     buf ^= 1;
   }
@@ -1067,7 +1161,8 @@ template <class R, int OP, bool FULL, int NB, bool WHOLE = false>
 hhl_status launch_split_nb(const SplitArgs& a, cudaStream_t st, const char* name) {
   using T = typename Cx<R>::T;
   const size_t tile = ((size_t)1 << (NB + SplitGeom<T>::LW)) * sizeof(T);
-  const size_t smem = (size_t)(WHOLE ? 1024 : twiddle_entries(a.m)) * sizeof(T) + ((OP == kSplitMid && FULL) ? 3 : 2) * tile;
+  const size_t smem = (size_t)(WHOLE ? 1024 : twiddle_entries(a.m)) * sizeof(T) + ((OP == kSplitMid && FULL) ? 3 : 2) * tile +
+                      (is_dfc<T>() && !WHOLE && OP != kSplitHad ? ((size_t)2 << NB) * sizeof(T) : 0);
   auto kern = k_split_pass<R, OP, FULL, NB, WHOLE>;
   HHL_CUDA_TRY(raise_dyn_smem((const void*)kern, smem));
   int dev = 0, sms = 0, occ = 0;
