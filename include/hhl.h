@@ -309,7 +309,10 @@ hhl_status hhl_apply_stage(hhl_plan_t plan, int32_t stage, void* state_dev, void
  * in a fixed order, so results repeat bit for bit), below that on the CUDA cores (for a
  * Toeplitz tridiagonal A with U_k generated on the fly from its eigenbasis; the threshold moves
  * with the environment variable HHL_TOEP_ROWS=<rows>); Strang-Trotter plans as grouped Strang
- * passes.
+ * passes. complex128 dense plans of a real A with gemm = HHL_GEMM_AUTO evaluate the same circuit in
+ * the eigenbasis of A (every gate on the system register is diagonal there), here and in
+ * hhl_apply_circuit; hhl_apply_stage applies the gate products. An explicit GEMM choice keeps them
+ * everywhere.
  * Errors: HHL_ERR_UNSUPPORTED unless full_uncompute = 0 and, for Strang-Trotter plans, every
  * clock bit's layer list fits one pass (2 r_k + 1 <= 17). */
 hhl_status hhl_solve_postselected(hhl_plan_t plan, const double* b_dev, void* state_dev, double* out_dev,
@@ -359,7 +362,7 @@ hhl_status hhl_dissipation(hhl_plan_t plan, const void* state_dev, double* eps_o
 /* ---------------------------------------------------------------------------------- batch
  * Many HHL instances of uneven size in one CUDA graph (growth direction of the path: the
  * paper's sweeps over T0, clock count and system size, Sec. VI, run as one batch). Every
- * instance is the postselected solve of hhl_solve_postselected in its dense form (complex64:
+ * instance is the gate-product form of hhl_solve_postselected for dense plans (complex64:
  * QPE by doubling and the uncompute by halving as controlled-U GEMMs on 2^k rows, tcgen05 where
  * 2^k >= 128, the clock block), with the outputs of hhl_measure_async and
  * hhl_dissipation_async; A must be a
@@ -367,16 +370,18 @@ hhl_status hhl_dissipation(hhl_plan_t plan, const void* state_dev, double* eps_o
  * eigenbasis (U_k[n][m] = g_k(|n-m|) - g_k(n+m)): hhl_batch_create computes the g_k of every
  * instance (an O(N^2) FP64 kernel per k, kept on the device as double-float pairs), and each
  * run generates U_k from them on the fly (tree steps below 128 rows) or expands it into a
- * per-stream GEMM operand right before its product. */
+ * per-stream GEMM operand right before its product. Instances with n_c <= 7, N <= 128 and the CUDA-core
+ * GEMM are solved by one thread block each, in a few launches beside the graph (the same
+ * arithmetic); a batch of only such instances has no graph. */
 typedef struct hhl_batch_s* hhl_batch_t;
 
 typedef struct hhl_batch_info {
   int32_t count;            /* instances */
-  int32_t streams;          /* worker streams of the graph */
+  int32_t streams;          /* worker streams of the graph (none busy with one-block solves) */
   uint64_t state_bytes;     /* all instance states (device) */
   uint64_t workspace_bytes; /* per-stream operand and row buffers (device) */
   double gemm_flops;        /* algorithmic flops of all controlled products of one run */
-  uint64_t graph_launches;  /* kernels in the graph (0 before the first run) */
+  uint64_t graph_launches;  /* kernels of one run: the graph's and the one-block solves' (0 before the first run) */
   int64_t b_doubles;        /* length of the packed right-hand-side array */
   int64_t out_doubles;      /* length of the packed measurement array */
 } hhl_batch_info;
@@ -398,8 +403,8 @@ hhl_status hhl_batch_instance(hhl_batch_t batch, int32_t index, int32_t* n_sys_q
 /* Run every instance. b_dev: DEVICE packed complex128 right-hand sides (instance i at its
  * b_offset, N_i complex values). out_dev: DEVICE packed blocks of 4 + 2 N_i doubles in the
  * layout of hhl_measure_async; eps_dev: DEVICE count doubles (dissipation). The first call
- * captures the graph (so it must not itself be inside a stream capture); later calls replay
- * it with one launch. Asynchronous on stream. */
+ * captures the graph, if any instance needs one (so it must not itself be inside a stream capture);
+ * later calls replay it with one launch. Asynchronous on stream. */
 hhl_status hhl_batch_run(hhl_batch_t batch, const double* b_dev, double* out_dev, double* eps_dev, void* stream);
 /* The same work enqueued launch by launch on the worker streams instead of replaying the
  * graph (for per-kernel timing with hhl_profile_*): reads the right-hand sides already in

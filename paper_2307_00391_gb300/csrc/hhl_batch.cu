@@ -129,7 +129,7 @@ __global__ void k_ugen_embed_simt(int n_s, const float4* __restrict__ g, int adj
 // Instances whose clock and system registers fit one block's shared memory (n_c <= 7, N <= 128): the
 // whole postselected solve in one launch for all of them, a block each, instead of about 17
 // launches per instance (384 instances of 2^3..2^6 points: 6,900 launches of 0.6 us each on 8
-// streams, 3.9 ms; now one launch). Bound by the latency of the 2 n_c dependent products. The
+// streams, 3.95 ms; one launch takes 125 us). Bound by the latency of the 2 n_c dependent products. The
 // arithmetic is that of the launches it replaces, operation for operation: U_k from its g table,
 // every output of a product as 32 partial sums over m (mod 32) added in the order of
 // k_toeplitz_rows' shuffles and warps, the transform stages of k_clock_block, the squares of
@@ -842,11 +842,17 @@ hhl_status hhl_batch_run(hhl_batch_t b, const double* b_dev, double* out_dev, do
   }
   hhl_status s = capture(b);
   if (s != HHL_OK) return s;
-  if (b->exec == nullptr)  // one-block solves only (they keep the right-hand sides for hhl_batch_run_eager)
+  // One-block solves only: they read and write the caller's arrays themselves (and keep the right-hand
+  // sides for hhl_batch_run_eager) where 16-byte loads may and no output lies in what another block reads.
+  const double* b_end = b_dev + bo;
+  const bool apart = (out_dev >= b_end || out_dev + oo <= b_dev) && (eps_dev >= b_end || eps_dev + b->count <= b_dev);
+  if (b->exec == nullptr && (uintptr_t)b_dev % sizeof(double2) == 0 && apart)
     return run_small(b, b_dev, b->d_b, out_dev, eps_dev, st);
   HHL_CUDA_TRY(cudaMemcpyAsync(b->d_b, b_dev, bo * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  HHL_CUDA_TRY(cudaGraphLaunch(b->exec, st));
-  g_launches.fetch_add(b->captured, std::memory_order_relaxed);
+  if (b->exec != nullptr) {
+    HHL_CUDA_TRY(cudaGraphLaunch(b->exec, st));
+    g_launches.fetch_add(b->captured, std::memory_order_relaxed);
+  }
   s = run_small(b, b->d_b, nullptr, b->d_out, b->d_eps, st);
   if (s != HHL_OK) return s;
   HHL_CUDA_TRY(cudaMemcpyAsync(out_dev, b->d_out, oo * sizeof(double), cudaMemcpyDeviceToDevice, st));

@@ -49,7 +49,7 @@ void prof_end(const char* name);
 // ------------------------------------------------------------------ dependent launches
 // Chains of short kernels on one stream: a kernel launched with launch_dep may be scheduled once every
 // block of the kernel before it has started, so its launch and prologue run under that kernel's
-// tail (about 1.5 us a launch on GB300). Every such kernel calls dep_wait() in all its threads before it
+// tail (a solve of 59 launches: 456 -> 316 us). Every such kernel calls dep_wait() in all its threads before it
 // touches global memory: that returns when the kernel before it, and so by induction everything
 // before that, has completed and its writes are visible. dep_launch() lets the next one in.
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

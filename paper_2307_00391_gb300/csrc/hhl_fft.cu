@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(kFftWide, 1) k_clock_block(typename Cx<R>::T* 
 // FP64 pipe bounds it, not the row segments). Radix-2 stages with their roots read from the plan's
 // table: on that pipe a table read is cheaper than forming a root, and every butterfly is a
 // thread of its own, which at 2^6 clock rows matters more than the round trips it costs (radix-8
-// groups with composed roots took 30 us at 16 columns of 2^6 rows, this form 9).
+// groups with composed roots took 30 us at 16 columns of 2^6 rows, this form 14).
 // OP 0: DIF inverse-QFT butterflies, 1: DIT QFT butterflies, 2: Hadamards.
 template <int OP>
 __device__ __forceinline__ void radix2_stages(double2* X, int Lp, int W, int m, const double2* __restrict__ roots) {

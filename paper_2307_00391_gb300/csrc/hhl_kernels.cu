@@ -92,7 +92,7 @@ __global__ void k_prep_fill(const uint4* __restrict__ bs, uint4* __restrict__ st
 }
 
 // Systems of at most kSmallN points: the norm, the scaled row and the fill in one launch instead of
-// four (memset, norm, scale, fill: 22 us back to back against 4 us on an 11-qubit state). Every
+// four (memset, norm, scale, fill), whose launches bound them. Every
 // block forms |b|^2 and the row itself (at most 16 KiB of reads that hit L2); beyond kSmallN that
 // repetition would cost more than the launches. row_only: just the clock = 0 row (one block).
 constexpr int kSmallN = 1024;
@@ -363,7 +363,7 @@ __device__ void measure_write(const typename Cx<R>::T* __restrict__ v, int64_t N
 // Systems of at most kSmallN points: the sums over the state and the measurement block in one
 // launch. Every block leaves its three partial sums in `part`; the block that draws the last
 // ticket adds them in block order (the same total on every run), writes the block and returns
-// the ticket counter to zero. Saves a memset and a launch (5 us of 13 on a 2 MiB state).
+// the ticket counter to zero. Saves a memset and a launch, which bound such states.
 template <class R, bool DF>
 __global__ void __launch_bounds__(kThreads) k_measure_small(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
                                                             double* __restrict__ scal, double* __restrict__ part,
@@ -828,8 +828,8 @@ hhl_status launch_ctrl_u_simt(const Plan& p, void* half, int k, const void* B, c
 hhl_status launch_ctrl_u_simt_map(const Plan& p, void* half, const RowMap& k, int64_t m_sub, const void* B,
                                   cudaStream_t st) {
   const int64_t N = p.N;
-  // 64 x 64 tiles; when those leave SMs idle, 16-row tiles as wide as the row (64 rows of 128 points:
-  // 2 blocks of 34 us become 4 of 9), which also write in place up to 256 points
+  // 64 x 64 tiles; when those leave SMs idle, 16-row tiles as wide as the row, which also write in
+  // place up to 256 points (7 + 7 qubits, 64 rows of 128 points a product: 476 -> 367 us a solve)
   dim3 grid((unsigned)((N + 63) / 64), (unsigned)((m_sub + 63) / 64));
   const int sg = grid_for(m_sub * N, kThreads, 152 * 32);
   const bool c64 = p.prec == HHL_PREC_C64, few = (int64_t)grid.x * grid.y < 152 && N <= (c64 ? 256 : 128);

@@ -8,7 +8,7 @@
 // lambdahat_j T0 / 2^{n_c}), then V^T on every row of both halves: three real N x N products
 // instead of 2 n_c complex ones on half the rows. GB300's FP64 pipe is about 1/32 of its FP32
 // one, so the products bound these plans: N = 16, 2^6 clock rows (11 qubits) took 12 products of
-// 70 us each, 0.93 ms a solve, and takes 45 us this way. complex64 plans keep their gate products:
+// 70 us each, 0.93 ms a solve, and takes 35 us this way. complex64 plans keep their gate products:
 // their read-outs are FP64 values of FP32 states, and this form rounds those states differently
 // (nearer to the exact circuit, but by 1e-7 to 4e-5 of the read-out).
 //
@@ -394,7 +394,8 @@ hhl_status spec_create(Plan& p, const std::vector<double>& lam, const std::vecto
   if (cudaMalloc(&s->mem, bytes) != cudaSuccess) {
     cudaGetLastError();
     s->mem = nullptr;
-    return fail(HHL_ERR_OOM, "eigenbasis tables");
+    spec_free(p);  // no room beside the operands: the plan runs its gate products
+    return HHL_OK;
   }
   p.table_bytes += bytes;
   double* d = static_cast<double*>(s->mem);

@@ -86,3 +86,22 @@ def test_mixed_with_larger_instances(hhl):
         np.testing.assert_allclose(got[inst["out_offset"]:inst["out_offset"] + 4 + 2 * inst["N"]], ref, rtol=1e-12, atol=1e-14)
         assert float(eps[i]) == pytest.approx(ref_eps, rel=1e-12)
     batch.close()
+
+
+@pytest.mark.parametrize("form", ["offset", "overlap"])
+def test_caller_arrays_of_any_alignment_and_overlap(hhl, form):
+    """Right-hand sides at an odd multiple of 8 bytes, and results laid over them: as with arrays of
+    their own, bit for bit (one path copies the inputs first, the other reads them in place)."""
+    import torch
+    probs, bs = _problems(hhl, SIZES)
+    batch = hhl.HHLBatch(probs)
+    n_b, n_out = batch.info["b_doubles"], batch.info["out_doubles"]
+    pool = torch.zeros(max(n_b, n_out) + 1, dtype=torch.float64, device="cuda")
+    b = pool[1:1 + n_b] if form == "offset" else pool[:n_b]
+    out = torch.empty(n_out, dtype=torch.float64, device="cuda") if form == "offset" else pool[:n_out]
+    eps = torch.empty(batch.count, dtype=torch.float64, device="cuda")
+    b.copy_(torch.tensor(batch.pack_rhs(bs)))
+    batch.run(b, out, eps)
+    ref, ref_eps = batch.run_host(batch.pack_rhs(bs))
+    assert np.array_equal(out.cpu().numpy(), ref) and np.array_equal(eps.cpu().numpy(), ref_eps)
+    batch.close()
