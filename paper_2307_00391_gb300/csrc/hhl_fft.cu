@@ -732,6 +732,17 @@ struct SplitGeom {
   static constexpr int MR = sizeof(T) == 8 ? 4 : 3;  // radix bits per shared-memory round trip
 };
 
+// Passes whose twiddles are read from a table (build_factors): all transforms of the double-float
+// kernels, and pass B of the complex64 ones, where the table is the same for every tile: from 5 bits
+// on (10-bit clocks; 4 bits are one group of 16, whose products the compiler rounds otherwise), with
+// sums from 6 on (12-bit clocks; at 5 the compiler rounds the terms of the sums otherwise).
+template <class R, int OP, bool WHOLE, int NB>
+constexpr bool split_tab() {
+  return !WHOLE && OP != kSplitHad &&
+         (std::is_same<R, df>::value ||
+          (sizeof(R) == 4 && ((OP == kSplitMid && NB >= 5) || (OP == kSplitMidSums && NB >= 6))));
+}
+
 // The RB radix-2 stages of one group (same arithmetic as butterflies() above), with the
 // twiddles of each stage formed once per distinct value: stage t needs 2^t factors
 // base_t * exp(-2 pi i xr / 2^(t+1)), xr < 2^t.
@@ -831,29 +842,61 @@ __device__ __forceinline__ void tile_stages(T* X, int b0, int lo_fixed, int m, c
   }
 }
 
-// The double-float passes read their twiddles from a table instead of forming them per group: a
-// complex product is about 32 FP32 operations there, and each group of 8 formed 7 factors with 7
-// products (three table look-ups, four roots) next to 12 butterflies of one product each. All lanes
-// of a warp work on the same rows, so a read is a broadcast. The stages of 2^NB rows have 2^NB - 1
-// factors in all: pass (TB, RB), in order, holds 2^RB - 1 for each value of its TB lower bits.
+// Such passes read their twiddles from a table instead of forming them per group: each group of 8
+// formed 7 factors with 7 products (three table look-ups, four roots) next to 12 butterflies of one
+// product each, and a double-float product is about 32 FP32 operations. All lanes of a warp work on
+// the same rows, so a read is a broadcast. Pass (TB, RB), in order, holds 2^RB slots for each value of
+// its TB lower bits, the factors of stage t in slots [2^t, 2^(t+1)). The complex64 products round as
+// group_butterflies' do (cmul_as): the table changes no bit of the state.
+// Bits of DIF pass q of NB in n passes; the DIT passes take the same sizes in reverse order, so the
+// last DIF pass and the first DIT one work on the same rows (tile_mid).
+__host__ __device__ constexpr int tab_bits(int NB, int n, int q) {
+  int done = 0, r = 0;
+  for (int i = 0; i <= q; ++i) {
+    r = (NB - done) / (n - i);
+    done += r;
+  }
+  return r;
+}
+template <class T, int NB>
+__host__ __device__ constexpr int tab_passes() { return (NB + SplitGeom<T>::MR - 1) / SplitGeom<T>::MR; }
+// Slots of the table, each way: 2^(bits not yet transformed) a DIF pass.
+template <class T, int NB>
+__host__ __device__ constexpr int tab_entries() {
+  int sum = 0, left = NB;
+  for (int q = 0; q < tab_passes<T, NB>(); ++q) {
+    sum += 1 << left;
+    left -= tab_bits(NB, tab_passes<T, NB>(), q);
+  }
+  return sum;
+}
+
 template <class T, int NB, bool DIT, int Q = 0, int DONE = 0, class TW>
 __device__ __forceinline__ void build_factors(T* tab, int b0, int lo_fixed, int m, const TW& tw, bool conj) {
-  constexpr int MR = SplitGeom<T>::MR;
-  constexpr int NPASS = (NB + MR - 1) / MR;
+  constexpr int NPASS = tab_passes<T, NB>();
   using R = decltype(T().x);
   if constexpr (Q < NPASS) {
-    constexpr int RB = (NB - DONE) / (NPASS - Q), TB = DIT ? DONE : NB - DONE - RB;
-    constexpr int F = (1 << RB) - 1, count = F << TB;
+    constexpr int RB = tab_bits(NB, NPASS, DIT ? NPASS - 1 - Q : Q), TB = DIT ? DONE : NB - DONE - RB;
+    constexpr int count = 1 << (RB + TB);
     for (int e = threadIdx.x; e < count; e += blockDim.x) {
-      const int lo = e / F, i = e - lo * F;
-      const int t = 31 - __clz(i + 1), xr = i + 1 - (1 << t), s = t + 1 + b0 + TB;
-      T f = tw((lo_fixed + (lo << b0)) << (m - s), conj);
+      const int lo = e >> RB, i = e & ((1 << RB) - 1);
+      if (i == 0) continue;
+      // stage p of the tile, lower index l; composed as tile_stages would in its pass from bit g0 on
+      // (its DIT passes take the sizes in the DIF order)
+      const int p = TB + 31 - __clz(i), l = lo + ((i - (1 << (p - TB))) << TB);
+      int g0 = TB;
+      if (DIT) {
+        g0 = 0;
+        for (int q = 0; q + 1 < NPASS && p >= g0 + tab_bits(NB, NPASS, q); ++q) g0 += tab_bits(NB, NPASS, q);
+      }
+      const int t = p - g0, xr = l >> g0, s = p + 1 + b0;
+      T f = tw((lo_fixed + ((l & ((1 << g0) - 1)) << b0)) << (m - s), conj);
       if (xr != 0) {
         const int k16 = xr << (3 - t);
         T w;
         w.x = root16<R>(k16, 0);
         w.y = conj ? -root16<R>(k16, 1) : root16<R>(k16, 1);
-        f = cmul(f, w);
+        f = cmul_as<true, true>(f, w);
       }
       tab[e] = f;
     }
@@ -861,43 +904,63 @@ __device__ __forceinline__ void build_factors(T* tab, int b0, int lo_fixed, int 
   }
 }
 
-// tile_stages with those factors.
-template <class T, int NB, bool DIT, int LW, bool CV, int Q = 0, int DONE = 0>
+// The RB stages of one group with the factors f.
+template <class T, int RB, bool DIT>
+__device__ __forceinline__ void group_stages_tab(T (&v)[1 << RB], const T* f) {
+  constexpr int G = 1 << RB;
+#pragma unroll
+  for (int tt = 0; tt < RB; ++tt) {
+    const int t = DIT ? tt : (RB - 1 - tt);
+    T ft[1 << (RB - 1)];
+#pragma unroll
+    for (int x = 0; x < (1 << t); ++x) {
+      if constexpr (sizeof(T) == 8) {  // two factors a read
+        if (t == 0) {
+          ft[x] = f[1];
+        } else if (x % 2 == 0) {
+          const float4 two = *reinterpret_cast<const float4*>(f + (1 << t) + x);
+          ft[x] = T{two.x, two.y};
+          ft[x + 1] = T{two.z, two.w};
+        }
+      } else {
+        ft[x] = f[(1 << t) + x];
+      }
+    }
+#pragma unroll
+    for (int x = 0; x < G; ++x) {
+      if (x & (1 << t)) continue;
+      const int x1 = x | (1 << t);
+      const T fx = ft[x & ((1 << t) - 1)];
+      const T a = v[x], b = DIT ? cmul_as<true, true>(v[x1], fx) : v[x1];
+      v[x] = cadd(a, b);
+      v[x1] = DIT ? csub(a, b) : cmul_as<true, RB != 4>(csub(a, b), fx);
+    }
+  }
+}
+
+// tile_stages with those factors: passes [Q, LAST).
+template <class T, int NB, bool DIT, int LW, bool CV, int Q = 0, int LAST = tab_passes<T, NB>(), int DONE = 0>
 __device__ __forceinline__ void tile_stages_tab(T* X, const T* tab) {
-  constexpr int MR = SplitGeom<T>::MR;
-  constexpr int NPASS = (NB + MR - 1) / MR;
-  if constexpr (Q < NPASS) {
-    constexpr int RB = (NB - DONE) / (NPASS - Q), TB = DIT ? DONE : NB - DONE - RB;
-    constexpr int W = 1 << LW, G = 1 << RB, F = G - 1;
+  constexpr int NPASS = tab_passes<T, NB>();
+  if constexpr (Q < LAST) {
+    constexpr int RB = tab_bits(NB, NPASS, DIT ? NPASS - 1 - Q : Q), TB = DIT ? DONE : NB - DONE - RB;
+    constexpr int W = 1 << LW, G = 1 << RB;
 #pragma unroll 1
     for (int g = threadIdx.x; g < (W << (NB - RB)); g += blockDim.x) {
       const int w = g & (W - 1), gg = g >> LW, lo = gg & ((1 << TB) - 1);
       T* q = X + ((((gg >> TB) << (TB + RB)) + lo) << LW) + w;
-      const T* f = tab + lo * F;
       T v[G];
 #pragma unroll
       for (int x = 0; x < G; ++x) {
         if constexpr (CV && Q == 0) v[x] = amp_in<T>(q, (long long)x << (TB + LW));
         else v[x] = q[x << (TB + LW)];
       }
-#pragma unroll
-      for (int tt = 0; tt < RB; ++tt) {
-        const int t = DIT ? tt : (RB - 1 - tt);
-#pragma unroll
-        for (int x = 0; x < G; ++x) {
-          if (x & (1 << t)) continue;
-          const int x1 = x | (1 << t);
-          const T fx = f[(1 << t) - 1 + (x & ((1 << t) - 1))];
-          const T a = v[x], b = DIT ? cmul(v[x1], fx) : v[x1];
-          v[x] = cadd(a, b);
-          v[x1] = DIT ? csub(a, b) : cmul(csub(a, b), fx);
-        }
-      }
+      group_stages_tab<T, RB, DIT>(v, tab + (lo << RB));
 #pragma unroll
       for (int x = 0; x < G; ++x) q[x << (TB + LW)] = v[x];
     }
     __syncthreads();
-    tile_stages_tab<T, NB, DIT, LW, CV, Q + 1, DONE + RB>(X, tab + (F << TB));
+    tile_stages_tab<T, NB, DIT, LW, CV, Q + 1, LAST, DONE + RB>(X, tab + (1 << (RB + TB)));
   }
 }
 
@@ -976,7 +1039,50 @@ __device__ __forceinline__ TilePos tile_pos(const SplitArgs& a, long long t) {
 
 // The work on one landed tile of a split pass (transform stages, the pass's epilogue and the
 // store back), shared by the streaming passes and the L2-staged group passes below.
-template <class R, int OP, bool FULL, int NB, bool WHOLE, bool CS = false, class TW>
+// Pass B of the full complex64 solve: inverse-QFT stages, rotation, QFT stages. The last DIF pass, the
+// rotation of its 2^RB rows and the first DIT pass stay in registers, two round trips through the
+// tile and two barriers fewer (with the factors' table, 32 qubits: 9.48 -> 9.10 ms; the table alone
+// changes nothing there). Not the form with sums: its FP32 partial sums would take their terms in
+// another order, which moves the weights by up to 1e-8 (the table alone: 9.48 -> 8.72 ms). Not the
+// double-float form, which spills (4.20 -> 4.93 ms at 28 qubits).
+template <int NB>
+__device__ __forceinline__ void tile_mid(const SplitArgs& a, const TilePos& q, float2* X, const float2* tab,
+                                         long long row_units) {
+  constexpr int LW = SplitGeom<float2>::LW, W = 1 << LW;
+  constexpr int NPASS = tab_passes<float2, NB>(), RB = tab_bits(NB, NPASS, NPASS - 1), G = 1 << RB;
+  tile_stages_tab<float2, NB, false, LW, false, 0, NPASS - 1>(X, tab);
+  const float2* dit = tab + tab_entries<float2, NB>();
+  const float2* dif = dit - G;  // the factors of the last DIF pass stand last
+  const float s = a.scale_f;
+  float2* cos_out = static_cast<float2*>(a.dst_cos) + q.base_amp;
+#pragma unroll 1
+  for (int g = threadIdx.x; g < (W << (NB - RB)); g += blockDim.x) {
+    const int w = g & (W - 1), row0 = (g >> LW) << RB;
+    float2* c = X + (row0 << LW) + w;
+    float2 v[G];
+#pragma unroll
+    for (int x = 0; x < G; ++x) v[x] = c[x << LW];
+    group_stages_tab<float2, RB, false>(v, dif);
+    const int y0 = bitrev_m(row0 + (q.hi_fixed << NB), a.m);
+#pragma unroll
+    for (int x = 0; x < G; ++x) {
+      const int y = y0 | (int)(__brev((unsigned)x) >> (32 - a.m));
+      const float2 r = static_cast<const float2*>(a.rot)[y];
+      const float2 z = float2{__fmul_rn(v[x].x, s), __fmul_rn(v[x].y, s)};
+      cos_out[(long long)y * row_units * 2 + w] = cscale(z, r.x);
+      const float f = __fmul_rn(r.y, s);  // rounded products: none is fused into the next stage's additions
+      v[x] = float2{__fmul_rn(z.x, f), __fmul_rn(z.y, f)};
+    }
+    group_stages_tab<float2, RB, true>(v, dit);
+#pragma unroll
+    for (int x = 0; x < G; ++x) c[x << LW] = v[x];
+  }
+  __syncthreads();
+  tile_stages_tab<float2, NB, true, LW, false, 1, NPASS, RB>(X, dit + G);
+}
+
+// TAB: tab holds the pass's twiddles (split_tab).
+template <class R, int OP, bool FULL, int NB, bool WHOLE, bool CS, bool TAB, class TW>
 __device__ __forceinline__ void split_tile(const SplitArgs& a, const TilePos& q, typename Cx<R>::T* X,
                                            typename Cx<R>::T* Y, const TW& tw, int mt, long long row_units,
                                            MidSums<R>* sums = nullptr, typename Cx<R>::T* tab = nullptr) {
@@ -992,19 +1098,22 @@ __device__ __forceinline__ void split_tile(const SplitArgs& a, const TilePos& q,
     else tile_stages<T, NB, true, 0>(X, a.b0, q.lo_fixed, mt, tw, false, q.inner_base, a.lo);
     tile_store<T, NB, CS>(dst, X, row_units, q.row0, a.b0, (R)1, false);
   } else if (OP == kSplitDif) {
-    if constexpr (CVT) tile_stages_tab<T, NB, false, LWT, true>(X, tab);
+    if constexpr (TAB) tile_stages_tab<T, NB, false, LWT, true>(X, tab);
     else tile_stages<T, NB, false, 0, LWT, 0, 0, CVT>(X, a.b0, q.lo_fixed, a.m, tw, false);
     tile_store<T, NB, CS>(dst, X, row_units, q.row0, a.b0, (R)1, false);
   } else if (OP == kSplitDit) {
-    if constexpr (CVT) tile_stages_tab<T, NB, true, LWT, true>(X, tab);
+    if constexpr (TAB) tile_stages_tab<T, NB, true, LWT, true>(X, tab);
     else tile_stages<T, NB, true, 0, LWT, 0, 0, CVT>(X, a.b0, q.lo_fixed, a.m, tw, true);
     tile_store<T, NB, CS>(dst, X, row_units, q.row0, a.b0, (R)1, false);
   } else if (OP == kSplitHad) {
     tile_stages<T, NB, false, 1, LWT, 0, 0, CVT>(X, a.b0, q.lo_fixed, a.m, tw, false);
     tile_store<T, NB, CS>(dst, X, row_units, q.row0, a.b0, split_scale<R>(a), a.scaled != 0);
+  } else if constexpr (TAB && !FULL && !CVT && OP == kSplitMid) {
+    tile_mid<NB>(a, q, X, tab, row_units);
+    tile_store<T, NB, CS>(dst, X, row_units, q.row0, 0, (R)1, false);
   } else {  // kSplitMid(Sums): b0 = 0, the tile holds every low bit of the rows hi_fixed << NB
     constexpr bool SUMS = OP == kSplitMidSums;
-    if constexpr (CVT) tile_stages_tab<T, NB, false, LWT, true>(X, tab);
+    if constexpr (TAB) tile_stages_tab<T, NB, false, LWT, CVT>(X, tab);
     else tile_stages<T, NB, false, 0, LWT, 0, 0, CVT>(X, 0, 0, a.m, tw, false);
     const R s = split_scale<R>(a);
     uint4* cos_out = reinterpret_cast<uint4*>(static_cast<T*>(a.dst_cos) + q.base_amp);
@@ -1038,9 +1147,9 @@ __device__ __forceinline__ void split_tile(const SplitArgs& a, const TilePos& q,
       }
     }
     __syncthreads();
-    if constexpr (CVT) {
-      tile_stages_tab<T, NB, true, LWT, false>(X, tab + (1 << NB));
-      if (FULL) tile_stages_tab<T, NB, true, LWT, false>(Y, tab + (1 << NB));
+    if constexpr (TAB) {
+      tile_stages_tab<T, NB, true, LWT, false>(X, tab + tab_entries<T, NB>());
+      if (FULL) tile_stages_tab<T, NB, true, LWT, false>(Y, tab + tab_entries<T, NB>());
     } else {
       tile_stages<T, NB, true, 0>(X, 0, 0, a.m, tw, true);
       if (FULL) tile_stages<T, NB, true, 0>(Y, 0, 0, a.m, tw, true);
@@ -1072,8 +1181,8 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitMinBlocks<R, OP>) k_split
   T* t1 = t0 + 64;
   T* Xb = t0 + (WHOLE ? 1024 : twiddle_entries(a.m));  // two tile buffers (double buffering), then Y
   T* Y = Xb + 2 * tile_amps;
-  constexpr bool TAB = is_dfc<T>() && !WHOLE && OP != kSplitHad, MID = OP == kSplitMid || OP == kSplitMidSums;
-  T* tab = Y + (MID && FULL ? tile_amps : 0);  // (double-float) twiddles of the pass, 2^NB each way
+  constexpr bool TAB = split_tab<R, OP, WHOLE, NB>(), MID = OP == kSplitMid || OP == kSplitMidSums;
+  T* tab = Y + (MID && FULL ? tile_amps : 0);  // twiddles of the pass, tab_entries each way
   if (!WHOLE && OP != kSplitHad) fill_twiddles<R>(t0, t1, a.m);
   if constexpr (WHOLE) fill_twiddle4<R>(t0, a.lo + a.m);  // first read after the barrier of the first tile
   using TW = typename std::conditional<WHOLE, Twiddle4<T>, Twiddle<T>>::type;
@@ -1101,7 +1210,7 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitMinBlocks<R, OP>) k_split
     __syncthreads();  // the two-level tables are complete
     if constexpr (MID) {
       build_factors<T, NB, false>(tab, 0, 0, a.m, tw, false);
-      build_factors<T, NB, true>(tab + (1 << NB), 0, 0, a.m, tw, true);
+      build_factors<T, NB, true>(tab + tab_entries<T, NB>(), 0, 0, a.m, tw, true);
     }
   }
   int buf = 0;
@@ -1122,7 +1231,7 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitMinBlocks<R, OP>) k_split
     }
     split_cp_async_wait1();
     __syncthreads();  // the current tile has landed for every thread
-    split_tile<R, OP, FULL, NB, WHOLE>(a, q, Xb + buf * tile_amps, Y, tw, mt, row_units, &sums, tab);
+    split_tile<R, OP, FULL, NB, WHOLE, false, TAB>(a, q, Xb + buf * tile_amps, Y, tw, mt, row_units, &sums, tab);
     __syncthreads();  // this buffer is read out before it is refilled
     buf ^= 1;
   }
@@ -1162,7 +1271,7 @@ hhl_status launch_split_nb(const SplitArgs& a, cudaStream_t st, const char* name
   using T = typename Cx<R>::T;
   const size_t tile = ((size_t)1 << (NB + SplitGeom<T>::LW)) * sizeof(T);
   const size_t smem = (size_t)(WHOLE ? 1024 : twiddle_entries(a.m)) * sizeof(T) + ((OP == kSplitMid && FULL) ? 3 : 2) * tile +
-                      (is_dfc<T>() && !WHOLE && OP != kSplitHad ? ((size_t)2 << NB) * sizeof(T) : 0);
+                      (split_tab<R, OP, WHOLE, NB>() ? 2 * (size_t)tab_entries<T, NB>() * sizeof(T) : 0);
   auto kern = k_split_pass<R, OP, FULL, NB, WHOLE>;
   HHL_CUDA_TRY(raise_dyn_smem((const void*)kern, smem));
   int dev = 0, sms = 0, occ = 0;
@@ -1247,7 +1356,7 @@ __device__ __forceinline__ void group_phase(const SplitArgs& a, long long ib, in
     split_cp_async_wait1();
     __syncthreads();  // the current tile has landed for every thread
     const TilePos q = tile_pos<NB, LW>(a, ib + (u << a.log_cb));
-    split_tile<R, OP, FULL, NB, false, CS>(a, q, Xb + buf * tile_amps, Y, tw, a.m, row_units);
+    split_tile<R, OP, FULL, NB, false, CS, false>(a, q, Xb + buf * tile_amps, Y, tw, a.m, row_units);
     __syncthreads();  // this buffer is read out before it is refilled
     buf ^= 1;
   }
