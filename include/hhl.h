@@ -193,9 +193,10 @@ uint64_t hhl_state_bytes(hhl_plan_t plan);
 
 /* a1 - amplitude encoding of b (Sec. IV.A: the right-hand side loaded as a quantum state)
  * followed by a Hadamard on every clock qubit: S[0][c][:] = b / (|b| 2^(n_c/2)),
- * S[1][:][:] = 0. b_dev: DEVICE complex128 (re, im interleaved), length N. |b| is kept
- * on the device for the dissipation readout. Error if |b| = 0 is detected later by
- * hhl_measure / hhl_dissipation (HHL_ERR_SINGULAR). */
+ * S[1][:][:] = 0. b_dev: DEVICE complex128 (re, im interleaved), length N; it may lie in the
+ * state (it is read whole before the state is written). |b| is kept on the device for the
+ * dissipation readout. Error if |b| = 0 is detected later by hhl_measure / hhl_dissipation
+ * (HHL_ERR_SINGULAR). */
 hhl_status hhl_prepare_rhs(hhl_plan_t plan, const double* b_dev, void* state_dev, void* stream);
 
 /* As hhl_prepare_rhs with b in HOST memory (b_im may be NULL for real b): copies b to

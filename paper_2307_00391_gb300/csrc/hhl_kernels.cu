@@ -751,7 +751,13 @@ hhl_status prep_small(const Plan& p, const double* b, void* state, bool row_only
 }  // namespace
 
 hhl_status launch_prep_fill(const Plan& p, const double* b, void* state, cudaStream_t st) {
-  const bool small = p.N <= kSmallN, one = small && (size_t)(2 * p.R * p.N) * p.amp_bytes() <= kPrepOneLaunch;
+  // In one launch a block may store its share of the state before another has read b, so a b that lies
+  // in the state (the clock = 0 row of the anc = 1 half is a right-hand side of a complex128 plan as it
+  // stands) takes the two-launch form: the row by one block, which reads all of b first, then the fill.
+  const size_t state_bytes = (size_t)(2 * p.R * p.N) * p.amp_bytes();
+  const char *b0 = (const char*)b, *s0 = (const char*)state;
+  const bool apart = b0 + p.N * sizeof(double2) <= s0 || s0 + state_bytes <= b0;
+  const bool small = p.N <= kSmallN, one = small && apart && state_bytes <= kPrepOneLaunch;
   if (small) {
     hhl_status s = p.prec == HHL_PREC_C64 ? prep_small<float>(p, b, one ? state : p.d_bs, !one, st)
                                           : prep_small<double>(p, b, one ? state : p.d_bs, !one, st);
