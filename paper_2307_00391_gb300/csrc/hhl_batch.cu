@@ -739,6 +739,9 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
     const int n_small = count - (int)B->large.size();
     cudaError_t e = cudaMalloc((void**)&d_gen, gen.size() * sizeof(GenInst));
     if (e == cudaSuccess) e = cudaMemcpy(d_gen, gen.data(), gen.size() * sizeof(GenInst), cudaMemcpyHostToDevice);
+    // A copy from pageable memory may return before it has reached the device, and the worker streams do
+    // not wait for the legacy stream that carries it: every table is there before the first launch.
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     for (int z = 0; z < n_small && e == cudaSuccess; z += 65535) {
       const dim3 grid((unsigned)((2 * small_n + 2 + 255) / 256), (unsigned)small_k, (unsigned)std::min(65535, n_small - z));
       k_ugen_g<<<grid, 256, small_n * sizeof(double2)>>>(d_gen + z);
