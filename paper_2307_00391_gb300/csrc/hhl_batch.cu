@@ -317,8 +317,8 @@ __global__ void __launch_bounds__(kSmallThreads, 3) k_batch_small(const SmallIns
     }
     w[1] = df_add(w[1], df(small_square(v[0], v[1]), 0.f));
   }
-  double wt[2];
-  block_sum_all_df(w, wt);
+  double ws[2] = {(double)w[0].h + (double)w[0].l, (double)w[1].h + (double)w[1].l}, wt[2];
+  block_sum_all(ws, wt);
   __syncthreads();
   // uncompute, Hadamards and postselection by halving: the table of step k is in buffer k & 1 or,
   // for the first, in the one the last expansion step loaded

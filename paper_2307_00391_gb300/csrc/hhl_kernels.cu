@@ -245,7 +245,8 @@ __device__ __forceinline__ void kahan_add(R& s, R& c, R p) {
 // Complex128 form on the FP32 pipe: the FP64 amplitudes split into double-float with integer
 // operations, |z|^2 and the running sums in double-float (about 48 significant bits per
 // partial; the block and grid totals in FP64).
-__device__ __forceinline__ void measure_thread_df(const double2* __restrict__ S, int64_t half, int64_t N, df (&a)[3]) {
+__device__ __forceinline__ void measure_thread_df(const double2* __restrict__ S, int64_t half, int64_t N,
+                                                  double (&a)[3]) {
   const int64_t units = 2 * half;
   constexpr int U = 4;  // loads in flight per thread
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -270,12 +271,12 @@ __device__ __forceinline__ void measure_thread_df(const double2* __restrict__ S,
     }
   }
 #pragma unroll
-  for (int i = 0; i < 3; ++i) a[i] = s[i];
+  for (int i = 0; i < 3; ++i) a[i] = (double)s[i].h + (double)s[i].l;
 }
 
 template <class R>
 __device__ __forceinline__ void measure_thread(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
-                                               typename std::conditional<sizeof(R) == 4, df, double>::type (&a)[3]) {
+                                               double (&a)[3]) {
   constexpr int per = 16 / sizeof(typename Cx<R>::T);  // amplitudes per 16-byte unit
   using V = typename std::conditional<sizeof(R) == 4, float4, double2>::type;
   const V* u = reinterpret_cast<const V*>(S);
@@ -311,31 +312,20 @@ __device__ __forceinline__ void measure_thread(const typename Cx<R>::T* __restri
     }
   }
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    if constexpr (sizeof(R) == 4) a[i] = df(s[i], -c[i]);
-    else a[i] = s[i] - c[i];
-  }
+  for (int i = 0; i < 3; ++i) a[i] = (double)s[i] - (double)c[i];
 }
-// The block's totals: from double-float partials (complex64, and complex128 on the FP32 pipe) or FP64.
+// The block's totals, FP64 across the threads (complex128 with DF: from double-float partials).
 template <class R, bool DF>
 __device__ __forceinline__ void measure_block(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
                                               double (&t)[3]) {
-  if constexpr (DF) {
-    df a[3];
-    measure_thread_df(S, half, N, a);
-    block_sum_all_df(a, t);
-  } else if constexpr (sizeof(R) == 4) {
-    df a[3];
-    measure_thread<R>(S, half, N, a);
-    block_sum_all_df(a, t);
-  } else {
-    double a[3];
-    measure_thread<R>(S, half, N, a);
-    block_sum_all(a, t);
-  }
+  double a[3];
+  if constexpr (DF) measure_thread_df(S, half, N, a);
+  else measure_thread<R>(S, half, N, a);
+  block_sum_staged<3, kThreads>(a, t);
 }
 template <class R, bool DF>
-__global__ void k_measure_sums(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N, double* acc) {
+__global__ void __launch_bounds__(kThreads) k_measure_sums(const typename Cx<R>::T* __restrict__ S, int64_t half,
+                                                           int64_t N, double* acc) {
   dep_begin();
   double t[3];
   measure_block<R, DF>(S, half, N, t);
