@@ -52,6 +52,10 @@ void prof_end(const char* name);
 // tail (a solve of 59 launches: 456 -> 316 us). Every such kernel calls dep_wait() in all its threads before it
 // touches global memory: that returns when the kernel before it, and so by induction everything
 // before that, has completed and its writes are visible. dep_launch() lets the next one in.
+// Such a kernel is resident while the one before it writes, so none of its operands that an earlier launch
+// may write (the state, b, scratch rows, scalars) is `const __restrict__`: that promises data unchanged
+// over the kernel's whole lifetime, and lets the compiler use non-coherent loads and move them across
+// dep_wait(). Tables made at plan or batch creation keep the qualifiers.
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_begin() {

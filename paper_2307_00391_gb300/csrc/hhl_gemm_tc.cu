@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
 // the contributors' partials in CTA order (the same sum on every run), scales by 2^-30 and
 // writes (or adds to) the state row. Tiles held whole by one CTA were written by the GEMM.
 template <int BN>
-__global__ void __launch_bounds__(256) k_tc_fixup(const float4* __restrict__ ws, float* __restrict__ state_half,
+__global__ void __launch_bounds__(256) k_tc_fixup(const float4* ws, float* __restrict__ state_half,
                                                   int n_s, RowMap rows, int k_iters, int tiles_n, int64_t units,
                                                   int64_t G, int* err, const TcNext nx) {
   dep_begin();
@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(256) k_tc_fixup(const float4* __restrict__ ws,
 // The mapped rows (those with clock bit k set, or a tree step's source rows) -> compact FP16
 // hi / lo arrays (M_sub x 2N), scaled by 2^15.
 // An amplitude component of magnitude >= 2 cannot be represented: error flag 4.
-__global__ void k_tc_split_rows(const float4* __restrict__ half, uint2* __restrict__ a_hi, uint2* __restrict__ a_lo,
+__global__ void k_tc_split_rows(const float4* half, uint2* __restrict__ a_hi, uint2* __restrict__ a_lo,
                                 int n_s, RowMap rows, int64_t m_sub, int* err) {
   dep_begin();
   const int row4_bits = n_s - 1;  // float4 per row = 2N/4 = 2^(n_s-1)

@@ -58,7 +58,7 @@ __device__ __forceinline__ int64_t row_with_bit(int64_t i, int k) {
 
 // ------------------------------------------------------------------------------ prep
 
-__global__ void k_bnorm(const double2* __restrict__ b, int64_t n, double* acc) {
+__global__ void k_bnorm(const double2* b, int64_t n, double* acc) {
   dep_begin();
   double s[1] = {0.0};
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -70,7 +70,7 @@ __global__ void k_bnorm(const double2* __restrict__ b, int64_t n, double* acc) {
 
 // bs = b / (|b| 2^(n_c/2)) in the amplitude precision (one row of the anc = 0 half).
 template <class R>
-__global__ void k_prep_scale(const double2* __restrict__ b, const double* __restrict__ acc,
+__global__ void k_prep_scale(const double2* b, const double* acc,
                              typename Cx<R>::T* __restrict__ bs, int64_t N, int n_c) {
   dep_begin();
   const double nb2 = acc[0];
@@ -82,7 +82,7 @@ __global__ void k_prep_scale(const double2* __restrict__ b, const double* __rest
 }
 
 // Every clock row of the anc = 0 half gets bs, the anc = 1 half is zeroed: 16-byte stores.
-__global__ void k_prep_fill(const uint4* __restrict__ bs, uint4* __restrict__ st, int64_t row_units,
+__global__ void k_prep_fill(const uint4* bs, uint4* __restrict__ st, int64_t row_units,
                             int64_t half_units) {
   dep_begin();
   const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
@@ -98,7 +98,7 @@ __global__ void k_prep_fill(const uint4* __restrict__ bs, uint4* __restrict__ st
 constexpr int kSmallN = 1024;
 constexpr size_t kPrepOneLaunch = 4 << 20;  // larger states: the row by one block, then the fill over all SMs
 template <class R>
-__global__ void __launch_bounds__(kThreads) k_prep_small(const double2* __restrict__ b, int N, int n_c,
+__global__ void __launch_bounds__(kThreads) k_prep_small(const double2* b, int N, int n_c,
                                                          double* __restrict__ scal, uint4* __restrict__ st,
                                                          int64_t half_units, int row_only) {
   dep_begin();
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(kThreads) k_prep_small(const double2* __restri
 template <class R, int BM, int BN, int BK, bool INPLACE>
 __global__ void __launch_bounds__(256) k_ctrl_gemm_simt(typename Cx<R>::T* S,
                                                         typename Cx<R>::T* __restrict__ out,
-                                                        const typename Cx<R>::T* __restrict__ B,
+                                                        const typename Cx<R>::T* B,
                                                         int n_s, RowMap rows, int64_t m_sub) {
   dep_begin();
   using T = typename Cx<R>::T;
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(256) k_ctrl_gemm_simt(typename Cx<R>::T* S,
 // S[row(i)][:] = out[i][:] (the rows with clock bit k set, or a tree's mapped rows, where the
 // reduction adds out[i][:] to the row and its last step scales the sum).
 template <class R>
-__global__ void k_rows_scatter(typename Cx<R>::T* __restrict__ S, const typename Cx<R>::T* __restrict__ out,
+__global__ void k_rows_scatter(typename Cx<R>::T* __restrict__ S, const typename Cx<R>::T* out,
                                int n_s, RowMap rows, int64_t m_sub) {
   dep_begin();
   const int64_t N = 1LL << n_s;
@@ -245,7 +245,7 @@ __device__ __forceinline__ void kahan_add(R& s, R& c, R p) {
 // Complex128 form on the FP32 pipe: the FP64 amplitudes split into double-float with integer
 // operations, |z|^2 and the running sums in double-float (about 48 significant bits per
 // partial; the block and grid totals in FP64).
-__device__ __forceinline__ void measure_thread_df(const double2* __restrict__ S, int64_t half, int64_t N,
+__device__ __forceinline__ void measure_thread_df(const double2* S, int64_t half, int64_t N,
                                                   double (&a)[3]) {
   const int64_t units = 2 * half;
   constexpr int U = 4;  // loads in flight per thread
@@ -275,7 +275,7 @@ __device__ __forceinline__ void measure_thread_df(const double2* __restrict__ S,
 }
 
 template <class R>
-__device__ __forceinline__ void measure_thread(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
+__device__ __forceinline__ void measure_thread(const typename Cx<R>::T* S, int64_t half, int64_t N,
                                                double (&a)[3]) {
   constexpr int per = 16 / sizeof(typename Cx<R>::T);  // amplitudes per 16-byte unit
   using V = typename std::conditional<sizeof(R) == 4, float4, double2>::type;
@@ -316,7 +316,7 @@ __device__ __forceinline__ void measure_thread(const typename Cx<R>::T* __restri
 }
 // The block's totals, FP64 across the threads (complex128 with DF: from double-float partials).
 template <class R, bool DF>
-__device__ __forceinline__ void measure_block(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
+__device__ __forceinline__ void measure_block(const typename Cx<R>::T* S, int64_t half, int64_t N,
                                               double (&t)[3]) {
   double a[3];
   if constexpr (DF) measure_thread_df(S, half, N, a);
@@ -324,7 +324,7 @@ __device__ __forceinline__ void measure_block(const typename Cx<R>::T* __restric
   block_sum_staged<3, kThreads>(a, t);
 }
 template <class R, bool DF>
-__global__ void __launch_bounds__(kThreads) k_measure_sums(const typename Cx<R>::T* __restrict__ S, int64_t half,
+__global__ void __launch_bounds__(kThreads) k_measure_sums(const typename Cx<R>::T* S, int64_t half,
                                                            int64_t N, double* acc) {
   dep_begin();
   double t[3];
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kThreads) k_measure_sums(const typename Cx<R>:
 
 // out = [p_success, p_anc1, norm, |b|, xhat] by one block from the totals (w0, w1, |v|^2).
 template <class R>
-__device__ void measure_write(const typename Cx<R>::T* __restrict__ v, int64_t N, double w0, double w1, double ps,
+__device__ void measure_write(const typename Cx<R>::T* v, int64_t N, double w0, double w1, double ps,
                               double nb2, double* __restrict__ out) {
   if (threadIdx.x == 0) {
     out[0] = ps;
@@ -355,7 +355,7 @@ __device__ void measure_write(const typename Cx<R>::T* __restrict__ v, int64_t N
 // ticket adds them in block order (the same total on every run), writes the block and returns
 // the ticket counter to zero. Saves a memset and a launch, which bound such states.
 template <class R, bool DF>
-__global__ void __launch_bounds__(kThreads) k_measure_small(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
+__global__ void __launch_bounds__(kThreads) k_measure_small(const typename Cx<R>::T* S, int64_t half, int64_t N,
                                                             double* __restrict__ scal, double* __restrict__ part,
                                                             unsigned* __restrict__ ticket, double* __restrict__ out) {
   dep_begin();
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(kThreads) k_measure_small(const typename Cx<R>
 // The postselected row's norm and the measurement block from the weights already in scal[1..2]
 // (one block; at most kSmallN points).
 template <class R>
-__global__ void __launch_bounds__(kThreads) k_row_finish_small(const typename Cx<R>::T* __restrict__ v, int64_t N,
+__global__ void __launch_bounds__(kThreads) k_row_finish_small(const typename Cx<R>::T* v, int64_t N,
                                                                double* __restrict__ scal, double* __restrict__ out) {
   dep_begin();
   double s[1] = {0.0}, t[1];
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(kThreads) k_row_finish_small(const typename Cx
 
 // |v|^2 of one row of N amplitudes (the postselected row), FP64.
 template <class R>
-__global__ void k_row_norm(const typename Cx<R>::T* __restrict__ v, int64_t N, double* acc) {
+__global__ void k_row_norm(const typename Cx<R>::T* v, int64_t N, double* acc) {
   dep_begin();
   double s[1] = {0.0};
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x) {
@@ -411,8 +411,8 @@ __global__ void k_row_norm(const typename Cx<R>::T* __restrict__ v, int64_t N, d
 
 // out = [p_success, p_anc1, norm, |b|, xhat (2N doubles)]
 template <class R>
-__global__ void k_measure_finish(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
-                                 const double* __restrict__ scal, double* __restrict__ out) {
+__global__ void k_measure_finish(const typename Cx<R>::T* S, int64_t half, int64_t N,
+                                 const double* scal, double* __restrict__ out) {
   dep_begin();
   const double ps = scal[3];
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -571,8 +571,8 @@ __global__ void k_sample_bins(const double* __restrict__ cdf, int64_t N, const d
 
 // Dissipation: sum over the N+1 cells of (u_{i+1} - u_i)^2 with walls at both ends.
 template <class R>
-__global__ void k_diss_sum(const typename Cx<R>::T* __restrict__ S, int64_t half, int64_t N,
-                           const double* __restrict__ scal, double inv_c_lam, double wlo, double whi,
+__global__ void k_diss_sum(const typename Cx<R>::T* S, int64_t half, int64_t N,
+                           const double* scal, double inv_c_lam, double wlo, double whi,
                            double* acc, double* __restrict__ u_out) {
   dep_begin();
   const double scale = sqrt(scal[0]) * inv_c_lam;
@@ -589,7 +589,7 @@ __global__ void k_diss_sum(const typename Cx<R>::T* __restrict__ S, int64_t half
 
 // The whole read-out by one block (at most kSmallN points): no memset, no second launch.
 template <class R>
-__global__ void __launch_bounds__(kThreads) k_diss_small(const typename Cx<R>::T* __restrict__ v, int N,
+__global__ void __launch_bounds__(kThreads) k_diss_small(const typename Cx<R>::T* v, int N,
                                                          double* __restrict__ scal, double inv_c_lam, double wlo, double whi,
                                                          double nu_over_h, double* __restrict__ eps,
                                                          double* __restrict__ u_out) {
@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(kThreads) k_diss_small(const typename Cx<R>::T
   }
 }
 
-__global__ void k_diss_finish(const double* __restrict__ acc, double nu_over_h, double* eps) {
+__global__ void k_diss_finish(const double* acc, double nu_over_h, double* eps) {
   dep_begin();
   if (threadIdx.x == 0 && blockIdx.x == 0) eps[0] = nu_over_h * acc[0];
 }

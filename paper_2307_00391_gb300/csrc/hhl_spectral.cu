@@ -153,7 +153,7 @@ hhl_status spec_rows(double2* X, const double* B, int N, long long rows, cudaStr
 
 // ------------------------------------------------------------------ the postselected solve
 // |b|^2 and bhat = b / |b|; one block.
-__global__ void __launch_bounds__(kSpecThreads) k_spec_prep(const double2* __restrict__ b, int N,
+__global__ void __launch_bounds__(kSpecThreads) k_spec_prep(const double2* b, int N,
                                                             double* __restrict__ scal, double2* __restrict__ x) {
   dep_begin();
   double s[1] = {0.0}, nb2[1];
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kSpecThreads) k_spec_prep(const double2* __res
 
 // y = B^T x, B N x N row-major: a block takes 8 outputs and splits the sum over its 32 groups of
 // 8 threads, whose partial sums are added in a fixed order.
-__global__ void __launch_bounds__(kSpecThreads) k_spec_matvec(const double* __restrict__ B, const double2* __restrict__ x,
+__global__ void __launch_bounds__(kSpecThreads) k_spec_matvec(const double* __restrict__ B, const double2* x,
                                                               int N, double2* __restrict__ y) {
   dep_begin();
   __shared__ double2 part[kSpecThreads / 32][8];
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kClockThreads) k_spec_tree(const unsigned long
 // The measurement block and the dissipation rate (layout of hhl_measure_async /
 // hhl_dissipation_async). Every block forms |v|^2 itself and writes its share of xhat; block 0 writes
 // the scalars.
-__global__ void __launch_bounds__(kSpecThreads) k_spec_finish(const double2* __restrict__ v, const double2* __restrict__ wts,
+__global__ void __launch_bounds__(kSpecThreads) k_spec_finish(const double2* v, const double2* wts,
                                                               int N, double* __restrict__ scal, double inv_c_lam,
                                                               double wall_lo, double wall_hi, double nu_over_h,
                                                               double* __restrict__ out, double* __restrict__ eps) {
