@@ -352,8 +352,10 @@ __device__ void measure_write(const typename Cx<R>::T* v, int64_t N, double w0, 
 
 // Systems of at most kSmallN points: the sums over the state and the measurement block in one
 // launch. Every block leaves its three partial sums in `part`; the block that draws the last
-// ticket adds them in block order (the same total on every run), writes the block and returns
-// the ticket counter to zero. Saves a memset and a launch, which bound such states.
+// ticket adds them in block order (the same total on every run) and writes the block. The counter
+// wraps to zero by itself, also where two streams measure with one plan at the same time: their
+// results may then be mixed, as ever, but later calls are whole. Saves a memset and a launch, which
+// bound such states.
 template <class R, bool DF>
 __global__ void __launch_bounds__(kThreads) k_measure_small(const typename Cx<R>::T* S, int64_t half, int64_t N,
                                                             double* __restrict__ scal, double* __restrict__ part,
@@ -365,7 +367,7 @@ __global__ void __launch_bounds__(kThreads) k_measure_small(const typename Cx<R>
   if (threadIdx.x == 0) {
     for (int i = 0; i < 3; ++i) part[3 * blockIdx.x + i] = t[i];
     __threadfence();
-    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
   }
   __syncthreads();
   if (!last) return;
@@ -376,7 +378,6 @@ __global__ void __launch_bounds__(kThreads) k_measure_small(const typename Cx<R>
   block_sum_all(a, t);
   if (threadIdx.x == 0) {
     for (int i = 0; i < 3; ++i) scal[1 + i] = t[i];
-    *ticket = 0;
   }
   measure_write<R>(S + half, N, t[0], t[1], t[2], scal[0], out);
 }
