@@ -372,17 +372,18 @@ hhl_status hhl_dissipation(hhl_plan_t plan, const void* state_dev, double* eps_o
  * instance (an O(N^2) FP64 kernel per k, kept on the device as double-float pairs), and each
  * run generates U_k from them on the fly (tree steps below 128 rows) or expands it into a
  * per-stream GEMM operand right before its product. Instances with n_c <= 7, N <= 128 and the CUDA-core
- * GEMM are solved by one thread block each, in a few launches beside the graph (the same
- * arithmetic); a batch of only such instances has no graph. */
+ * GEMM are solved by one thread block or one cluster of them each, in one or two launches that run
+ * beside the others in the graph (the same arithmetic; up to two instances of 7 + 7 qubits in a
+ * batch of at most two are launches of the graph too); a batch of only such instances has no graph. */
 typedef struct hhl_batch_s* hhl_batch_t;
 
 typedef struct hhl_batch_info {
   int32_t count;            /* instances */
-  int32_t streams;          /* worker streams of the graph (none busy with one-block solves) */
+  int32_t streams;          /* worker streams asked for (one-block solves occupy none) */
   uint64_t state_bytes;     /* all instance states (device) */
   uint64_t workspace_bytes; /* per-stream operand and row buffers (device) */
   double gemm_flops;        /* algorithmic flops of all controlled products of one run */
-  uint64_t graph_launches;  /* kernels of one run: the graph's and the one-block solves' (0 before the first run) */
+  uint64_t graph_launches;  /* kernels of one run (0 before the first) */
   int64_t b_doubles;        /* length of the packed right-hand-side array */
   int64_t out_doubles;      /* length of the packed measurement array */
 } hhl_batch_info;

@@ -32,9 +32,12 @@
 #include <numeric>
 #include <vector>
 
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
 #include "hhl_fft_core.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace hhl {
 namespace {
@@ -129,7 +132,13 @@ __global__ void k_ugen_embed_simt(int n_s, const float4* __restrict__ g, int adj
 // Instances whose clock and system registers fit one block's shared memory (n_c <= 7, N <= 128): the
 // whole postselected solve in one launch for all of them, a block each, instead of about 17
 // launches per instance (384 instances of 2^3..2^6 points: 6,900 launches of 0.6 us each on 8
-// streams, 3.95 ms; one launch takes 125 us). Bound by the latency of the 2 n_c dependent products. The
+// streams, 3.95 ms; one launch takes 85 us). Bound by issue within an SM and the latency of the 2 n_c
+// dependent products: a block takes 21 us at 4 + 4 qubits and 360 us at 7 + 7, where the launches on eight
+// streams took 79 us for one instance, 109 for 8 and 192 for 16. So while there are few, a
+// cluster of up to 8 blocks shares an instance: 7 + 7 qubits 89 us for up to 8 instances, 120 for
+// 16 and 32, 190 for 64 (the streams 360 and 697); 6 + 6 qubits 45 us up to 32 (84 by one block, the
+// streams 72 to 297). In a batch with larger instances these launches are a branch of its graph (8 of
+// 8 + 8 qubits with 16 of 7 + 7: 344 us; after the graph, a block each, 766). The
 // arithmetic is that of the launches it replaces, operation for operation: U_k from its g table,
 // every output of a product as 32 partial sums over m (mod 32) added in the order of
 // k_toeplitz_rows' shuffles and warps, the transform stages of k_clock_block, the squares of
@@ -145,6 +154,8 @@ struct SmallInst {
 
 constexpr int kSmallBits = 7;       // n_s and n_c at most
 constexpr int kSmallThreads = 256;
+constexpr int kSmallColumns = 16;   // system columns of a block at least, where a cluster shares an instance
+constexpr int kSmallCluster = 8;    // blocks of a cluster at most
 
 __host__ __device__ constexpr int small_column(int n_c) { return (1 << n_c) + (1 << n_c) / 16 + 1; }
 size_t small_smem(int n_s, int n_c) {
@@ -182,6 +193,11 @@ __device__ __forceinline__ void small_parts(const float2* __restrict__ X, int Lp
   for (int r = 0; r < RB; ++r) y[r] = cadd(cadd(a[0][r], a[1][r]), cadd(a[2][r], a[3][r]));
 }
 
+// The system columns [n0, n0 + 2^wb) that this block computes.
+struct SmallSlice {
+  int n0, wb;
+};
+
 __device__ __forceinline__ void small_store(float2* X, int Lp, int n, int row, float2 y, bool accumulate, float scale,
                                             bool scaled) {
   float2* d = X + n * Lp + pad16(row);
@@ -196,18 +212,20 @@ __device__ __forceinline__ void small_store(float2* X, int Lp, int n, int row, f
   *d = y;
 }
 
-// m output rows from out0 on, each U (or U^dagger) applied to its row from in0 on: a thread takes RB
-// rows of one column; while those are fewer than the block's threads, eight threads share them (the
-// parts of one warp each) and add their sums in the order of the warps.
+// m output rows from out0 on, each U (or U^dagger) applied to its row from in0 on, the slice's columns: a
+// thread takes RB rows of one column; while those are fewer than the block's threads, eight threads share
+// them (the parts of one warp each) and add their sums in the order of the warps.
 template <int RB>
-__device__ __forceinline__ void small_rows(float2* X, int Lp, const float4* __restrict__ g, int n_s, int m, int in0, int out0,
-                                           bool adjoint, bool accumulate, float scale, bool scaled) {
-  const int N = 1 << n_s, items = (m / RB) << n_s;
+__device__ __forceinline__ void small_rows(float2* X, int Lp, const float4* __restrict__ g, int N, SmallSlice sl, int m,
+                                           int in0, int out0, bool adjoint, bool accumulate, float scale, bool scaled) {
+  const int W = 1 << sl.wb, items = (m / RB) << sl.wb;
   float2 y[RB], p[RB];
   if (items < kSmallThreads) {
-    const int w8 = threadIdx.x & 7, base = threadIdx.x & 24;
+    // (a lane's neighbours take neighbouring columns: eight lanes then read 128 consecutive bytes of g, where
+    // eight parts of one column lie 64 bytes apart and conflict four ways; 384 small instances 125 -> 85 us)
+    const int w8 = (threadIdx.x >> 2) & 7, base = threadIdx.x & 3, mine = (threadIdx.x >> 5) * 4 + base;
     for (int i0 = 0; i0 < items; i0 += kSmallThreads / 8) {  // (whole warps take part in the shuffles)
-      const int it = i0 + (threadIdx.x >> 3), n = it & (N - 1), r = (it >> n_s) * RB;
+      const int it = i0 + mine, n = sl.n0 + (it & (W - 1)), r = (it >> sl.wb) * RB;
 #pragma unroll
       for (int q = 0; q < RB; ++q) p[q] = make_float2(0.f, 0.f);
       if (it < items && 4 * w8 < N) small_parts<RB>(X, Lp, g, N, n, in0 + r, w8, adjoint, p);
@@ -217,8 +235,8 @@ __device__ __forceinline__ void small_rows(float2* X, int Lp, const float4* __re
       for (int w = 1; w < 8; ++w) {
 #pragma unroll
         for (int q = 0; q < RB; ++q) {
-          y[q].x += __shfl_sync(0xffffffffu, p[q].x, base + w);
-          y[q].y += __shfl_sync(0xffffffffu, p[q].y, base + w);
+          y[q].x += __shfl_sync(0xffffffffu, p[q].x, base + 4 * w);
+          y[q].y += __shfl_sync(0xffffffffu, p[q].y, base + 4 * w);
         }
       }
       if (it < items && w8 == 0) {
@@ -228,7 +246,7 @@ __device__ __forceinline__ void small_rows(float2* X, int Lp, const float4* __re
     }
   } else {
     for (int it = threadIdx.x; it < items; it += kSmallThreads) {
-      const int n = it & (N - 1), r = (it >> n_s) * RB;
+      const int n = sl.n0 + (it & (W - 1)), r = (it >> sl.wb) * RB;
       small_parts<RB>(X, Lp, g, N, n, in0 + r, 0, adjoint, y);
       for (int w = 1; 4 * w < N && w < 8; ++w) {
         small_parts<RB>(X, Lp, g, N, n, in0 + r, w, adjoint, p);
@@ -241,27 +259,54 @@ __device__ __forceinline__ void small_rows(float2* X, int Lp, const float4* __re
   }
 }
 
-__device__ void small_product(float2* X, int Lp, const float4* __restrict__ g, int n_s, int m, int in0, int out0,
+__device__ void small_product(float2* X, int Lp, const float4* __restrict__ g, int N, SmallSlice sl, int m, int in0, int out0,
                               bool adjoint, bool accumulate, float scale, bool scaled) {
-  if (m >= 4) small_rows<4>(X, Lp, g, n_s, m, in0, out0, adjoint, accumulate, scale, scaled);
-  else if (m == 2) small_rows<2>(X, Lp, g, n_s, m, in0, out0, adjoint, accumulate, scale, scaled);
-  else small_rows<1>(X, Lp, g, n_s, m, in0, out0, adjoint, accumulate, scale, scaled);
+  if (m >= 4) small_rows<4>(X, Lp, g, N, sl, m, in0, out0, adjoint, accumulate, scale, scaled);
+  else if (m == 2) small_rows<2>(X, Lp, g, N, sl, m, in0, out0, adjoint, accumulate, scale, scaled);
+  else small_rows<1>(X, Lp, g, N, sl, m, in0, out0, adjoint, accumulate, scale, scaled);
 }
 
 __device__ __forceinline__ float small_square(float2 a, float2 b) {
   return fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(b.x, b.x, b.y * b.y)));
 }
 
-__global__ void __launch_bounds__(kSmallThreads, 3) k_batch_small(const SmallInst* __restrict__ inst,
-                                                               const double* __restrict__ b_all, double* __restrict__ b_copy,
-                                                               double* __restrict__ out_all, double* __restrict__ eps) {
-  extern __shared__ __align__(16) unsigned char small_raw[];
-  const SmallInst d = inst[blockIdx.x];
+// The other blocks' columns of rows [row0, row0 + 2^lr) into this block's copy of the state.
+__device__ __forceinline__ void small_pull(float2* X, int Lp, int N, SmallSlice sl, int row0, int lr) {
+  const int W = 1 << sl.wb, total = (N - W) << lr;
+  constexpr int U = 4;  // loads in flight per thread
+  for (int e0 = threadIdx.x; e0 < total; e0 += U * kSmallThreads) {
+    float2 v[U];
+    float2* d[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const int e = e0 + q * kSmallThreads;
+      if (e >= total) break;
+      const int other = e >> lr, n = other < sl.n0 ? other : other + W;
+      d[q] = X + n * Lp + pad16(row0 + (e & ((1 << lr) - 1)));
+      v[q] = *cg::this_cluster().map_shared_rank(d[q], n >> sl.wb);
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      if (e0 + q * kSmallThreads < total) *d[q] = v[q];
+  }
+}
+
+// One solve, by one block (c = 1) or, with CL, by the first c blocks of a cluster, each of which computes
+// N / c system columns and reads the rows that its next product needs from the others through distributed
+// shared memory, after the cluster's barrier. Such rows are never written again: an expansion's output
+// rows are new, and a reduction's are read only once nothing more is added to them.
+template <bool CL>
+__device__ __forceinline__ void small_solve(const SmallInst& d, int c, int rank, unsigned char* small_raw,
+                                            const double* __restrict__ b_all, double* __restrict__ b_copy,
+                                            double* __restrict__ out_all, double* __restrict__ eps) {
+  __shared__ double weights[kSmallCluster][2];  // block 0 of a cluster: the blocks' weights
   const int N = 1 << d.n_s, L = 1 << d.n_c, m = d.n_c, Lp = small_column(d.n_c), M = 2 * N + 2;
   float4* gk = reinterpret_cast<float4*>(small_raw);  // two tables: the next step's loads under this one
   float2* t0 = reinterpret_cast<float2*>(gk + 2 * M);
   float2* t1 = t0 + 64;
   float2* X = t0 + twiddle_entries(m);
+  const int W = N / c;
+  const SmallSlice sl{rank * W, 31 - __clz(W)};
   const double2* b = reinterpret_cast<const double2*>(b_all + d.b_off);
   auto load_g = [&](int k, int buf) {
     for (int q = threadIdx.x; q < M; q += kSmallThreads) gk[buf * M + q] = d.g[(size_t)k * M + q];
@@ -274,60 +319,84 @@ __global__ void __launch_bounds__(kSmallThreads, 3) k_batch_small(const SmallIns
   if (threadIdx.x < N) {
     z = b[threadIdx.x];
     s[0] = z.x * z.x + z.y * z.y;
-    if (b_copy != nullptr) reinterpret_cast<double2*>(b_copy + d.b_off)[threadIdx.x] = z;
+    if (b_copy != nullptr && rank == 0) reinterpret_cast<double2*>(b_copy + d.b_off)[threadIdx.x] = z;
   }
   block_sum_all(s, nb2);
   const double scale = nb2[0] > 0.0 ? 1.0 / sqrt(nb2[0] * (double)L) : 0.0;
   if (threadIdx.x < N) X[threadIdx.x * Lp] = make_float2((float)(z.x * scale), (float)(z.y * scale));
   __syncthreads();
+  if constexpr (CL) cg::this_cluster().sync();  // every block runs: its shared memory may be used
   // QPE by doubling
   for (int k = 0; k < m; ++k) {
     load_g(k + 1 < m ? k + 1 : m - 1, (k + 1) & 1);  // (the last load is the first reduction step's)
-    small_product(X, Lp, gk + (k & 1) * M, d.n_s, 1 << k, 0, 1 << k, false, false, 1.f, false);
+    small_product(X, Lp, gk + (k & 1) * M, N, sl, 1 << k, 0, 1 << k, false, false, 1.f, false);
+    if constexpr (CL) {  // (the clock block needs this block's columns only, and overwrites what others read)
+      cg::this_cluster().sync();
+      if (k + 1 < m) small_pull(X, Lp, N, sl, 1 << k, k);
+    }
     __syncthreads();
   }
   // inverse QFT, rotation (the anc = 0 half is only weighed), QFT
   const Twiddle<float2> tw{t0, t1};
-  local_stages<float2, false, 0, true>(X, Lp, N, tw, m, m, false);
+  float2* Xs = X + sl.n0 * Lp;
+  local_stages<float2, false, 0, true>(Xs, Lp, W, tw, m, m, false);
   const float inv = (float)(1.0 / sqrt((double)L));
   df w[2] = {df(0), df(0)};
-  for (int u = threadIdx.x; u < L * (N / 2); u += kSmallThreads) {
+  for (int u = threadIdx.x; u < L * (W / 2); u += kSmallThreads) {
     const int p = u & (L - 1), j = (u >> m) * 2;
     const float2 r = d.rot[bitrev_m(p, m)];
     float2 kt[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int idx = (j + q) * Lp + pad16(p);
-      const float2 x = cscale(X[idx], inv);
+      const float2 x = cscale(Xs[idx], inv);
       kt[q] = cscale(x, r.x);
-      X[idx] = cscale(x, r.y);
+      Xs[idx] = cscale(x, r.y);
     }
     w[0] = df_add(w[0], df(small_square(kt[0], kt[1]), 0.f));
   }
   __syncthreads();
-  local_stages<float2, true, 0, true>(X, Lp, N, tw, m, m, true);
-  for (int u = threadIdx.x; u < L * (N / 2); u += kSmallThreads) {
+  local_stages<float2, true, 0, true>(Xs, Lp, W, tw, m, m, true);
+  for (int u = threadIdx.x; u < L * (W / 2); u += kSmallThreads) {
     const int p = u & (L - 1), j = (u >> m) * 2;
     float2 v[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int idx = (j + q) * Lp + pad16(p);
-      v[q] = cscale(X[idx], inv);
-      X[idx] = v[q];
+      v[q] = cscale(Xs[idx], inv);
+      Xs[idx] = v[q];
     }
     w[1] = df_add(w[1], df(small_square(v[0], v[1]), 0.f));
   }
   double ws[2] = {(double)w[0].h + (double)w[0].l, (double)w[1].h + (double)w[1].l}, wt[2];
   block_sum_all(ws, wt);
+  if constexpr (CL) {
+    if (threadIdx.x < 2) *cg::this_cluster().map_shared_rank(&weights[rank][threadIdx.x], 0) = threadIdx.x ? wt[1] : wt[0];
+    cg::this_cluster().sync();
+    small_pull(X, Lp, N, sl, L / 2, m - 1);
+  }
   __syncthreads();
   // uncompute, Hadamards and postselection by halving: the table of step k is in buffer k & 1 or,
   // for the first, in the one the last expansion step loaded
   int buf = m & 1;
   for (int k = m - 1; k >= 0; --k) {
     if (k > 0) load_g(k - 1, buf ^ 1);
-    small_product(X, Lp, gk + buf * M, d.n_s, 1 << k, 1 << k, 0, true, true, inv, k == 0);
+    small_product(X, Lp, gk + buf * M, N, sl, 1 << k, 1 << k, 0, true, true, inv, k == 0);
+    if constexpr (CL) {  // the next step's rows [2^(k-1), 2^k), at the end row 0
+      cg::this_cluster().sync();
+      if (k > 0 || rank == 0) small_pull(X, Lp, N, sl, k > 0 ? 1 << (k - 1) : 0, k > 0 ? k - 1 : 0);
+    }
     __syncthreads();
     buf ^= 1;
+  }
+  if constexpr (CL) {
+    cg::this_cluster().sync();  // block 0 has read the others' row 0
+    if (rank > 0) return;
+    wt[0] = wt[1] = 0.0;
+    for (int q = 0; q < c; ++q) {
+      wt[0] += weights[q][0];
+      wt[1] += weights[q][1];
+    }
   }
   // the measurement block and the dissipation rate
   double a[2] = {0.0, 0.0}, t[2];
@@ -357,9 +426,31 @@ __global__ void __launch_bounds__(kSmallThreads, 3) k_batch_small(const SmallIns
   }
 }
 
+template <bool CL>
+__global__ void __launch_bounds__(kSmallThreads, CL ? 1 : 3) k_batch_small(const SmallInst* __restrict__ inst,
+                                                                       const double* __restrict__ b_all,
+                                                                       double* __restrict__ b_copy,
+                                                                       double* __restrict__ out_all, double* __restrict__ eps) {
+  extern __shared__ __align__(16) unsigned char small_raw[];
+  if constexpr (CL) {
+    const int size = (int)cg::this_cluster().num_blocks(), rank = (int)cg::this_cluster().block_rank();
+    const SmallInst d = inst[blockIdx.x / size];
+    const int most = (1 << d.n_s) / kSmallColumns, c = most < size ? most : size;
+    if (c > 1) {  // (blocks beyond c leave: the cluster's barrier counts those that have not)
+      if (rank < c) small_solve<true>(d, c, rank, small_raw, b_all, b_copy, out_all, eps);
+    } else if (rank == 0) {
+      small_solve<false>(d, 1, 0, small_raw, b_all, b_copy, out_all, eps);
+    }
+  } else {
+    small_solve<false>(inst[blockIdx.x], 1, 0, small_raw, b_all, b_copy, out_all, eps);
+  }
+}
+
 struct SmallClass {  // instances of similar shared-memory need: one launch
   int first = 0, count = 0;
   size_t smem = 0;
+  int max_n = 0;    // points of the largest
+  int cluster = 1;  // blocks an instance
 };
 
 struct Work {
@@ -412,7 +503,6 @@ struct hhl_batch_s {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   uint64_t graph_launches = 0;  // kernels of one run (0 before the first)
-  uint64_t captured = 0;        // those of them in the graph
   std::vector<double> host_b;  // staging for hhl_batch_run_host
 };
 
@@ -491,22 +581,55 @@ hhl_status enqueue_instance(hhl_batch_s* B, int i) {
   return s;
 }
 
+// The launch of a class with `cluster` blocks an instance; attr: room for its one attribute.
+cudaLaunchConfig_t small_config(const SmallClass& k, int cluster, cudaLaunchAttribute* attr, cudaStream_t st) {
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)cluster;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(k.count * cluster));
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.dynamicSmemBytes = k.smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  return cfg;
+}
+
+// Blocks an instance of a launch: as many as give each 16 columns (fewer gain nothing: 5 + 7 qubits 46 us by
+// two blocks, 50 by one; 4 + 7 qubits 41 and 35) while all its clusters run at once (16 instances of 7 + 7 qubits:
+// clusters of 8 come in two waves, 228 us, of 4 in one, 151; both before g was read without conflicts).
+int small_cluster(const SmallClass& k) {
+  int c = kSmallCluster;
+  while (c > 1 && k.max_n < c * kSmallColumns) c /= 2;
+  if (c > 1 && raise_dyn_smem((const void*)k_batch_small<true>, k.smem) != cudaSuccess) c = 1;
+  for (; c > 1; c /= 2) {
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = small_config(k, c, attr, nullptr);
+    int at_once = 0;
+    if (cudaOccupancyMaxActiveClusters(&at_once, k_batch_small<true>, &cfg) == cudaSuccess && k.count <= at_once) break;
+  }
+  cudaGetLastError();
+  return c;
+}
+
 // The one-block solves, on the caller's stream.
 hhl_status run_small(const hhl_batch_s* B, const double* b, double* b_copy, double* out, double* eps, cudaStream_t st) {
   for (const SmallClass& c : B->small) {
-    HHL_CUDA_TRY(raise_dyn_smem((const void*)k_batch_small, c.smem));
+    auto kern = c.cluster > 1 ? k_batch_small<true> : k_batch_small<false>;
+    HHL_CUDA_TRY(raise_dyn_smem((const void*)kern, c.smem));
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = small_config(c, c.cluster, attr, st);
     HHL_PROF_BEGIN(st);
-    k_batch_small<<<(unsigned)c.count, kSmallThreads, c.smem, st>>>(B->d_small + c.first, b, b_copy, out, eps);
+    HHL_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, (const SmallInst*)(B->d_small + c.first), b, b_copy, out, eps));
     HHL_LAUNCH_CHECK("k_batch_small");
   }
   return HHL_OK;
 }
 
 hhl_status capture(hhl_batch_s* B) {
-  if (B->exec || B->large.empty()) {
-    B->graph_launches = B->captured + B->small.size();
-    return HHL_OK;
-  }
+  if (B->large.empty()) B->graph_launches = B->small.size();
+  if (B->exec || B->large.empty()) return HHL_OK;
   cudaStream_t cap = nullptr;
   HHL_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
   cudaEvent_t fork = nullptr;
@@ -521,6 +644,7 @@ hhl_status capture(hhl_batch_s* B) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(w.s, fork, 0);
   for (int i : B->large)
     if (e == cudaSuccess && s == HHL_OK) s = enqueue_instance(B, i);
+  if (e == cudaSuccess && s == HHL_OK) s = run_small(B, B->d_b, nullptr, B->d_out, B->d_eps, cap);  // beside them
   for (auto& w : B->work) {
     if (e == cudaSuccess) e = cudaEventRecord(w.done, w.s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(cap, w.done, 0);
@@ -537,8 +661,7 @@ hhl_status capture(hhl_batch_s* B) {
   if (e2 != cudaSuccess) return cuda_fail(e2, "cudaStreamEndCapture");
   B->graph = graph;
   HHL_CUDA_TRY(cudaGraphInstantiate(&B->exec, graph, 0));
-  B->captured = g_launches.load() - l0;
-  B->graph_launches = B->captured + B->small.size();
+  B->graph_launches = g_launches.load() - l0;
   return HHL_OK;
 }
 
@@ -590,7 +713,9 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
     p.gemm_impl = gsel ? HHL_GEMM_TCGEN05 : HHL_GEMM_SIMT;
     // one-block solves: every tree step of n_c <= 7 is a Toeplitz product (fewer than 128 rows) whose
     // blocks take 8 outputs at N <= 128, which is the summation order the block repeats
-    if (gsel != 0 || p.n_c > kSmallBits || p.n_s > kSmallBits || toeplitz_rows_limit() < 128) B->large.push_back(i);
+    // (one or two of 7 + 7 qubits are faster as launches: 79 and 84 us, by a cluster each 89)
+    const bool launches = count <= 2 && p.n_s + p.n_c == 2 * kSmallBits;
+    if (gsel != 0 || p.n_c > kSmallBits || p.n_s > kSmallBits || toeplitz_rows_limit() < 128 || launches) B->large.push_back(i);
     // the two trees: sum over k of 2^k rows each (expansion and reduction)
     B->gemm_flops += 2.0 * 8.0 * (double)(p.R - 1) * (double)p.N * (double)p.N;
   }
@@ -755,7 +880,7 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
     if (e != cudaSuccess) s = cuda_fail(e, "k_ugen_g");
   }
   if (s == HHL_OK && (int)B->large.size() < count) {
-    // the one-block solves, largest first, in at most three launches (the shared memory of a launch is
+    // the one-block solves, largest first, in at most two launches (the shared memory of a launch is
     // its largest instance's; past 72 KiB, fewer than three blocks an SM, a quarter of it starts the next)
     std::vector<SmallInst> small;
     std::vector<int> idx;
@@ -777,10 +902,14 @@ hhl_status hhl_batch_create(const hhl_problem* probs, const hhl_params* params, 
       d.wall_hi = p.wall_hi;
       d.nu_over_h = p.nu * (double)(p.N + 1);
       d.index = i;
-      if (B->small.empty() || (4 * need(i) < B->small.back().smem && B->small.back().smem > (72 << 10))) B->small.push_back({(int)small.size(), 0, need(i)});
-      ++B->small.back().count;
+      if (B->small.empty() || (4 * need(i) < B->small.back().smem && B->small.back().smem > (72 << 10)))
+        B->small.push_back({(int)small.size(), 0, need(i)});
+      SmallClass& c = B->small.back();
+      ++c.count;
+      c.max_n = std::max(c.max_n, (int)p.N);
       small.push_back(d);
     }
+    for (SmallClass& c : B->small) c.cluster = small_cluster(c);
     cudaError_t e = cudaMemcpy(B->d_small, small.data(), small.size() * sizeof(SmallInst), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) s = cuda_fail(e, "batch setup");
   }
@@ -854,10 +983,11 @@ hhl_status hhl_batch_run(hhl_batch_t b, const double* b_dev, double* out_dev, do
   HHL_CUDA_TRY(cudaMemcpyAsync(b->d_b, b_dev, bo * sizeof(double), cudaMemcpyDeviceToDevice, st));
   if (b->exec != nullptr) {
     HHL_CUDA_TRY(cudaGraphLaunch(b->exec, st));
-    g_launches.fetch_add(b->captured, std::memory_order_relaxed);
+    g_launches.fetch_add(b->graph_launches, std::memory_order_relaxed);
+  } else {
+    s = run_small(b, b->d_b, nullptr, b->d_out, b->d_eps, st);
+    if (s != HHL_OK) return s;
   }
-  s = run_small(b, b->d_b, nullptr, b->d_out, b->d_eps, st);
-  if (s != HHL_OK) return s;
   HHL_CUDA_TRY(cudaMemcpyAsync(out_dev, b->d_out, oo * sizeof(double), cudaMemcpyDeviceToDevice, st));
   HHL_CUDA_TRY(cudaMemcpyAsync(eps_dev, b->d_eps, b->count * sizeof(double), cudaMemcpyDeviceToDevice, st));
   return HHL_OK;
@@ -898,10 +1028,11 @@ hhl_status hhl_batch_run_host(hhl_batch_t b, const double* b_host, double* out_h
   HHL_CUDA_TRY(cudaMemcpyAsync(b->d_b, b_host, bo * sizeof(double), cudaMemcpyHostToDevice, st));
   if (b->exec != nullptr) {
     HHL_CUDA_TRY(cudaGraphLaunch(b->exec, st));
-    g_launches.fetch_add(b->captured, std::memory_order_relaxed);
+    g_launches.fetch_add(b->graph_launches, std::memory_order_relaxed);
+  } else {
+    s = run_small(b, b->d_b, nullptr, b->d_out, b->d_eps, st);
+    if (s != HHL_OK) return s;
   }
-  s = run_small(b, b->d_b, nullptr, b->d_out, b->d_eps, st);
-  if (s != HHL_OK) return s;
   HHL_CUDA_TRY(cudaMemcpyAsync(out_host, b->d_out, oo * sizeof(double), cudaMemcpyDeviceToHost, st));
   HHL_CUDA_TRY(cudaMemcpyAsync(eps_host, b->d_eps, b->count * sizeof(double), cudaMemcpyDeviceToHost, st));
   return hhl_batch_status(b, stream);
