@@ -482,7 +482,9 @@ uint64_t hhl_kernel_launch_count(void);
  * tcgen05 GEMM is launched (or a batch graph is captured), that GEMM issues no operand copy
  * and bounds its waits by about a millisecond, so it ends with HHL_ERR_TIMEOUT (no copy or
  * product in flight when its waits run out). HHL_FAULT=alloc|plan|launch inject host failures
- * (HHL_ERR_OOM, HHL_ERR_INVALID_ARG, HHL_ERR_CUDA) into allocation, planning and launches. */
+ * (HHL_ERR_OOM, HHL_ERR_INVALID_ARG, HHL_ERR_CUDA) into allocation, planning and launches;
+ * HHL_FAULT=optional withholds the memory that a plan can do without (eigenbasis tables, the
+ * second tcgen05 operand buffer), which costs it speed only. */
 
 /* Clock-controlled U for callers that cannot allocate device memory while they run (the
  * paper has no counterpart; this is an interface convenience). Hosts that hand all device

@@ -118,7 +118,7 @@ namespace {
 
 constexpr double kPi = 3.14159265358979323846;
 
-// Host fault injection for testing error paths: HHL_FAULT=alloc|plan|launch.
+// Host fault injection for testing error paths: HHL_FAULT=alloc|plan|launch|optional.
 bool fault(const char* what) {
   const char* f = getenv("HHL_FAULT");
   return f != nullptr && strcmp(f, what) == 0;
@@ -135,6 +135,20 @@ hhl_status store_operands_k(Plan& p, const double2* d_u, int k, cudaStream_t st)
   if (s == HHL_OK && k < kTreeSimtBits && p.d_bfwd != nullptr) s = launch_store_operands(p, d_u, k, st);
   return s;
 }
+
+}  // namespace
+
+bool alloc_optional(void** p, size_t bytes, uint64_t* counter) {
+  if (!fault("optional") && cudaMalloc(p, bytes) == cudaSuccess) {
+    *counter += bytes;
+    return true;
+  }
+  *p = nullptr;
+  cudaGetLastError();
+  return false;
+}
+
+namespace {
 
 hhl_status dev_alloc(void** p, size_t bytes, uint64_t* counter) {
   if (fault("alloc")) return fail(HHL_ERR_OOM, "injected allocation failure (HHL_FAULT=alloc)");
@@ -598,11 +612,6 @@ hhl_status hhl_plan_create(const hhl_problem* prob, const hhl_params* params, hh
       hhl_plan_destroy(h);
       return fail(HHL_ERR_UNSUPPORTED, "tcgen05 GEMM not available for this size/precision");
     }
-    // The library's choice of product in complex128: the whole circuit and the postselected solve in
-    // the eigenbasis of A where that is real (hhl_spectral.cu); the stages keep the gate products.
-    if (params->gemm_impl == HHL_GEMM_AUTO && p.prec == HHL_PREC_C128 && prob->kind != HHL_MATRIX_UNITARY &&
-        eg.vi.empty() && clock_spec_fits(p))
-      HHL_PLAN_TRY(spec_create(p, eg.lam, eg.toeplitz ? nullptr : &eg.vr, st));
     const size_t mat = (size_t)N * N;
     // CUDA-core operands: every k (SIMT plans), or the k whose tree steps of the postselected
     // solve have fewer rows than one tcgen05 tile (2^k < 128) (tcgen05 plans)
@@ -720,6 +729,12 @@ hhl_status hhl_plan_create(const hhl_problem* prob, const hhl_params* params, hh
     const int mult = p.full ? 3 : 2;
     p.gemm_flops = (double)mult * p.n_c * 8.0 * (double)(p.R / 2) * (double)N * (double)N;
     }
+    // The library's choice of product in complex128: the whole circuit and the postselected solve in
+    // the eigenbasis of A where that is real (hhl_spectral.cu); the stages keep the gate products. Last, when
+    // the operands have their memory: the plan does without these tables if they do not fit.
+    if (params->gemm_impl == HHL_GEMM_AUTO && p.prec == HHL_PREC_C128 && prob->kind != HHL_MATRIX_UNITARY &&
+        eg.vi.empty() && clock_spec_fits(p))
+      HHL_PLAN_TRY(spec_create(p, eg.lam, eg.toeplitz ? nullptr : &eg.vr, st));
   } else {
     // Strang blocks of exp(i s M) for the Toeplitz Ahat: E blocks [[d, o], [o, d]] on
     // pairs (2i, 2i+1) and O blocks [[0, o], [o, 0]] on pairs (2i+1, 2i+2).

@@ -17,6 +17,8 @@ namespace hhl {
 void set_error(const std::string& msg);
 // Raise (never lower) a kernel's dynamic shared-memory limit on the current device.
 cudaError_t raise_dyn_smem(const void* func, size_t bytes);
+// Device memory that a plan can do without: false (and *p NULL) if it is not to be had.
+bool alloc_optional(void** p, size_t bytes, uint64_t* counter);
 hhl_status fail(hhl_status s, const std::string& msg);
 hhl_status cuda_fail(cudaError_t e, const char* what);
 extern std::atomic<uint64_t> g_launches;

@@ -84,8 +84,8 @@ constexpr long long kWaitCycles = 4000000000LL;      // default bound of a wait:
 constexpr long long kFaultWaitCycles = 2000000LL;    // injected timeout: ~1 ms
 
 struct TcState {
-  __half* a_hi[2] = {nullptr, nullptr};  // M_sub x 2N each, two operand buffers (TcChain)
-  __half* a_lo[2] = {nullptr, nullptr};
+  __half* a_hi[2] = {nullptr, nullptr};  // M_sub x 2N each, two operand buffers (TcChain); the
+  __half* a_lo[2] = {nullptr, nullptr};  // second may be missing, then every product gathers
   __half* b = nullptr;     // n_c x {fwd_hi, fwd_lo, adj_hi, adj_lo} x (2N x 2N)
   int* err = nullptr;      // device error flag
   TcWork work;             // stream-K partials and tile counters
@@ -656,7 +656,6 @@ hhl_status tc_prepare_operands(Plan& p, const double2* d_u, int k, cudaStream_t 
     p.d_tc = t;
     const size_t abytes = (size_t)(p.R / 2) * N2 * sizeof(__half);
     if (cudaMalloc(&t->a_hi[0], abytes) != cudaSuccess || cudaMalloc(&t->a_lo[0], abytes) != cudaSuccess ||
-        cudaMalloc(&t->a_hi[1], abytes) != cudaSuccess || cudaMalloc(&t->a_lo[1], abytes) != cudaSuccess ||
         cudaMalloc(&t->b, (size_t)p.n_c * 4 * mat * sizeof(__half)) != cudaSuccess ||
         cudaMalloc(&t->err, sizeof(int)) != cudaSuccess) {
       cudaGetLastError();
@@ -664,7 +663,7 @@ hhl_status tc_prepare_operands(Plan& p, const double2* d_u, int k, cudaStream_t 
     }
     hhl_status ws = tc_work_alloc(t->work, &p.workspace_bytes);
     if (ws != HHL_OK) return ws;
-    p.workspace_bytes += 4 * abytes;
+    p.workspace_bytes += 2 * abytes;
     p.table_bytes += (size_t)p.n_c * 4 * mat * sizeof(__half);
     HHL_CUDA_TRY(cudaMemsetAsync(t->err, 0, sizeof(int), st));
     // tile width: 256 unless HHL_TC_BN=128 (tuning) or the operand is narrower
@@ -672,7 +671,15 @@ hhl_status tc_prepare_operands(Plan& p, const double2* d_u, int k, cudaStream_t 
     if (N2 < t->bn) t->bn = 128;
     t->maps.resize(4 + 4 * (size_t)p.n_c);
     hhl_status s = HHL_OK;
-    for (int b = 0; b < 2 && s == HHL_OK; ++b) {
+    if (!alloc_optional((void**)&t->a_hi[1], abytes, &p.workspace_bytes) ||
+        !alloc_optional((void**)&t->a_lo[1], abytes, &p.workspace_bytes)) {
+      if (t->a_hi[1]) {
+        cudaFree(t->a_hi[1]);
+        p.workspace_bytes -= abytes;
+      }
+      t->a_hi[1] = nullptr;
+    }
+    for (int b = 0; b < (t->a_hi[1] != nullptr ? 2 : 1) && s == HHL_OK; ++b) {
       s = make_map(&t->maps[2 * b], t->a_hi[b], N2, p.R / 2, kBM);
       if (s == HHL_OK) s = make_map(&t->maps[2 * b + 1], t->a_lo[b], N2, p.R / 2, kBM);
     }
@@ -707,6 +714,10 @@ hhl_status launch_ctrl_u_tc_map(const Plan& p, void* half, const RowMap& rows, i
   const TcState* t = static_cast<const TcState*>(p.d_tc);
   if (t == nullptr) return fail(HHL_ERR_INVALID_ARG, "tcgen05 operands not prepared");
   const CUtensorMap* mb = &t->maps[4 + 4 * (size_t)k + (adjoint ? 2 : 0)];
+  if (t->a_hi[1] == nullptr) {
+    chain = nullptr;
+    next = TcNext{};
+  }
   const int buf = chain != nullptr ? chain->buf : 0;
   const bool ready = chain != nullptr && chain->ready;
   if (chain != nullptr) {

@@ -391,13 +391,10 @@ hhl_status spec_create(Plan& p, const std::vector<double>& lam, const std::vecto
   const size_t host_units = (host.size() + 1) & ~(size_t)1;  // (complex tables from a 16-byte boundary)
   const size_t cplx = N * 32 + N * nh + R + 3 * N;
   const size_t bytes = (host_units + (vec != nullptr ? 0 : mat) + 2 * cplx) * sizeof(double);
-  if (cudaMalloc(&s->mem, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    s->mem = nullptr;
+  if (!alloc_optional(&s->mem, bytes, &p.table_bytes)) {
     spec_free(p);  // no room beside the operands: the plan runs its gate products
     return HHL_OK;
   }
-  p.table_bytes += bytes;
   double* d = static_cast<double*>(s->mem);
   s->frac = reinterpret_cast<unsigned long long*>(d);
   s->sin_half = d + N;
