@@ -28,6 +28,10 @@ constexpr int kThr = 128;        // one thread per hidden unit
 constexpr int kGradThr = 1024;   // gradient pass: 2 units x 128 inputs x 4 row groups
 constexpr int kGradUnits = 2;
 constexpr int kGradRows = 1024;  // rows of one gradient chunk
+// Rows that the activation buffers hold (0.5 GB): a longer batch goes through them slab by slab, its chunks'
+// gradients added in the same order.
+constexpr int kSlabRows = 1 << 18;
+static_assert(kSlabRows % kGradRows == 0 && kSlabRows / kGradRows <= 65535, "chunks of a slab");
 static_assert(kRows == 4 && kThr == kH && kGradThr == kGradUnits * kH * 4, "thread maps below");
 
 __device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
@@ -42,7 +46,7 @@ __device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 
 template <bool TRAIN>
 __global__ void __launch_bounds__(kThr) k_mlp_rows(const __nv_bfloat16* __restrict__ wb, const float* __restrict__ p,
                                                    const float* __restrict__ x, const float* __restrict__ target,
-                                                   int rows, float* __restrict__ y, float* __restrict__ act,
+                                                   int rows, int total, float* __restrict__ y, float* __restrict__ act,
                                                    float* __restrict__ gy, float* __restrict__ loss_part) {
   __shared__ float4 h1s[kH], h2s[kH], g2s[kH];  // unit j of the four rows
   __shared__ float sx[kRows][kIn];
@@ -112,8 +116,8 @@ __global__ void __launch_bounds__(kThr) k_mlp_rows(const __nv_bfloat16* __restri
       if (!TRAIN) {
         if (ok) y[(size_t)(r0 + warp) * kOut + lane] = v;
       } else {
-        // loss = sum_{r,o} (y - t)^2 / (rows * kOut); gy = d loss / d y
-        const float scale = 1.f / (float)(rows * kOut);
+        // loss = sum_{r,o} (y - t)^2 / (total * kOut), over the batch's slabs; gy = d loss / d y
+        const float scale = 1.f / (float)(total * kOut);
         const float d = ok ? v - target[(size_t)(r0 + warp) * kOut + lane] : 0.f;
         sgy[warp][lane] = 2.f * d * scale;
         if (ok) gy[(size_t)(r0 + warp) * kOut + lane] = 2.f * d * scale;
@@ -198,7 +202,7 @@ __global__ void __launch_bounds__(kGradThr) k_mlp_grad(const float* __restrict__
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) g[kOffB3 + warp - 20] = s;
-  } else if (warp == 22 && blockIdx.x == 0 && blockIdx.y == 0) {
+  } else if (warp == 22 && blockIdx.x == 0 && blockIdx.y == 0 && loss != nullptr) {
     float s = 0.f;
     for (int q = lane; q < loss_parts; q += 32) s += loss_part[q];
 #pragma unroll
@@ -210,10 +214,11 @@ __global__ void __launch_bounds__(kGradThr) k_mlp_grad(const float* __restrict__
     g[kOffW2 + (j0 + u) * kH + k] = (part[0][u][k] + part[1][u][k]) + (part[2][u][k] + part[3][u][k]);
 }
 
-__global__ void k_mlp_chunks(const float* __restrict__ g_all, int chunks, float* __restrict__ g) {
+// first: the batch's first slab (else g holds the sum of those before).
+__global__ void k_mlp_chunks(const float* __restrict__ g_all, int chunks, bool first, float* __restrict__ g) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < kParams; e += gridDim.x * blockDim.x) {
-    float s = g_all[e];
-    for (int c = 1; c < chunks; ++c) s += g_all[(size_t)c * kParams + e];
+    float s = first ? g_all[e] : g[e];
+    for (int c = first ? 1 : 0; c < chunks; ++c) s += g_all[(size_t)c * kParams + e];
     g[e] = s;
   }
 }
@@ -249,57 +254,59 @@ struct hhl_mlp_s {
   float* v = nullptr;
   float* g = nullptr;           // gradients of a training step
   __nv_bfloat16* wb = nullptr;  // BF16 copy used by forward / backward
-  float* act = nullptr;         // activations and their gradients (4 x cap x 128), gy (cap x 2), loss partials
-  float* gc = nullptr;          // per-chunk gradients of batches over kGradRows rows
-  int cap = 0, cap_chunks = 0;
+  float* act = nullptr;         // activations and their gradients (4 x cap x 128), gy (cap x 2) of one slab
+  float* lp = nullptr;          // loss partials of the batch, one per four rows
+  float* gc = nullptr;          // per-chunk gradients of batches over kGradRows rows, one slab's
+  int cap = 0, cap_parts = 0, cap_chunks = 0;
   int64_t step = 0;
 };
 
 namespace hhl {
 namespace {
 
-hhl_status mlp_reserve(hhl_mlp_s* n, int rows) {
-  const int chunks = (rows + kGradRows - 1) / kGradRows;
-  if (rows > n->cap) {
-    if (n->act) cudaFree(n->act);
-    n->act = nullptr;
-    n->cap = 0;
-    if (cudaMalloc(&n->act, (size_t)rows * (4 * kH + kOut + 1) * sizeof(float)) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(HHL_ERR_OOM, "MLP activation buffers");
-    }
-    n->cap = rows;
+hhl_status mlp_grow(float** buf, int* cap, int want, size_t each, const char* what) {
+  if (want <= *cap) return HHL_OK;
+  if (*buf) cudaFree(*buf);
+  *buf = nullptr;
+  *cap = 0;
+  if (cudaMalloc(buf, (size_t)want * each * sizeof(float)) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(HHL_ERR_OOM, what);
   }
-  if (chunks > 1 && chunks > n->cap_chunks) {
-    if (n->gc) cudaFree(n->gc);
-    n->gc = nullptr;
-    n->cap_chunks = 0;
-    if (cudaMalloc(&n->gc, (size_t)chunks * kParams * sizeof(float)) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(HHL_ERR_OOM, "MLP gradient buffers");
-    }
-    n->cap_chunks = chunks;
-  }
+  *cap = want;
   return HHL_OK;
+}
+
+hhl_status mlp_reserve(hhl_mlp_s* n, int rows) {
+  const int slab = std::min(rows, kSlabRows), chunks = (slab + kGradRows - 1) / kGradRows;
+  hhl_status s = mlp_grow(&n->act, &n->cap, slab, 4 * kH + kOut, "MLP activation buffers");
+  if (s == HHL_OK) s = mlp_grow(&n->lp, &n->cap_parts, (rows - 1) / kRows + 1, 1, "MLP loss buffer");
+  if (s == HHL_OK && chunks > 1) s = mlp_grow(&n->gc, &n->cap_chunks, chunks, kParams, "MLP gradient buffers");
+  return s;
 }
 
 hhl_status mlp_grad(hhl_mlp_s* n, const float* x, const float* t, int rows, float* g, float* loss, cudaStream_t st) {
   hhl_status s = mlp_reserve(n, rows);
   if (s != HHL_OK) return s;
-  const int blocks = (rows + kRows - 1) / kRows, chunks = (rows + kGradRows - 1) / kGradRows;
-  float* gy = n->act + (size_t)rows * 4 * kH;
-  float* loss_part = gy + (size_t)rows * kOut;
-  HHL_PROF_BEGIN(st);
-  k_mlp_rows<true><<<blocks, kThr, 0, st>>>(n->wb, n->p, x, t, rows, nullptr, n->act, gy, loss_part);
-  HHL_LAUNCH_CHECK("k_mlp_rows");
-  HHL_PROF_BEGIN(st);
-  k_mlp_grad<<<dim3(kH / kGradUnits, chunks), kGradThr, 0, st>>>(x, n->act, gy, rows, chunks > 1 ? n->gc : g, loss_part, blocks,
-                                                                loss);
-  HHL_LAUNCH_CHECK("k_mlp_grad");
-  if (chunks > 1) {
+  const int parts = (rows - 1) / kRows + 1;
+  for (int64_t r0 = 0; r0 < rows; r0 += kSlabRows) {
+    const int nr = (int)std::min<int64_t>(rows - r0, kSlabRows), chunks = (nr + kGradRows - 1) / kGradRows;
+    const bool last = r0 + nr == rows;
+    float* gy = n->act + (size_t)nr * 4 * kH;
     HHL_PROF_BEGIN(st);
-    k_mlp_chunks<<<(kParams + 255) / 256, 256, 0, st>>>(n->gc, chunks, g);
-    HHL_LAUNCH_CHECK("k_mlp_chunks");
+    k_mlp_rows<true><<<(nr + kRows - 1) / kRows, kThr, 0, st>>>(n->wb, n->p, x + r0 * kIn, t + r0 * kOut, nr, rows, nullptr,
+                                                               n->act, gy, n->lp + r0 / kRows);
+    HHL_LAUNCH_CHECK("k_mlp_rows");
+    const bool whole = rows <= kGradRows;  // one chunk: its sums are the gradient
+    HHL_PROF_BEGIN(st);
+    k_mlp_grad<<<dim3(kH / kGradUnits, chunks), kGradThr, 0, st>>>(x + r0 * kIn, n->act, gy, nr, whole ? g : n->gc, n->lp, parts,
+                                                                  last ? loss : nullptr);
+    HHL_LAUNCH_CHECK("k_mlp_grad");
+    if (!whole) {
+      HHL_PROF_BEGIN(st);
+      k_mlp_chunks<<<(kParams + 255) / 256, 256, 0, st>>>(n->gc, chunks, r0 == 0, g);
+      HHL_LAUNCH_CHECK("k_mlp_chunks");
+    }
   }
   return HHL_OK;
 }
@@ -331,7 +338,7 @@ hhl_status hhl_mlp_create(hhl_mlp_t* out) {
 
 void hhl_mlp_destroy(hhl_mlp_t n) {
   if (n == nullptr) return;
-  void* ptrs[] = {n->p, n->m, n->v, n->g, n->wb, n->act, n->gc};
+  void* ptrs[] = {n->p, n->m, n->v, n->g, n->wb, n->act, n->lp, n->gc};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   delete n;
@@ -366,8 +373,8 @@ hhl_status hhl_mlp_forward(hhl_mlp_t n, const float* x_dev, int32_t rows, float*
   if (n == nullptr || x_dev == nullptr || y_dev == nullptr || rows < 1) return fail(HHL_ERR_INVALID_ARG, "bad argument");
   cudaStream_t st = (cudaStream_t)stream;
   HHL_PROF_BEGIN(st);
-  k_mlp_rows<false><<<(rows + kRows - 1) / kRows, kThr, 0, st>>>(n->wb, n->p, x_dev, nullptr, rows, y_dev, nullptr, nullptr,
-                                                                nullptr);
+  k_mlp_rows<false><<<(rows + kRows - 1) / kRows, kThr, 0, st>>>(n->wb, n->p, x_dev, nullptr, rows, rows, y_dev, nullptr,
+                                                                nullptr, nullptr);
   HHL_LAUNCH_CHECK("k_mlp_rows");
   return HHL_OK;
 }
