@@ -203,11 +203,10 @@ __global__ void __launch_bounds__(kGradThr) k_mlp_grad(const float* __restrict__
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) g[kOffB3 + warp - 20] = s;
   } else if (warp == 22 && blockIdx.x == 0 && blockIdx.y == 0 && loss != nullptr) {
-    float s = 0.f;
-    for (int q = lane; q < loss_parts; q += 32) s += loss_part[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) loss[0] = s;
+    double s = 0.0;  // (a lane adds rows / 128 parts one after another)
+    for (int q = lane; q < loss_parts; q += 32) s += (double)loss_part[q];
+    s = warp_sum(s);
+    if (lane == 0) loss[0] = (float)s;
   }
   __syncthreads();
   if (grp == 0)
