@@ -445,7 +445,8 @@ hhl_status hhl_mlp_forward(hhl_mlp_t mlp, const float* x_dev, int32_t rows, floa
 /* The same network as the T0 predictor of the plan stage (features, outputs as above). */
 hhl_status hhl_t0_predict(hhl_mlp_t mlp, const float* features_dev, int32_t rows, float* out_dev, void* stream);
 /* Gradient of loss = mean((y - t)^2) over rows and outputs with respect to the parameters
- * (through the BF16 weights): grad_dev[HHL_MLP_PARAMS], loss_dev[1] (DEVICE). */
+ * (through the BF16 weights): grad_dev[HHL_MLP_PARAMS], loss_dev[1] (DEVICE). grad_dev may lie
+ * over x_dev and t_dev. */
 hhl_status hhl_mlp_gradients(hhl_mlp_t mlp, const float* x_dev, const float* t_dev, int32_t rows, float* grad_dev,
                              float* loss_dev, void* stream);
 /* One Adam step (beta 0.9 / 0.999, eps 1e-8, learning rate lr) on that loss; loss_dev[1]

@@ -388,7 +388,14 @@ hhl_status hhl_mlp_gradients(hhl_mlp_t n, const float* x_dev, const float* t_dev
   if (n == nullptr || x_dev == nullptr || t_dev == nullptr || grad_dev == nullptr || loss_dev == nullptr || rows < 1)
     return fail(HHL_ERR_INVALID_ARG, "bad argument");
   cudaStream_t st = (cudaStream_t)stream;
-  return mlp_grad(n, x_dev, t_dev, rows, grad_dev, loss_dev, st);
+  // the gradient pass still reads the rows while it writes: a gradient laid over them is formed beside
+  auto over = [&](const float* in, size_t each) {
+    return in < grad_dev + kParams && grad_dev < in + (size_t)rows * each;
+  };
+  if (!over(x_dev, kIn) && !over(t_dev, kOut)) return mlp_grad(n, x_dev, t_dev, rows, grad_dev, loss_dev, st);
+  hhl_status s = mlp_grad(n, x_dev, t_dev, rows, n->g, loss_dev, st);
+  if (s == HHL_OK) HHL_CUDA_TRY(cudaMemcpyAsync(grad_dev, n->g, kParams * sizeof(float), cudaMemcpyDeviceToDevice, st));
+  return s;
 }
 
 hhl_status hhl_mlp_train_step(hhl_mlp_t n, const float* x_dev, const float* t_dev, int32_t rows, float lr,
