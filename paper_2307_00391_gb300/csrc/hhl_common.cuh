@@ -76,8 +76,11 @@ inline bool dep_allowed(cudaStream_t st) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
 }
+// dep = false: a plain launch. Blocks let in early take whatever slots the kernel before leaves, several to
+// an SM while others stay without, and keep them: a kernel of fewer blocks than SMs that runs longer
+// than the launch it hides is slower that way (dep at its launch says where that line lies).
 template <class... P, class... A>
-void launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+void launch_dep_if(bool dep, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchAttribute attr[1] = {dep_attribute()};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -85,8 +88,12 @@ void launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStre
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = dep_allowed(st) ? 1 : 0;
+  cfg.numAttrs = dep && dep_allowed(st) ? 1 : 0;
   (void)cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);  // (HHL_LAUNCH_CHECK reads the error)
+}
+template <class... P, class... A>
+void launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  launch_dep_if(true, kern, grid, block, smem, st, std::forward<A>(args)...);
 }
 
 // ------------------------------------------------------------------ complex helpers

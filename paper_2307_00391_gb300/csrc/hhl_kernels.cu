@@ -832,16 +832,20 @@ hhl_status launch_ctrl_u_simt_map(const Plan& p, void* half, const RowMap& k, in
   const bool c64 = p.prec == HHL_PREC_C64, few = (int64_t)grid.x * grid.y < 152 && N <= (c64 ? 256 : 128);
   const bool in_place = few || N <= 64;
   if (few) grid = dim3(1, (unsigned)((m_sub + 15) / 16));
+  // a dependent launch while a product takes less than about 50 us (launch_dep_if): 7 + 9 qubits 488 us a
+  // complex64 circuit so, 520 as plain launches, but 11 + 6 qubits 7.93 and 6.70 ms, 8 + 9 qubits read out
+  // 363 and 345 us; complex128 6 + 9 qubits 1.36 and 1.40 ms, 8 + 9 qubits 21.2 and 19.2
+  const bool dep = N < (c64 ? 256 : 128);
   HHL_PROF_BEGIN(st);
   if (c64) {
     auto kern = few ? (N <= 64 ? k_ctrl_gemm_simt<float, 16, 64, 16, true> : N <= 128 ? k_ctrl_gemm_simt<float, 16, 128, 16, true>
                                                                                      : k_ctrl_gemm_simt<float, 16, 256, 16, true>)
                 : in_place ? k_ctrl_gemm_simt<float, 64, 64, 16, true> : k_ctrl_gemm_simt<float, 64, 64, 16, false>;
-    launch_dep(kern, grid, 256, 0, st, (float2*)half, (float2*)p.d_scratch, (const float2*)B, p.n_s, k, m_sub);
+    launch_dep_if(dep, kern, grid, 256, 0, st, (float2*)half, (float2*)p.d_scratch, (const float2*)B, p.n_s, k, m_sub);
   } else {
     auto kern = few ? (N <= 64 ? k_ctrl_gemm_simt<double, 16, 64, 8, true> : k_ctrl_gemm_simt<double, 16, 128, 8, true>)
                 : in_place ? k_ctrl_gemm_simt<double, 64, 64, 8, true> : k_ctrl_gemm_simt<double, 64, 64, 8, false>;
-    launch_dep(kern, grid, 256, 0, st, (double2*)half, (double2*)p.d_scratch, (const double2*)B, p.n_s, k, m_sub);
+    launch_dep_if(dep, kern, grid, 256, 0, st, (double2*)half, (double2*)p.d_scratch, (const double2*)B, p.n_s, k, m_sub);
   }
   HHL_LAUNCH_CHECK(c64 ? "k_ctrl_gemm_simt<f32>" : "k_ctrl_gemm_simt<f64>");
   if (in_place) return HHL_OK;
@@ -1444,6 +1448,10 @@ __global__ void __launch_bounds__(256) k_toeplitz_rows_ks(float2* __restrict__ h
   cl.sync();  // the partial tiles stay until every reader is done
 }
 
+// Whether the products are dependent launches (launch_dep_if): read-out solves of 10 + 12 qubits 572 us so,
+// 592 as plain launches, 11 + 10 qubits 725 and 718, 12 + 9 qubits 1639 and 1565.
+inline bool toep_dep(int n_s) { return n_s < 12; }
+
 template <int MT, int TN>
 cudaError_t toeplitz_rows_ks_launch(dim3 grid, cudaStream_t st, float2* half, int n_s, const float4* g, int adjoint,
                                     const RowMap& rows, int64_t m) {
@@ -1458,7 +1466,7 @@ cudaError_t toeplitz_rows_ks_launch(dim3 grid, cudaStream_t st, float2* half, in
   attr[0].val.clusterDim.z = 1;
   attr[1] = dep_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = dep_allowed(st) ? 2 : 1;
+  cfg.numAttrs = toep_dep(n_s) && dep_allowed(st) ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k_toeplitz_rows_ks<MT, TN>, half, n_s, g, adjoint, rows, m);
 }
 
@@ -1476,7 +1484,7 @@ cudaError_t toeplitz_rows_launch(dim3 grid, cudaStream_t st, float2* half, int n
   constexpr int smem = toep_smem<MT, TN>();
   cudaError_t e = raise_dyn_smem((const void*)k_toeplitz_rows<MT, TN>, smem);
   if (e != cudaSuccess) return e;
-  launch_dep(k_toeplitz_rows<MT, TN>, grid, 256, smem, st, half, n_s, g, adjoint, rows, m);
+  launch_dep_if(toep_dep(n_s), k_toeplitz_rows<MT, TN>, grid, 256, smem, st, half, n_s, g, adjoint, rows, m);
   return cudaSuccess;
 }
 
