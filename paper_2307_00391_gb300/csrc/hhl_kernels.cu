@@ -829,7 +829,9 @@ hhl_status launch_ctrl_u_simt_map(const Plan& p, void* half, const RowMap& k, in
   // place up to 256 points (7 + 7 qubits, 64 rows of 128 points a product: 476 -> 367 us a solve)
   dim3 grid((unsigned)((N + 63) / 64), (unsigned)((m_sub + 63) / 64));
   const int sg = grid_for(m_sub * N, kThreads, 152 * 32);
-  const bool c64 = p.prec == HHL_PREC_C64, few = (int64_t)grid.x * grid.y < 152 && N <= (c64 ? 256 : 128);
+  // (256 points: from 65 rows on; one row of 64 x 64 tiles takes 53 us there, the wide tiles 61)
+  const bool c64 = p.prec == HHL_PREC_C64;
+  const bool few = (int64_t)grid.x * grid.y < 152 && N <= (c64 ? 256 : 128) && (N <= 128 || m_sub > 64);
   const bool in_place = few || N <= 64;
   if (few) grid = dim3(1, (unsigned)((m_sub + 15) / 16));
   // a dependent launch while a product takes less than about 50 us (launch_dep_if): 7 + 9 qubits 488 us a
