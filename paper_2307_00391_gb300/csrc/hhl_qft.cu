@@ -274,7 +274,7 @@ hhl_status pass_launch(float2* S, int n, int log_states, int b, cudaStream_t st)
   HHL_CUDA_TRY(raise_dyn_smem((const void*)kern, smem));
   HHL_PROF_BEGIN(st);
   kern<<<1u << (n + log_states - TB), kQftThreads, smem, st>>>(S, b);
-  HHL_LAUNCH_CHECK("k_whole_pass");
+  HHL_LAUNCH_CHECK("k_qft_pass");
   return HHL_OK;
 }
 
@@ -295,7 +295,7 @@ hhl_status low_launch(float2* S, int n, int log_states, float scale, bool dit, c
   HHL_PROF_BEGIN(st);
   if (dit) k_qft_low<true><<<grid, kQftThreads, 0, st>>>(S, scale);
   else k_qft_low<false><<<grid, kQftThreads, 0, st>>>(S, scale);
-  HHL_LAUNCH_CHECK("k_lowbits_transform");
+  HHL_LAUNCH_CHECK("k_qft_low");
   return HHL_OK;
 }
 
