@@ -92,9 +92,10 @@ __global__ void k_prep_fill(const uint4* bs, uint4* __restrict__ st, int64_t row
 }
 
 // Systems of at most kSmallN points: the norm, the scaled row and the fill in one launch instead of
-// four (memset, norm, scale, fill), whose launches bound them. Every
-// block forms |b|^2 and the row itself (at most 16 KiB of reads that hit L2); beyond kSmallN that
-// repetition would cost more than the launches. row_only: just the clock = 0 row (one block).
+// four (memset, norm, scale, fill), whose launches bound them. Every block forms |b|^2 and the row
+// itself (at most 16 KiB of reads that hit L2). Preparation, measurement and dissipation of 10 + 4
+// qubits take 19 us so, 31 as separate launches; 11 + 7 qubits would take 40 so and take 32.
+// row_only: just the clock = 0 row (one block).
 constexpr int kSmallN = 1024;
 constexpr size_t kPrepOneLaunch = 4 << 20;  // larger states: the row by one block, then the fill over all SMs
 template <class R>
@@ -734,8 +735,10 @@ hhl_status prep_small(const Plan& p, const double* b, void* state, bool row_only
   const int64_t half_units = p.R * p.N * (int64_t)p.amp_bytes() / 16;
   const int g = row_only ? 1 : grid_for(2 * half_units, kThreads, 152);  // the FP64 norm and scale: once per SM
   HHL_PROF_BEGIN(st);
-  launch_dep(k_prep_small<R>, g, kThreads, (size_t)p.N * p.amp_bytes(), st, (const double2*)b, (int)p.N, p.n_c, p.d_scal,
-                                                                   (uint4*)state, half_units, row_only);
+  // A dependent launch only while the blocks are few (launch_dep_if): preparation and read-outs of 10 + 6
+  // qubits take 33 us with it, 23 without, the 11-qubit solve 34 with it, 36 without.
+  launch_dep_if(row_only || g <= 76, k_prep_small<R>, g, kThreads, (size_t)p.N * p.amp_bytes(), st, (const double2*)b, (int)p.N, p.n_c,
+                p.d_scal, (uint4*)state, half_units, row_only);
   HHL_LAUNCH_CHECK("k_prep_small");
   return HHL_OK;
 }
