@@ -471,8 +471,9 @@ hhl_status hhl_apply_qft(void* state_dev, int32_t n_qubits, int32_t lo, int32_t 
  *                natural order.
  * Direction 0 followed by direction 1 is the QFT-IQFT circuit (the identity up to rounding).
  * Requires 1 <= n <= 32, n + log2(n_states) <= 34; precision HHL_PREC_C64 or HHL_PREC_C128.
- * Asynchronous on stream; the first call for a given n builds a 48 KiB (c64) twiddle table
- * on the device, kept until exit. */
+ * Asynchronous on stream. complex64 transforms of n >= 16 and 2^20 amplitudes or more keep nothing;
+ * for the others the first call for a given n builds a twiddle table on the device (48 KiB in
+ * complex64), kept until exit. */
 hhl_status hhl_qft_whole(void* state_dev, int32_t n_qubits, int32_t n_states, int32_t direction, int32_t precision,
                          void* stream);
 

@@ -98,7 +98,8 @@ __device__ __forceinline__ R root16(int k, int part) {
 // exp(-2 pi i (x mod 2^t) / 2^(t+1)) (a sixteenth root of unity, from constant memory).
 // PIN (complex64): the products' roundings spelled out. The compiler fuses one of a complex product's
 // two multiplications into the addition and picks which by context, so the same source gives other
-// last bits in another kernel; a pinned kernel gives those of k_clock_block on every compiler.
+// last bits in another kernel; a pinned kernel gives those that k_clock_block, which is not pinned, has
+// from the CUDA 13.0 compiler (the tests compare the two).
 template <bool PIN, bool SECOND, class T>
 __device__ __forceinline__ T cmul_as(T a, T b) {  // SECOND: the imaginary part rounds a.x b.y first
   if constexpr (PIN && sizeof(T) == 8) {

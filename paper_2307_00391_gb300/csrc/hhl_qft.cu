@@ -13,8 +13,8 @@
 // k r 2^-(b + NB) of a turn: one sine / cosine pair for each power-of-two k, the others as
 // products of at most five of them.
 //
-// Bound: HBM (2^NB rows of 128 bytes at NB = 9), with about 55 instructions an amplitude issued
-// under it. Measured on 2^30 amplitudes: 3.0 ms for the low bits, 3.2 ms a 9-bit pass, three passes a transform (the
+// Bound: HBM latency in the passes (2^NB rows of 128 bytes at NB = 9; 16 warps an SM, issue slots half
+// full) and the shared-memory data path in the low bits (72% of its wavefronts). Measured on 2^30 amplitudes: 3.0 ms for the low bits, 3.2 ms a 9-bit pass, three passes a transform (the
 // previous form: 4.75 ms for the low bits, 3 x 3.4 ms for passes of 6 bits).
 #include <math.h>
 #include <stdlib.h>
